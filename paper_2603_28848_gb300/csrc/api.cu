@@ -1339,11 +1339,12 @@ best_status best_collision_vjp(best_ctx* ctx, const double* f_dev, double t, con
     CK(adjoint_grid(ctx, fn, ctx->vjp_smem, &vgrid));
     CK(cudaMemsetAsync(P.chunk_counter, 0, sizeof(int32_t), st));
     CK(cudaLaunchKernel(fn, dim3(vgrid), dim3(kThreads), args, ctx->vjp_smem, st));
-    vjp_task_kernel<<<(pl.n_active + 127) / 128, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
+    vjp_task_kernel<<<(pl.n_active + 7) / 8, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
                                                                ctx->d_partials, pl.n_active, ctx->d_vjp_tot);
-    vjp_finish_kernel<<<1, 32, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, ctx->d_sconst, ctx->d_ts, v_dev,
-                                        ctx->d_u, ctx->d_vjp_tot, ctx->d_coupling, C_dev, gf_dev, gm_dev,
-                                        gcoupling_dev, ctx->d_gtail, ctx->n_processes);
+    const int fin = g.n_species + ctx->n_processes + (g.n_species * g.n_grid + 255) / 256;
+    vjp_finish_kernel<<<fin, 256, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, ctx->d_sconst, ctx->d_ts,
+                                           v_dev, ctx->d_u, ctx->d_vjp_tot, ctx->d_coupling, C_dev, gf_dev, gm_dev,
+                                           gcoupling_dev, ctx->d_gtail, ctx->n_processes);
     spline_adjoint_kernel<<<g.n_species, 32, ctx->spline_smem, st>>>(g, ctx->d_knots, ctx->d_fgrid, ctx->d_sconst,
                                                                      ctx->d_ts, ctx->d_gcoef, ctx->d_gtail, gf_dev,
                                                                      gm_dev);
@@ -1453,9 +1454,10 @@ static best_status enqueue_jvp(best_ctx* ctx, const double* f_dev, double t, con
     CK(adjoint_grid(ctx, fn, ctx->jvp_smem, &vgrid));
     CK(cudaMemsetAsync(P.chunk_counter, 0, sizeof(int32_t), st));
     CK(cudaLaunchKernel(fn, dim3(vgrid), dim3(kThreads), args, ctx->jvp_smem, st));
-    vjp_task_kernel<<<(pl.n_active + 127) / 128, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
+    vjp_task_kernel<<<(pl.n_active + 7) / 8, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
                                                                ctx->d_partials, pl.n_active, ctx->d_vjp_tot);
-    jvp_finish_kernel<<<1, 32, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, ctx->d_vjp_tot, C_dev, JU_dev);
+    jvp_finish_kernel<<<(g.n_species * g.n_grid + 63) / 64, 64, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst,
+                                                                         ctx->d_vjp_tot, C_dev, JU_dev);
     ctx->launches += 5;
     CK(cudaGetLastError());
     return BEST_OK;

@@ -55,73 +55,148 @@ __global__ void jvp_seed_kernel(Geometry g, const SideDesc* __restrict__ sides, 
     u[t] = dobs * uvec[static_cast<int64_t>(sd.species_obs) * g.n_grid + td.point] / tconst[t].scale;
 }
 
-// C~ and dC~ = J u from the tasks' tangent records; one thread, tasks in order.
-__global__ void jvp_finish_kernel(Geometry g, const SideDesc* __restrict__ sides, const TaskDesc* __restrict__ tasks,
-                                  const TaskConst* __restrict__ tconst, const double* __restrict__ tot, double* C,
-                                  double* JU) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int n = g.n_grid;
-    for (int k = 0; k < g.n_species * n; ++k) { C[k] = 0.0; JU[k] = 0.0; }
-    for (int t = 0; t < g.n_tasks; ++t) {
-        const TaskDesc td = tasks[t];
-        const SideDesc& sd = sides[td.si];
-        const double* T = tot + static_cast<int64_t>(t) * 16;
-        const int64_t ai = static_cast<int64_t>(sd.species_obs) * n + td.point;
-        const double f = sd.mult * (td.term == 0 ? 1.0 : -1.0) * tconst[t].K * tconst[t].scale /
-                         static_cast<double>(td.neval);
-        C[ai] += f * T[0];
-        JU[ai] += f * T[1];
+// Tasks of species s at grid point i in task order: f(task) for the gain and
+// loss task of every side integral observed there (none outside a shard's
+// points).
+template <typename F>
+__device__ inline void for_tasks_at(const Geometry& g, const SideDesc* __restrict__ sides, int s, int i, F&& f) {
+    if (i < g.pt_lo || i >= g.pt_hi) return;
+    const int nl = g.pt_hi - g.pt_lo;
+    for (int si = 0; si < g.n_side; ++si) {
+        if (sides[si].species_obs != s) continue;
+        const int t = (si * nl + i - g.pt_lo) * 2;
+        f(t);
+        f(t + 1);
     }
 }
 
-// Sum of each task's segment records (fixed order), 16 doubles per task.
+// C~ and dC~ = J u from the tasks' tangent records: one thread per species
+// and grid point, its tasks in task order (the same sums as one pass over all
+// tasks).  A handful of dependent loads and FP64 operations per thread; one
+// thread walking all tasks took 220 us for 256 tasks.
+__global__ void jvp_finish_kernel(Geometry g, const SideDesc* __restrict__ sides, const TaskDesc* __restrict__ tasks,
+                                  const TaskConst* __restrict__ tconst, const double* __restrict__ tot, double* C,
+                                  double* JU) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= g.n_species * g.n_grid) return;
+    double c = 0.0, ju = 0.0;
+    for_tasks_at(g, sides, k / g.n_grid, k % g.n_grid, [&](int t) {
+        const TaskDesc& td = tasks[t];
+        const double* T = tot + static_cast<int64_t>(t) * 16;
+        const double f = sides[td.si].mult * (td.term == 0 ? 1.0 : -1.0) * tconst[t].K * tconst[t].scale /
+                         static_cast<double>(td.neval);
+        c += f * T[0];
+        ju += f * T[1];
+    });
+    C[k] = c;
+    JU[k] = ju;
+}
+
+// Sum of each task's segment records in segment order, 16 doubles per task:
+// 16 lanes per task, lane v summing value v, so that a record is one
+// coalesced load and the chain per lane is its segments alone, eight loads in
+// flight (116 us for 512 tasks when one thread summed all values of a task).
 __global__ void vjp_task_kernel(Geometry g, const int32_t* __restrict__ active, const int32_t* __restrict__ task_seg,
                                 const Segment* __restrict__ segs, const double* __restrict__ partials, int n_active,
                                 double* tot) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int a = k >> 4, v = k & 15;
     if (a >= n_active) return;
-    const int t = active[a];
-    double s[16] = {};
-    for (int k = task_seg[a]; k < task_seg[a + 1]; ++k)
-        for (int v = 0; v < 12; ++v) s[v] += partials[segs[k].part + v];
-    for (int v = 0; v < 16; ++v) tot[static_cast<int64_t>(t) * 16 + v] = s[v];
+    double sum = 0.0;
+    if (v < 12) {
+        const int s1 = task_seg[a + 1];
+        int s = task_seg[a];
+        for (; s + 8 <= s1; s += 8) {
+            double x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = partials[segs[s + u].part + v];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sum += x[u];
+        }
+        for (; s < s1; ++s) sum += partials[segs[s].part + v];
+    }
+    tot[static_cast<int64_t>(active[a]) * 16 + v] = sum;
+}
+
+// Sum of v over the CTA (256 threads), in a fixed order.
+__device__ inline double cta_sum256(double v, double* red) {
+    __syncthreads();
+    red[threadIdx.x] = v;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if (static_cast<int>(threadIdx.x) < h) red[threadIdx.x] += red[threadIdx.x + h];
+        __syncthreads();
+    }
+    return red[0];
 }
 
 // C~, the observed-leg and mass / coupling parts of the gradient, and the
-// tail-parameter gradients per species; one thread, tasks in order.
+// tail-parameter gradients per species.  CTAs [0, n_species) reduce one
+// species' mass and tail gradients over all tasks, the next n_processes one
+// process's coupling gradient (fixed-order tree sums), the rest take one
+// (species, grid point) per thread, its tasks in task order.  (One thread
+// walking all tasks took 3.0 ms for 512 tasks.)  256 threads per CTA.
 __global__ void vjp_finish_kernel(Geometry g, const SideDesc* __restrict__ sides, const TaskDesc* __restrict__ tasks,
                                   const TaskConst* __restrict__ tconst, const SpeciesConst* __restrict__ sconst,
                                   const TimeState* ts, const double* __restrict__ v, const double* __restrict__ u,
                                   const double* __restrict__ tot, const double* __restrict__ coupling, double* C,
                                   double* gf, double* gm, double* gcoupling, double* gtail, int n_processes) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int n = g.n_grid;
-    for (int k = 0; k < g.n_species * n; ++k) { C[k] = 0.0; gf[k] = 0.0; }
-    for (int s = 0; s < g.n_species; ++s) {
-        gm[s] = 0.0;
-        for (int q = 0; q < 4; ++q) gtail[s * 4 + q] = 0.0;
-    }
-    for (int p = 0; p < n_processes; ++p) gcoupling[p] = 0.0;
-    for (int t = 0; t < g.n_tasks; ++t) {
-        const TaskDesc td = tasks[t];
-        const SideDesc& sd = sides[td.si];
+    __shared__ double red[256];
+    const int n = g.n_grid, S = g.n_species;
+    const int b = blockIdx.x;
+    auto integral = [&](int t, const TaskDesc& td) {
         const TaskConst& c = tconst[t];
-        const double* T = tot + static_cast<int64_t>(t) * 16;
-        const int a = sd.species_obs;
-        const int64_t ai = static_cast<int64_t>(a) * n + td.point;
-        const double sign = td.term == 0 ? 1.0 : -1.0;
-        const double I = T[0] / static_cast<double>(td.neval) * c.K * c.scale;
-        C[ai] += sd.mult * sign * I;
-        const double U = u[t];
-        const double dobs = td.term == 1 ? 1.0 : sconst[a].eta;
-        gf[ai] += U * T[1] * dobs / c.scale;
-        gm[a] += U * T[2] * ts->mass[a] / c.E_obs;
-        const int sc = sd.leg_species[sd.cons];
-        gm[sc] += U * T[3];
-        for (int q = 0; q < 4; ++q) gtail[sc * 4 + q] += U * T[4 + q];
-        for (int j = 0; j < sd.n - 2; ++j) gm[sd.leg_species[sd.integ[j]]] += U * T[8 + j];
-        gcoupling[sd.process] += 2.0 / coupling[sd.process] * sd.mult * sign * I * v[ai];
+        return tot[static_cast<int64_t>(t) * 16] / static_cast<double>(td.neval) * c.K * c.scale;
+    };
+    if (b < S) {
+        double m = 0.0, tail[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int t = threadIdx.x; t < g.n_tasks; t += blockDim.x) {
+            const SideDesc& sd = sides[tasks[t].si];
+            const double* T = tot + static_cast<int64_t>(t) * 16;
+            const double U = u[t];
+            if (sd.species_obs == b) m += U * T[2] * ts->mass[b] / tconst[t].E_obs;
+            if (sd.leg_species[sd.cons] == b) {
+                m += U * T[3];
+                for (int q = 0; q < 4; ++q) tail[q] += U * T[4 + q];
+            }
+            for (int j = 0; j < sd.n - 2; ++j)
+                if (sd.leg_species[sd.integ[j]] == b) m += U * T[8 + j];
+        }
+        m = cta_sum256(m, red);
+        if (threadIdx.x == 0) gm[b] = m;
+        for (int q = 0; q < 4; ++q) {
+            const double x = cta_sum256(tail[q], red);
+            if (threadIdx.x == 0) gtail[b * 4 + q] = x;
+        }
+        return;
     }
+    if (b < S + n_processes) {
+        const int p = b - S;
+        double l = 0.0;
+        for (int t = threadIdx.x; t < g.n_tasks; t += blockDim.x) {
+            const TaskDesc& td = tasks[t];
+            const SideDesc& sd = sides[td.si];
+            if (sd.process != p) continue;
+            const double sign = td.term == 0 ? 1.0 : -1.0;
+            l += 2.0 / coupling[p] * sd.mult * sign * integral(t, td) *
+                 v[static_cast<int64_t>(sd.species_obs) * n + td.point];
+        }
+        l = cta_sum256(l, red);
+        if (threadIdx.x == 0) gcoupling[p] = l;
+        return;
+    }
+    const int k = (b - S - n_processes) * blockDim.x + threadIdx.x;
+    if (k >= S * n) return;
+    const int a = k / n;
+    double c = 0.0, gr = 0.0;
+    for_tasks_at(g, sides, a, k - a * n, [&](int t) {
+        const TaskDesc& td = tasks[t];
+        const double dobs = td.term == 1 ? 1.0 : sconst[a].eta;
+        c += sides[td.si].mult * (td.term == 0 ? 1.0 : -1.0) * integral(t, td);
+        gr += u[t] * tot[static_cast<int64_t>(t) * 16 + 1] * dobs / tconst[t].scale;
+    });
+    C[k] = c;
+    gf[k] = gr;
 }
 
 // Transpose of the spline construction for one species per CTA (thread 0):
