@@ -16,12 +16,11 @@
 
 namespace best {
 // kernels.cu
-__global__ void set_time_kernel(Geometry, TimeState*, const double*, double, int, const MassLaw*);
-__global__ void spline_build_kernel(Geometry, const double*, int, const double*, TimeState*, SpeciesConst*,
-                                    double*, double*, float*);
+__global__ void spline_build_kernel(Geometry, SweepStart, const double*, int, const double*, SplinePlan, TimeState*,
+                                    SpeciesConst*, double*, double*, float*);
 __global__ void prepare_kernel(Geometry, const SideDesc*, const TaskDesc*, const double*, const double*,
                                const TimeState*, const double*, TaskConst*, TaskAcc*, int, const double*,
-                               const SpeciesConst*, SegConst32*);
+                               const SpeciesConst*, SegConst32*, const SideConst*);
 __global__ void moments_kernel(Geometry, const double*, const double*, const TimeState*, double*, double*);
 __global__ void width_control_kernel(Geometry, const SideDesc*, const TaskDesc*, const TaskAcc*, const WidthCtl*,
                                      double*, double*);
@@ -33,8 +32,8 @@ __global__ void strat_init_kernel(const TaskDesc*, int32_t*, uint32_t*, int);
 __global__ void strat_refine_kernel(const TaskDesc*, const int32_t*, const double*, int32_t*, double*, double*,
                                     uint32_t*, double*);
 __global__ void assemble_kernel(Geometry, const SideDesc*, TaskAcc*, TimeState*, double*, double*, double*);
-__global__ void step_first_kernel(Geometry, double*, const double*, const double*, double*, double*, TimeState*,
-                                  double*, int);
+__global__ void step_first_kernel(Geometry, double*, const double*, const double*, double*, double*, const double*,
+                                  TimeState*, double*, int);
 __global__ void heun_correct_kernel(Geometry, double*, const double*, const double*, const double*, double*,
                                     double*, TimeState*);
 __global__ void stage_kernel(Geometry, int, int, double*, const double*, const double*, double*, double*, double*,
@@ -48,8 +47,8 @@ __global__ void jvp_seed_kernel(Geometry, const SideDesc*, const TaskDesc*, cons
                                 const double*, double*);
 __global__ void jvp_finish_kernel(Geometry, const SideDesc*, const TaskDesc*, const TaskConst*, const double*, double*,
                                   double*);
-__global__ void spline_tangent_kernel(Geometry, const double*, const double*, const double*, const SpeciesConst*,
-                                      const TimeState*, double*, float*, double*);
+__global__ void spline_tangent_kernel(Geometry, const double*, const double*, SplinePlan, const double*,
+                                      const SpeciesConst*, const TimeState*, int32_t*, double*, float*, double*);
 __global__ void nk_exp_kernel(int, const double*, double*);
 __global__ void nk_axpy_kernel(int, const double*, const double*, double, double*);
 __global__ void nk_direction_kernel(int, const double*, const double*, double*);
@@ -64,8 +63,8 @@ __global__ void vjp_task_kernel(Geometry, const int32_t*, const int32_t*, const 
 __global__ void vjp_finish_kernel(Geometry, const SideDesc*, const TaskDesc*, const TaskConst*, const SpeciesConst*,
                                   const TimeState*, const double*, const double*, const double*, const double*,
                                   double*, double*, double*, double*, double*, int);
-__global__ void spline_adjoint_kernel(Geometry, const double*, const double*, const SpeciesConst*, const TimeState*,
-                                      const double*, const double*, double*, double*);
+__global__ void spline_adjoint_kernel(Geometry, const double*, SplinePlan, const double*, const SpeciesConst*,
+                                      const TimeState*, const double*, const double*, double*, double*);
 __global__ void budget_kernel(const BudgetCtl*, const TaskAcc*, TaskDesc*, double*);
 __global__ void plan_kernel(const TaskDesc*, int, const PlanDev*, int, int, int64_t*);
 }  // namespace best
@@ -131,6 +130,8 @@ struct best_ctx {
     double* d_edges = nullptr;
     double* d_knots = nullptr;
     float* d_knots32 = nullptr;
+    double* d_splplan = nullptr;    // elimination factors of the grid's spline (SplinePlan)
+    SideConst* d_sideconst = nullptr;
     double* d_coef64 = nullptr;
     float* d_coef32 = nullptr;
     double* d_fgrid = nullptr;
@@ -254,6 +255,7 @@ void free_all(best_ctx* c) {
     for (void* b : bufs) cudaFree(b);
     cudaFree(c->d_bctl); cudaFree(c->d_bv); cudaFree(c->d_plan_scratch); cudaFree(c->d_plandev);
     cudaFree(c->d_chunk_ctr);
+    cudaFree(c->d_splplan); cudaFree(c->d_sideconst);
 }
 
 best_status validate(const best_config* cfg) {
@@ -370,6 +372,35 @@ int group_size(int D, bool f32) {
 int map32_blocks(const Geometry& g) {
     const int64_t entries = static_cast<int64_t>(g.n_tasks) * map32_stride(g);
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((entries + 255) / 256, 4096)));
+}
+
+// The FP32 map tables of every task from its edges, after the edges were set
+// from outside (the refinement keeps both in step).
+cudaError_t refresh_map32(best_ctx* ctx, cudaStream_t st) {
+    if (!ctx->d_map32) return cudaSuccess;
+    map32_kernel<<<map32_blocks(ctx->geo), 256, 0, st>>>(ctx->geo, ctx->d_tasks, ctx->geo.n_tasks, ctx->d_edges,
+                                                         ctx->d_map32);
+    return cudaGetLastError();
+}
+
+// Time of a sweep and the chunk counters its first kernel clears.
+SweepStart sweep_start(const best_ctx* ctx, int mode, const double* t_dev, double t_host) {
+    return SweepStart{t_dev, ctx->d_mass_law, ctx->d_chunk_ctr, t_host, mode, ctx->max_nitn + 1};
+}
+
+// Time state, spline of f (src_mode 1: of exp(src)) and task constants: the
+// first two kernels of a sweep.
+void enqueue_setup(best_ctx* ctx, const SweepStart& ss, const double* src, int src_mode, int reset_acc,
+                   cudaStream_t st) {
+    const Geometry& g = ctx->geo;
+    spline_build_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
+        g, ss, src, src_mode, ctx->d_knots, SplinePlan{ctx->d_splplan, g.n_grid, 0}, ctx->d_ts, ctx->d_sconst,
+        ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
+    prepare_kernel<<<(g.n_tasks + 31) / 32, 32, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_knots, ctx->d_fgrid,
+                                                         ctx->d_ts, ctx->d_prev, ctx->d_tconst, ctx->d_acc, reset_acc,
+                                                         ctx->d_width, ctx->d_sconst, ctx->d_tconst32,
+                                                         ctx->d_sideconst);
+    ctx->launches += 2;
 }
 
 // Dynamic shared memory of the sample kernel with `threads` per CTA: spline
@@ -549,24 +580,13 @@ best_status set_variant(best_ctx* ctx, int v) {
     return BEST_OK;
 }
 
-// Kernels of one collision sweep after set_time: spline, task constants,
+// Kernels of one collision sweep: time state and spline, task constants,
 // nitn x (sample kernel + refinement), assembly into C / err.
-best_status enqueue_sweep(best_ctx* ctx, const double* src, int src_mode, double* C, double* err,
+best_status enqueue_sweep(best_ctx* ctx, const SweepStart& ss, const double* src, int src_mode, double* C, double* err,
                           cudaStream_t st) {
     const Geometry& g = ctx->geo;
-    spline_build_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
-        g, src, src_mode, ctx->d_knots, ctx->d_ts, ctx->d_sconst, ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
-    prepare_kernel<<<(g.n_tasks + 127) / 128, 128, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_knots,
-                                                            ctx->d_fgrid, ctx->d_ts, ctx->d_prev, ctx->d_tconst,
-                                                            ctx->d_acc, 1, ctx->d_width, ctx->d_sconst,
-                                                            ctx->d_tconst32);
-    ctx->launches += 2;
-    if (ctx->d_map32) {
-        map32_kernel<<<map32_blocks(g), 256, 0, st>>>(g, ctx->d_tasks, g.n_tasks, ctx->d_edges, ctx->d_map32);
-        ctx->launches += 1;
-    }
+    enqueue_setup(ctx, ss, src, src_mode, 1, st);
     const bool f32 = ctx->precision == BEST_FP32;
-    CK(cudaMemsetAsync(ctx->d_chunk_ctr, 0, sizeof(int32_t) * ctx->max_nitn, st));
     for (int it = 0; it < ctx->max_nitn; ++it) {
         const IterPlan& pl = ctx->plans[it];
         if (pl.n_active == 0) continue;
@@ -651,7 +671,6 @@ best_status enqueue_sweep(best_ctx* ctx, const double* src, int src_mode, double
 namespace best {
 
 __global__ void store_scalar_kernel(double* dst, double v) { *dst = v; }
-__global__ void copy_scalar_kernel(double* dst, const double* src) { *dst = *src; }
 
 // Checks a configuration like best_collision_init does (messages go to the
 // fixed-size buffer read by best_last_error(NULL); nothing is allocated).
@@ -903,7 +922,7 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
             return bail(fail(ctx, BEST_ERR_INVALID, "spline and map tables need %zu B of shared memory (max %d)",
                              sample_smem(ctx, kThreads), max_optin));
         cudaFuncAttributes fa{};
-        ctx->spline_smem = 5 * sizeof(double) * g.n_grid;
+        ctx->spline_smem = 4 * sizeof(double) * g.n_grid;
         for (const void* fn : {reinterpret_cast<const void*>(&spline_build_kernel),
                                reinterpret_cast<const void*>(&spline_tangent_kernel),
                                reinterpret_cast<const void*>(&spline_adjoint_kernel)}) {
@@ -975,6 +994,8 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
     CKI(dalloc(&ctx->d_edges, static_cast<size_t>(T) * g.map_stride));
     CKI(dalloc(&ctx->d_knots, n));
     CKI(dalloc(&ctx->d_knots32, n));
+    CKI(dalloc(&ctx->d_splplan, spline_plan_doubles(n)));
+    CKI(dalloc(&ctx->d_sideconst, g.n_side));
     CKI(dalloc(&ctx->d_coef64, static_cast<size_t>(S) * (n - 1) * 4));
     CKI(dalloc(&ctx->d_coef32, static_cast<size_t>(S) * (n - 1) * 4));
     CKI(dalloc(&ctx->d_fgrid, static_cast<size_t>(S) * n));
@@ -1036,7 +1057,16 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
     CKI(cudaMemcpy(ctx->d_edges, edges.data(), edges.size() * sizeof(double), cudaMemcpyHostToDevice));
     CKI(cudaMemcpy(ctx->d_knots, knots.data(), n * sizeof(double), cudaMemcpyHostToDevice));
     CKI(cudaMemcpy(ctx->d_knots32, knots32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
+    {
+        std::vector<double> plan(spline_plan_doubles(n), 0.0);
+        spline_plan(n, knots.data(), plan.data());
+        CKI(cudaMemcpy(ctx->d_splplan, plan.data(), plan.size() * sizeof(double), cudaMemcpyHostToDevice));
+        std::vector<SideConst> sc(g.n_side);
+        for (int k = 0; k < g.n_side; ++k) sc[k] = side_const(ctx->sides[k], cfg->processes[ctx->sides[k].process].nbins);
+        CKI(cudaMemcpy(ctx->d_sideconst, sc.data(), sc.size() * sizeof(SideConst), cudaMemcpyHostToDevice));
+    }
     CKI(cudaMemcpy(ctx->d_mass_law, ctx->mass_law.data(), S * sizeof(MassLaw), cudaMemcpyHostToDevice));
+    CKI(refresh_map32(ctx, nullptr));
     CKI(dalloc(&ctx->d_strat_est, static_cast<size_t>(T) * 4));
     CKI(cudaMemset(ctx->d_strat_est, 0, sizeof(double) * 4 * T));
     if (ctx->any_strat) {
@@ -1070,9 +1100,7 @@ best_status best_collision_eval(best_ctx* ctx, const double* f_dev, double t, do
     if (!std::isfinite(t)) return fail(ctx, BEST_ERR_INVALID, "t must be finite");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ctx->launches = 0;
-    set_time_kernel<<<1, 32, 0, st>>>(ctx->geo, ctx->d_ts, nullptr, t, 0, ctx->d_mass_law);
-    ctx->launches += 1;
-    return enqueue_sweep(ctx, f_dev, 0, C_dev, err_dev, st);
+    return enqueue_sweep(ctx, sweep_start(ctx, 0, nullptr, t), f_dev, 0, C_dev, err_dev, st);
 }
 
 best_status best_collision_eval_log(best_ctx* ctx, const double* logf_dev, double t, double* C_dev,
@@ -1082,9 +1110,7 @@ best_status best_collision_eval_log(best_ctx* ctx, const double* logf_dev, doubl
     if (!std::isfinite(t)) return fail(ctx, BEST_ERR_INVALID, "t must be finite");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ctx->launches = 0;
-    set_time_kernel<<<1, 32, 0, st>>>(ctx->geo, ctx->d_ts, nullptr, t, 0, ctx->d_mass_law);
-    ctx->launches += 1;
-    return enqueue_sweep(ctx, logf_dev, 1, C_dev, err_dev, st);
+    return enqueue_sweep(ctx, sweep_start(ctx, 0, nullptr, t), logf_dev, 1, C_dev, err_dev, st);
 }
 
 best_status best_step_stage(best_ctx* ctx, int32_t method, int32_t stage, double* logf_dev, const double* k1_dev,
@@ -1103,25 +1129,22 @@ best_status best_step_stage(best_ctx* ctx, int32_t method, int32_t stage, double
     return BEST_OK;
 }
 
-static best_status step_common(best_ctx* ctx, double* logf, double* t_dev, double* dt_dev, double* C_dev,
-                               void* stream, bool heun) {
+// One step; the requested dt is *dt_src (dt_dev, or a captured graph's own scalar).
+static best_status step_common(best_ctx* ctx, double* logf, double* t_dev, double* dt_dev, const double* dt_src,
+                               double* C_dev, void* stream, bool heun) {
     if (!ctx) return fail(nullptr, BEST_ERR_INVALID, "ctx is NULL");
     if (!logf || !t_dev || !dt_dev) return fail(ctx, BEST_ERR_INVALID, "logf, t and dt must not be NULL");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Geometry& g = ctx->geo;
     ctx->launches = 0;
     double* k1 = C_dev ? C_dev : ctx->d_k1;
-    set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, t_dev, 0.0, 1, ctx->d_mass_law);
-    ctx->launches += 1;
-    best_status s = enqueue_sweep(ctx, logf, 1, k1, nullptr, st);
+    best_status s = enqueue_sweep(ctx, sweep_start(ctx, 1, t_dev, 0.0), logf, 1, k1, nullptr, st);
     if (s != BEST_OK) return s;
-    step_first_kernel<<<1, 1024, 0, st>>>(g, logf, ctx->d_fgrid, k1, t_dev, dt_dev, ctx->d_ts, ctx->d_fstar,
+    step_first_kernel<<<1, 1024, 0, st>>>(g, logf, ctx->d_fgrid, k1, t_dev, dt_dev, dt_src, ctx->d_ts, ctx->d_fstar,
                                           heun ? 1 : 0);
     ctx->launches += 1;
     if (heun) {
-        set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, t_dev, 0.0, 2, ctx->d_mass_law);
-        ctx->launches += 1;
-        s = enqueue_sweep(ctx, ctx->d_fstar, 0, ctx->d_k2, nullptr, st);
+        s = enqueue_sweep(ctx, sweep_start(ctx, 2, t_dev, 0.0), ctx->d_fstar, 0, ctx->d_k2, nullptr, st);
         if (s != BEST_OK) return s;
         heun_correct_kernel<<<1, 1024, 0, st>>>(g, logf, ctx->d_fstar, k1, ctx->d_k2, t_dev, dt_dev, ctx->d_ts);
         ctx->launches += 1;
@@ -1132,12 +1155,12 @@ static best_status step_common(best_ctx* ctx, double* logf, double* t_dev, doubl
 
 best_status best_step_euler(best_ctx* ctx, double* logf_dev, double* t_dev, double* dt_dev, double* C_dev,
                             void* stream) {
-    return step_common(ctx, logf_dev, t_dev, dt_dev, C_dev, stream, false);
+    return step_common(ctx, logf_dev, t_dev, dt_dev, dt_dev, C_dev, stream, false);
 }
 
 best_status best_step_heun(best_ctx* ctx, double* logf_dev, double* t_dev, double* dt_dev, double* C_dev,
                            void* stream) {
-    return step_common(ctx, logf_dev, t_dev, dt_dev, C_dev, stream, true);
+    return step_common(ctx, logf_dev, t_dev, dt_dev, dt_dev, C_dev, stream, true);
 }
 
 best_status best_evolve(best_ctx* ctx, int32_t method, int32_t n_steps, double* logf_dev, double* t_dev,
@@ -1161,8 +1184,7 @@ best_status best_evolve(best_ctx* ctx, int32_t method, int32_t n_steps, double* 
         // replays they hold the sample-kernel times of the last replayed step.
         ctx->ev_used = 0;
         CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        copy_scalar_kernel<<<1, 1, 0, st>>>(dt_dev, ctx->d_dtreq);
-        best_status s = step_common(ctx, logf_dev, t_dev, dt_dev, nullptr, stream, method == 1);
+        best_status s = step_common(ctx, logf_dev, t_dev, dt_dev, ctx->d_dtreq, nullptr, stream, method == 1);
         cudaGraph_t gr = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(st, &gr);
         ctx->g_events = ctx->ev_used;
@@ -1181,7 +1203,7 @@ best_status best_evolve(best_ctx* ctx, int32_t method, int32_t n_steps, double* 
         ctx->g_t = t_dev;
         ctx->g_dt = dt_dev;
         ctx->g_method = method;
-        ctx->g_launches = ctx->launches + 1;
+        ctx->g_launches = ctx->launches;
     }
     store_scalar_kernel<<<1, 1, 0, st>>>(ctx->d_dtreq, dt_request);
     CK(cudaGetLastError());
@@ -1223,6 +1245,7 @@ best_status best_autotune(best_ctx* ctx, const double* f_dev, double t, int32_t*
         CK(cudaMemcpyAsync(ctx->d_prev, prev0, g.n_tasks * sizeof(double), cudaMemcpyDeviceToDevice, st));
         CK(cudaMemcpyAsync(ctx->d_tasks, tasks0, g.n_tasks * sizeof(TaskDesc), cudaMemcpyDeviceToDevice, st));
         CK(cudaMemcpyAsync(ctx->d_ts, &ts0, sizeof(TimeState), cudaMemcpyHostToDevice, st));
+        CK(refresh_map32(ctx, st));
         CK(cudaStreamSynchronize(st));
         return BEST_OK;
     };
@@ -1296,14 +1319,7 @@ best_status best_collision_vjp(best_ctx* ctx, const double* f_dev, double t, con
         CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ctx->vjp_smem)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ctx->launches = 0;
-    set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, nullptr, t, 0, ctx->d_mass_law);
-    spline_build_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
-        g, f_dev, 0, ctx->d_knots, ctx->d_ts, ctx->d_sconst, ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
-    prepare_kernel<<<(g.n_tasks + 127) / 128, 128, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_knots, ctx->d_fgrid,
-                                                            ctx->d_ts, ctx->d_prev, ctx->d_tconst, ctx->d_acc, 0,
-                                                            ctx->d_width, ctx->d_sconst, ctx->d_tconst32);
-    if (ctx->d_map32)
-        map32_kernel<<<map32_blocks(g), 256, 0, st>>>(g, ctx->d_tasks, g.n_tasks, ctx->d_edges, ctx->d_map32);
+    enqueue_setup(ctx, sweep_start(ctx, 0, nullptr, t), f_dev, 0, 0, st);
     vjp_seed_kernel<<<(g.n_tasks + 127) / 128, 128, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, v_dev,
                                                              ctx->d_u);
     CK(cudaMemsetAsync(ctx->d_gcoef, 0, sizeof(double) * g.n_species * (g.n_grid - 1) * 4, st));
@@ -1337,7 +1353,6 @@ best_status best_collision_vjp(best_ctx* ctx, const double* f_dev, double t, con
     void* args[] = {&V};
     int vgrid = 0;
     CK(adjoint_grid(ctx, fn, ctx->vjp_smem, &vgrid));
-    CK(cudaMemsetAsync(P.chunk_counter, 0, sizeof(int32_t), st));
     CK(cudaLaunchKernel(fn, dim3(vgrid), dim3(kThreads), args, ctx->vjp_smem, st));
     vjp_task_kernel<<<(pl.n_active + 7) / 8, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
                                                                ctx->d_partials, pl.n_active, ctx->d_vjp_tot);
@@ -1345,10 +1360,10 @@ best_status best_collision_vjp(best_ctx* ctx, const double* f_dev, double t, con
     vjp_finish_kernel<<<fin, 256, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, ctx->d_sconst, ctx->d_ts,
                                            v_dev, ctx->d_u, ctx->d_vjp_tot, ctx->d_coupling, C_dev, gf_dev, gm_dev,
                                            gcoupling_dev, ctx->d_gtail, ctx->n_processes);
-    spline_adjoint_kernel<<<g.n_species, 32, ctx->spline_smem, st>>>(g, ctx->d_knots, ctx->d_fgrid, ctx->d_sconst,
-                                                                     ctx->d_ts, ctx->d_gcoef, ctx->d_gtail, gf_dev,
-                                                                     gm_dev);
-    ctx->launches = ctx->d_map32 ? 10 : 9;
+    spline_adjoint_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
+        g, ctx->d_knots, SplinePlan{ctx->d_splplan, g.n_grid, 0}, ctx->d_fgrid, ctx->d_sconst, ctx->d_ts, ctx->d_gcoef,
+        ctx->d_gtail, gf_dev, gm_dev);
+    ctx->launches += 5;
     CK(cudaGetLastError());
     return BEST_OK;
 }
@@ -1403,25 +1418,12 @@ static best_status enqueue_jvp(best_ctx* ctx, const double* f_dev, double t, con
             CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ctx->jvp_smem)));
         ctx->jvp_ready = true;
     }
-    if (setup) {
-        set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, nullptr, t, 0, ctx->d_mass_law);
-        spline_build_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
-            g, f_dev, 0, ctx->d_knots, ctx->d_ts, ctx->d_sconst, ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
-        prepare_kernel<<<(g.n_tasks + 127) / 128, 128, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_knots,
-                                                                ctx->d_fgrid, ctx->d_ts, ctx->d_prev, ctx->d_tconst,
-                                                                ctx->d_acc, 0, ctx->d_width, ctx->d_sconst,
-                                                                ctx->d_tconst32);
-        if (ctx->d_map32) {
-            map32_kernel<<<map32_blocks(g), 256, 0, st>>>(g, ctx->d_tasks, g.n_tasks, ctx->d_edges, ctx->d_map32);
-            ctx->launches += 1;
-        }
-        ctx->launches += 3;
-    }
+    if (setup) enqueue_setup(ctx, sweep_start(ctx, 0, nullptr, t), f_dev, 0, 0, st);
     jvp_seed_kernel<<<(g.n_tasks + 127) / 128, 128, 0, st>>>(g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst,
                                                              ctx->d_sconst, u_dev, ctx->d_u);
-    spline_tangent_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(g, u_dev, ctx->d_knots, ctx->d_fgrid,
-                                                                      ctx->d_sconst, ctx->d_ts, ctx->d_dcoef64,
-                                                                      ctx->d_dcoef32, ctx->d_dtail);
+    spline_tangent_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
+        g, u_dev, ctx->d_knots, SplinePlan{ctx->d_splplan, g.n_grid, 0}, ctx->d_fgrid, ctx->d_sconst, ctx->d_ts,
+        ctx->d_chunk_ctr + ctx->max_nitn, ctx->d_dcoef64, ctx->d_dcoef32, ctx->d_dtail);
     const IterPlan& pl = ctx->plans[0];
     VjpParams V{};
     EvalParams& P = V.E;
@@ -1452,7 +1454,6 @@ static best_status enqueue_jvp(best_ctx* ctx, const double* f_dev, double t, con
     void* args[] = {&V};
     int vgrid = 0;
     CK(adjoint_grid(ctx, fn, ctx->jvp_smem, &vgrid));
-    CK(cudaMemsetAsync(P.chunk_counter, 0, sizeof(int32_t), st));
     CK(cudaLaunchKernel(fn, dim3(vgrid), dim3(kThreads), args, ctx->jvp_smem, st));
     vjp_task_kernel<<<(pl.n_active + 7) / 8, 128, 0, st>>>(g, pl.d_active, pl.d_task_seg, pl.d_segs,
                                                                ctx->d_partials, pl.n_active, ctx->d_vjp_tot);
@@ -1530,9 +1531,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
     const double t1 = t + dt;
 
     if (train) {
-        set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, nullptr, t1, 0, ctx->d_mass_law);
-        ctx->launches += 1;
-        s = enqueue_sweep(ctx, logf_dev, 1, ctx->d_k1, nullptr, st);
+        s = enqueue_sweep(ctx, sweep_start(ctx, 0, nullptr, t1), logf_dev, 1, ctx->d_k1, nullptr, st);
         if (s != BEST_OK) return s;
     }
     CK(cudaMemcpyAsync(gn, logf_dev, N * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -1661,6 +1660,7 @@ best_status best_load_state(best_ctx* ctx, const void* host_buf, int64_t size) {
     CK(cudaDeviceSynchronize());
     const size_t ne = static_cast<size_t>(ctx->geo.n_tasks) * ctx->geo.map_stride;
     CK(cudaMemcpy(ctx->d_edges, p, ne * sizeof(double), cudaMemcpyHostToDevice));
+    CK(refresh_map32(ctx, nullptr));
     p += ne * sizeof(double);
     CK(cudaMemcpy(ctx->d_prev, p, ctx->geo.n_tasks * sizeof(double), cudaMemcpyHostToDevice));
     p += ctx->geo.n_tasks * sizeof(double);
@@ -1689,6 +1689,7 @@ best_status best_load_state(best_ctx* ctx, const void* host_buf, int64_t size) {
         CK(cudaGetLastError());
         CK(cudaDeviceSynchronize());
     }
+    CK(cudaDeviceSynchronize());
     return BEST_OK;
 }
 
@@ -1699,11 +1700,11 @@ best_status best_moments(best_ctx* ctx, const double* f_dev, double t, double* n
     if (!std::isfinite(t)) return fail(ctx, BEST_ERR_INVALID, "t must be finite");
     const Geometry& g = ctx->geo;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    set_time_kernel<<<1, 32, 0, st>>>(g, ctx->d_ts, nullptr, t, 0, ctx->d_mass_law);
     spline_build_kernel<<<g.n_species, 256, ctx->spline_smem, st>>>(
-        g, f_dev, 0, ctx->d_knots, ctx->d_ts, ctx->d_sconst, ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
+        g, SweepStart{nullptr, ctx->d_mass_law, nullptr, t, 0, 0}, f_dev, 0, ctx->d_knots,
+        SplinePlan{ctx->d_splplan, g.n_grid, 0}, ctx->d_ts, ctx->d_sconst, ctx->d_fgrid, ctx->d_coef64, ctx->d_coef32);
     moments_kernel<<<g.n_species, 256, 0, st>>>(g, ctx->d_knots, ctx->d_coef64, ctx->d_ts, n_dev, rho_dev);
-    ctx->launches = 3;
+    ctx->launches = 2;
     CK(cudaGetLastError());
     return BEST_OK;
 }
@@ -1851,6 +1852,8 @@ best_status best_set_maps(best_ctx* ctx, const double* edges_host) {
     CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(ctx->d_edges, edges_host, sizeof(double) * ctx->geo.n_tasks * ctx->geo.map_stride,
                   cudaMemcpyHostToDevice));
+    CK(refresh_map32(ctx, nullptr));
+    CK(cudaDeviceSynchronize());
     return BEST_OK;
 }
 

@@ -187,6 +187,108 @@ struct SpeciesConst {
     int32_t pad_;
 };
 
+// The not-a-knot spline of one grid, laid out once per context: the tridiagonal
+// system of the second derivatives depends on the knots alone, so its
+// elimination (one dependent FP64 division per row, about 0.25 us each) is done
+// when the context is made and a spline build only substitutes.  Rows k = 0 ..
+// n - 3 for M_1 .. M_{n-2}: with the pivots 1/r_k, forward y_k = r_k d_k - g_k
+// y_{k-1}, backward x_k = y_k - c_k x_{k+1}; gT, cT the same for the transposed
+// system (its pivots are equal).  Arrays of n doubles one after the other.
+struct SplinePlan {
+    const double* base;
+    int32_t n, pad_;
+    __host__ __device__ const double* inv_h() const { return base; }           // 1 / (q_{j+1} - q_j)
+    __host__ __device__ const double* r() const { return base + n; }
+    __host__ __device__ const double* g() const { return base + 2 * n; }
+    __host__ __device__ const double* c() const { return base + 3 * n; }
+    __host__ __device__ const double* gT() const { return base + 4 * n; }
+    __host__ __device__ const double* cT() const { return base + 5 * n; }
+    __host__ __device__ const double* ends() const { return base + 6 * n; }     // M_0 = e0 M_1 - e1 M_2, M_{n-1} = e2 M_{n-2} - e3 M_{n-3}
+};
+__host__ __device__ constexpr int spline_plan_doubles(int n) { return 7 * n; }
+
+__host__ __device__ inline void spline_plan(int n, const double* q, double* out) {
+    double *inv_h = out, *r = out + n, *g = out + 2 * n, *c = out + 3 * n, *gT = out + 4 * n, *cT = out + 5 * n,
+           *e = out + 6 * n;
+    const int m = n - 2;
+    auto h = [&](int i) { return q[i + 1] - q[i]; };
+    for (int j = 0; j < n - 1; ++j) inv_h[j] = 1.0 / h(j);
+    // row k: sub-diagonal, diagonal, super-diagonal with the not-a-knot
+    // conditions (third derivative continuous at q_1 and q_{n-2}) eliminated
+    // into the first and last rows
+    auto row = [&](int k, double* ra, double* rb, double* rc) {
+        const int i = k + 1;
+        double a = h(i - 1), b = 2.0 * (h(i - 1) + h(i)), cc = h(i);
+        if (k == 0) {
+            b += h(0) * (h(0) + h(1)) / h(1);
+            cc -= h(0) * h(0) / h(1);
+            a = 0.0;
+        }
+        if (k == m - 1) {
+            const double hl = h(n - 2), hp = h(n - 3);
+            a -= hl * hl / hp;
+            b += hl * (hl + hp) / hp;
+            cc = 0.0;
+        }
+        *ra = a;
+        *rb = b;
+        *rc = cc;
+    };
+    double sup = 0.0;                                   // super-diagonal of the row before
+    for (int k = 0; k < m; ++k) {
+        double a, b, cc, a1 = 0.0, b1, c1;
+        row(k, &a, &b, &cc);
+        if (k + 1 < m) row(k + 1, &a1, &b1, &c1);
+        if (k == 0) a = 0.0;
+        const double pivot = 1.0 / (k > 0 ? b - a * c[k - 1] : b);
+        r[k] = pivot;
+        g[k] = a * pivot;
+        c[k] = cc * pivot;
+        gT[k] = sup * pivot;
+        cT[k] = a1 * pivot;
+        sup = cc;
+    }
+    e[0] = (h(0) + h(1)) / h(1);
+    e[1] = h(0) / h(1);
+    e[2] = (h(n - 2) + h(n - 3)) / h(n - 3);
+    e[3] = h(n - 2) / h(n - 3);
+}
+
+// Time of a sweep and what its first kernel (the spline build) sets up: mode
+// 0: t = t_host; 1: t = *t_dev; 2: t = *t_dev + the step's dt; with law NULL
+// the time state is left as it is.  ctr[0, n_ctr): chunk counters to clear.
+struct SweepStart {
+    const double* t_dev;
+    const MassLaw* law;
+    int32_t* ctr;
+    double t_host;
+    int32_t mode;
+    int32_t n_ctr;
+};
+
+// Per-side-integral constants of the task set-up that depend on neither the
+// time nor the distribution.
+struct SideConst {
+    double kfac;            // coupling^2 nb^D / ((2 pi)^{3(n-1)-4} 2^n sqrt(2 pi) sigma_E) (without sigma_E: fractional width)
+    double gauss_k;         // -log2(e) / (2 sigma_E^2)
+    double inv_sig2;        // 1 / sigma_E^2
+};
+inline SideConst side_const(const SideDesc& sd, int nbins) {
+    auto ipow = [](double x, int k) {
+        double r = 1.0;
+        for (; k > 0; --k) r *= x;
+        return r;
+    };
+    SideConst c;
+    const int n = sd.n;
+    c.kfac = sd.coupling2 * ipow(nbins, 3 * (n - 2)) /
+             (ipow(kTwoPi, 3 * (n - 1) - 4) * ipow(2.0, n) * 2.50662827463100050242 *
+              (sd.width_mode == 0 ? sd.sigma : 1.0));
+    c.gauss_k = -1.4426950408889634 / (2.0 * sd.sigma * sd.sigma);
+    c.inv_sig2 = 1.0 / (sd.sigma * sd.sigma);
+    return c;
+}
+
 // Everything the kernels of one context need, by value.
 struct Geometry {
     int32_t n_grid;

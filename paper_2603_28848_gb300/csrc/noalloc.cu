@@ -17,11 +17,11 @@
 #include "philox.cuh"
 
 namespace best {
-__global__ void spline_build_kernel(Geometry, const double*, int, const double*, TimeState*, SpeciesConst*,
-                                    double*, double*, float*);
+__global__ void spline_build_kernel(Geometry, SweepStart, const double*, int, const double*, SplinePlan, TimeState*,
+                                    SpeciesConst*, double*, double*, float*);
 __global__ void prepare_kernel(Geometry, const SideDesc*, const TaskDesc*, const double*, const double*,
                                const TimeState*, const double*, TaskConst*, TaskAcc*, int, const double*,
-                               const SpeciesConst*, SegConst32*);
+                               const SpeciesConst*, SegConst32*, const SideConst*);
 __global__ void map32_kernel(Geometry, const TaskDesc*, int, const double*, float2*);
 void* eval_kernel_ptr_f32(int nmax);
 void* eval_kernel_ptr_f64(int nmax);
@@ -53,7 +53,9 @@ constexpr size_t kOffTc32 = up(kOffTconst + sizeof(TaskConst));
 constexpr size_t kOffMap32 = up(kOffTc32 + sizeof(SegConst32));
 constexpr size_t kOffAcc = up(kOffMap32 + sizeof(float2) * kMaxDim * kMaxBins);
 constexpr size_t kOffPrev = up(kOffAcc + sizeof(TaskAcc));
-constexpr size_t kOffKnots = up(kOffPrev + sizeof(double));
+constexpr size_t kOffSideConst = up(kOffPrev + sizeof(double));
+constexpr size_t kOffSplPlan = up(kOffSideConst + sizeof(SideConst));
+constexpr size_t kOffKnots = up(kOffSplPlan + sizeof(double) * spline_plan_doubles(kMaxGrid));
 constexpr size_t kOffKnots32 = up(kOffKnots + sizeof(double) * kMaxGrid);
 constexpr size_t kOffFgrid = up(kOffKnots32 + sizeof(float) * kMaxGrid);
 constexpr size_t kOffCoef64 = up(kOffFgrid + sizeof(double) * BEST_MAX_SPECIES * kMaxGrid);
@@ -83,9 +85,22 @@ struct SetupArgs {
     SpeciesConst sc[BEST_MAX_SPECIES];
     SideDesc sd;
     TaskDesc td;
+    SideConst sideconst;
     int32_t ctas;
     int64_t groups;
 };
+
+// The grid's spline factors, made on the host (their recurrence is a chain of
+// dependent divisions) and handed over by value: 28 KB of kernel parameters,
+// so nothing on the host has to outlive the call.
+struct PlanArgs {
+    double v[spline_plan_doubles(kMaxGrid)];
+};
+static_assert(sizeof(PlanArgs) < 32000, "kernel parameters are limited to 32764 bytes");
+
+__global__ void noalloc_plan_kernel(PlanArgs A, int count, double* out) {
+    for (int k = threadIdx.x; k < count; k += blockDim.x) out[k] = A.v[k];
+}
 
 // Writes the descriptors, the grid, the time state and the partition of the
 // task's sample groups over the CTAs into the scratch array, and clears the
@@ -126,6 +141,7 @@ __global__ void noalloc_setup_kernel(SetupArgs A, unsigned char* base) {
         *reinterpret_cast<SideDesc*>(base + kOffSide) = A.sd;
         *reinterpret_cast<TaskDesc*>(base + kOffTask) = A.td;
         *reinterpret_cast<double*>(base + kOffPrev) = 0.0;
+        *reinterpret_cast<SideConst*>(base + kOffSideConst) = A.sideconst;
     }
 }
 
@@ -260,7 +276,18 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
     }
     A.sd = sd;
     A.td = td;
+    A.sideconst = side_const(sd, nb);
     A.ctas = ctas;
+    PlanArgs plan{};
+    {
+        double q[kMaxGrid];
+        for (int j = 0; j < n; ++j)
+            q[j] = g.log_spaced ? g.q_min * std::pow(g.q_max / g.q_min, static_cast<double>(j) / (n - 1))
+                                : g.q_min + (g.q_max - g.q_min) * j / (n - 1);
+        q[0] = g.q_min;
+        q[n - 1] = g.q_max;
+        spline_plan(n, q, plan.v);
+    }
     const int G = group_size(D, f32);
     A.groups = (td.neval + G - 1) / G;
 
@@ -280,9 +307,13 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
     float* coef32 = reinterpret_cast<float*>(base + kOffCoef32);
 
     noalloc_setup_kernel<<<1, 512, 0, st>>>(A, base);
-    const size_t spline_smem = 5 * sizeof(double) * n;
-    spline_build_kernel<<<S, 256, spline_smem, st>>>(g, f_dev, 0, knots, ts, sc, fgrid, coef64, coef32);
-    prepare_kernel<<<1, 32, 0, st>>>(g, dsd, dtd, knots, fgrid, ts, prev, dtc, dacc, 1, nullptr, sc, dtc32);
+    double* splplan = reinterpret_cast<double*>(base + kOffSplPlan);
+    noalloc_plan_kernel<<<1, 512, 0, st>>>(plan, spline_plan_doubles(n), splplan);
+    const size_t spline_smem = 4 * sizeof(double) * n;
+    spline_build_kernel<<<S, 256, spline_smem, st>>>(g, SweepStart{nullptr, nullptr, nullptr, 0.0, 0, 0}, f_dev, 0,
+                                                     knots, SplinePlan{splplan, n, 0}, ts, sc, fgrid, coef64, coef32);
+    prepare_kernel<<<1, 32, 0, st>>>(g, dsd, dtd, knots, fgrid, ts, prev, dtc, dacc, 1, nullptr, sc, dtc32,
+                                     reinterpret_cast<const SideConst*>(base + kOffSideConst));
     float2* map32 = reinterpret_cast<float2*>(base + kOffMap32);
     if (f32) map32_kernel<<<1, 256, 0, st>>>(g, dtd, 1, edges_dev, map32);
 
