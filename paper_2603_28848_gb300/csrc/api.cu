@@ -403,23 +403,11 @@ void enqueue_setup(best_ctx* ctx, const SweepStart& ss, const double* src, int s
     ctx->launches += 2;
 }
 
-// Dynamic shared memory of the sample kernel with `threads` per CTA: spline
-// tables of all species, the map table, per-warp histograms, the reduction
-// scratch and (FP32) the per-warp sample queues, in the kernel's layout.
-size_t sample_smem(const best_ctx* ctx, int threads) {
+// Dynamic shared memory of a variant of the context's sample kernel.
+size_t sample_smem(const best_ctx* ctx, const SampleVariant& v) {
     const Geometry& g = ctx->geo;
-    const bool f32 = ctx->precision == BEST_FP32;
-    const size_t rs = f32 ? 4 : 8;
-    const size_t spl = static_cast<size_t>(g.n_species) * 4 * (g.n_grid - 1) + g.n_grid;
-    // the kernel's table stride: 12 dimensions, or in the extended instantiations
-    // (stratified tasks or an s-dependent |M|^2) those of their NMAX (4 or 6 legs)
-    const bool ext = ctx->any_strat || ctx->any_me;
-    const int dims = ext ? (ctx->nmax_legs <= 4 ? 6 : 12) : kMaxDim;
-    const size_t map_elems = static_cast<size_t>(dims) * g.nbins_max;
-    const size_t hist_elems = static_cast<size_t>(threads / 32) * map_elems;
-    const size_t queue = ctx->any_strat ? strat_queue_floats(ctx->nmax_legs) : kQueueSlots * queue_words(ctx->nmax_legs);
-    return rs * ((spl + 3) & ~size_t(3)) + 2 * rs * map_elems + rs * ((hist_elems + 3) & ~size_t(3)) +
-           2 * 32 * sizeof(double) + (f32 ? sizeof(float) * (threads / 32) * queue : 0);
+    return sample_smem_bytes(ctx->precision == BEST_FP32, g.n_grid, g.n_species, g.nbins_max, ctx->nmax_legs,
+                             ctx->any_strat || ctx->any_me, ctx->any_strat, v.threads, v.spl);
 }
 
 // Partition of the active tasks of one iteration into n_chunks chunks cut at
@@ -520,7 +508,7 @@ best_status set_variant(best_ctx* ctx, int v) {
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     void* fn = ctx->variants[v].fn;
     const int threads = ctx->variants[v].threads;
-    ctx->eval_smem = sample_smem(ctx, threads);
+    ctx->eval_smem = sample_smem(ctx, ctx->variants[v]);
     cudaFuncAttributes fa{};
     CK(cudaFuncGetAttributes(&fa, fn));
     if (static_cast<size_t>(fa.maxDynamicSharedSizeBytes) < ctx->eval_smem)
@@ -916,11 +904,11 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
         cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         ctx->n_variants = 0;
         for (int v = 0; v < nv; ++v)
-            if (sample_smem(ctx, all[v].threads) <= static_cast<size_t>(max_optin))
+            if (sample_smem(ctx, all[v]) <= static_cast<size_t>(max_optin))
                 ctx->variants[ctx->n_variants++] = all[v];
         if (ctx->n_variants == 0)
             return bail(fail(ctx, BEST_ERR_INVALID, "spline and map tables need %zu B of shared memory (max %d)",
-                             sample_smem(ctx, kThreads), max_optin));
+                             sample_smem(ctx, all[nv - 1]), max_optin));
         cudaFuncAttributes fa{};
         ctx->spline_smem = 4 * sizeof(double) * g.n_grid;
         for (const void* fn : {reinterpret_cast<const void*>(&spline_build_kernel),

@@ -1,0 +1,389 @@
+// FP64 sample loop with an FP32 screen.
+//
+// FP64 runs at 1/64 of the FP32 rate on this GPU: one FP64 operation of a warp
+// takes an SM partition's pipe for 64 cycles, about 300 of them per 2 -> 2
+// sample, so the plain FP64 loop is bound by that pipe alone (1.6e9 samples/s).
+// Most samples, though, lie so far from the energy shell that the Gaussian of
+// Eq. (11) is zero in FP64, or too small to change any result.  So every
+// sample is first screened in FP32 (Philox words, map, momenta, energy
+// balance with a bound on its error), the samples that can matter are queued
+// per warp as their Philox words, and 32 queued samples at a time are
+// evaluated from scratch in FP64 on a full warp.
+//
+// What the screen drops, in terms of an upper bound L of log2 |w_n|:
+//   * samples whose Gaussian exponent is below -1100 (|dE| > 39 sigma): their
+//     FP64 weight is exactly 0 (2^-1075 is the smallest subnormal);
+//   * samples with L < log2(largest |w_n| this warp has evaluated in the
+//     segment) - kDropBits, kDropBits = 170.  L takes the kinematic factors
+//     from FP32 (a few bits) and the statistical factors from their maximum
+//     on the grid; a spline's overshoot or a tail above that maximum would
+//     have to exceed 2^60 for such a sample to reach 2^-110 of the largest.
+//     Even 2^31 of them are below the rounding of the sums of w and w^2, and
+//     an increment holding nothing else has a share below the 1e-30 that the
+//     refinement counts as empty.
+// A sample whose FP32 quantities leave the normal range is kept.
+//
+// Measured per launch on trained maps, plain loop -> this one: MB 2 -> 2, 32
+// points, 1e5 samples: 4.08 -> 0.50 ms; BE 2 -> 2, 2 species, 128 points, 1e5
+// samples: 27.4 -> 6.19 ms (the FP64 pipe then 84% busy).
+#pragma once
+
+#include "math_table.cuh"
+
+namespace best {
+
+constexpr float kDropBits = 170.0f;
+
+// ---- FP64 elementary functions of this loop: fewer FP64 operations than the
+// library's, at the price of a restricted range (checked or falling back) ----
+
+// The float next to a positive double in float range, towards zero, and back:
+// integer operations only (FP64 conversions use the FP64 pipe).
+__device__ __forceinline__ float trunc_f32(double x) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double widen_f32(float x) {        // positive normal float, exact
+    const uint32_t b = __float_as_uint(x);
+    return __hiloint2double(static_cast<int>((b >> 3) + 0x38000000u), static_cast<int>(b << 29));
+}
+__device__ __forceinline__ double flip_sign(double x, uint32_t mask) {
+    return __hiloint2double(__double2hiint(x) ^ static_cast<int>(mask), __double2loint(x));
+}
+
+// 1/sqrt(x): FP32 estimate (22 bits) and one step of Halley's third-order
+// iteration (relative error 5/16 e^3 < 2^-60 before rounding).
+__device__ __forceinline__ double rsqrt_halley(double x) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x));
+    if (hi - 0x39000000u > 0x0DFFFFFFu) return rsqrt(x);      // outside [2^-111, 2^113): zero, subnormal, huge, NaN
+    const double y = widen_f32(rsqrt_ftz(trunc_f32(x)));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// sin and cos of |x| <= pi: the nearest a_k = k pi / 64 of the table, the
+// Taylor polynomials of r = |x| - a_k (|r| <= pi / 128, the difference is
+// exact) and the addition theorem (table-driven reduction after Gal and Tang).
+__device__ __forceinline__ void sincos_table(double x, const double* tab, double* s, double* c) {
+    const uint32_t sign = static_cast<uint32_t>(__double2hiint(x)) & 0x80000000u;
+    const double ax = flip_sign(x, sign);
+    // a subnormal or zero |x| truncates to a huge or zero float: k is clamped
+    // either way (k = 0 for |x| < 2^-126 through the comparison below)
+    const uint32_t hx = static_cast<uint32_t>(__double2hiint(ax));
+    const float xf = hx < 0x38100000u ? 0.0f : trunc_f32(ax);
+    const int k = min(__float2int_rn(xf * 20.371832715762603f), kTrigEntries - 1);      // 64 / pi
+    const double a = tab[3 * k], S = tab[3 * k + 1], C = tab[3 * k + 2];
+    const double r = ax - a;
+    const double r2 = r * r;
+    const double p = fma(r2, fma(r2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0);
+    const double sr = fma(r * r2, p, r);
+    const double cm = r2 * fma(r2, fma(r2, -1.0 / 720.0, 1.0 / 24.0), -0.5);
+    *s = flip_sign(S + fma(C, sr, S * cm), sign);
+    *c = C + fma(-S, sr, C * cm);
+}
+
+// 2^x, x <= 0: 2^k 2^(j/32) 2^r, |r| <= 1/64, Taylor polynomial of 2^r - 1.
+__device__ __forceinline__ double exp2_table(double x, const double* tab) {
+    // hi word of x: beyond -1000 (or NaN) the library's function, which handles subnormal results
+    if (static_cast<uint32_t>(__double2hiint(x)) - 0x80000000u > 0x408F4000u - 1u) return exp2(x);
+    const uint32_t hx = static_cast<uint32_t>(__double2hiint(x)) & 0x7fffffffu;
+    const float xf = hx < 0x38100000u ? 0.0f : trunc_f32(flip_sign(x, 0x80000000u));    // |x|
+    const int n = __float2int_rn(xf * 32.0f);
+    // n / 32 as a double (0 for n = 0)
+    const double nd = n == 0 ? 0.0 : widen_f32(static_cast<float>(n) * 0.03125f);
+    const double r = x + nd;
+    double p = fma(r, 0x1.430912f86c787p-13, 0x1.5d87fe78a6731p-10);       // ln(2)^k / k!
+    p = fma(r, p, 0x1.3b2ab6fba4e77p-7);
+    p = fma(r, p, 0x1.c6b08d704a0c0p-5);
+    p = fma(r, p, 0x1.ebfbdff82c58fp-3);
+    p = fma(r, p, 0x1.62e42fefa39efp-1);
+    const int k = -n;                                                     // x = k/32 + r
+    const double T = tab[3 * kTrigEntries + (k & 31)];
+    const double v = fma(T, p * r, T);
+    return __hiloint2double(__double2hiint(v) + ((k >> 5) << 20), __double2loint(v));
+}
+
+// a < b for doubles neither of which is NaN, as integers (an FP64 comparison
+// takes the FP64 pipe): b > 0; a negative a compares less.
+__device__ __forceinline__ bool less_pos(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// Cubic spline value at comoving q inside [q_0, q_{n-1}], the interval from
+// FP32 (a guess within one interval, as in spline_eval).
+__device__ __forceinline__ double spline64(const double* coef, const double* knots, double q, const Geometry& g,
+                                           float inv_step, float q0, float lq0_step) {
+    const float qf = trunc_f32(q);
+    int j = static_cast<int>(g.log_spaced ? fmaf(lg2_ftz(qf), inv_step, -lq0_step) : (qf - q0) * inv_step);
+    j = min(max(j, 0), g.n_grid - 2);
+    const double t = q - knots[j];
+    const double2* cp = reinterpret_cast<const double2*>(coef) + 2 * j;
+    const double2 lo = cp[0], hi = cp[1];
+    const double f = fma(fma(fma(hi.y, t, hi.x), t, lo.y), t, lo.x);
+    return __double2hiint(f) < 0 ? 0.0 : f;
+}
+
+// Weight of one sample in FP64 (kin_at and stat_at of eval_impl.cuh, the same
+// formulas) with the functions above; C lives in shared memory.
+template <int NLEG>
+__device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, const double* y, double jac,
+                                           const double* s_spline, const double* knots, const Geometry& g,
+                                           const SegSetup<float, NLEG>& s32, double q0, double qN, int ncoef,
+                                           const double* tab) {
+    constexpr int NI = NLEG - 2;
+    double px = 0.0, py = 0.0, pz = C.pobs_sig;
+    double bal = C.sgn_obs_E;
+    double Esum = C.e_obs;
+    double meas = jac, rinv = 1.0, stat = C.c0;
+    const bool scaled = C.inv_a != 1.0;
+    bool cut = false;
+#pragma unroll
+    for (int j = 0; j < NI; ++j) {
+        const double r = y[3 * j];
+        double st, ct, sp, cp;
+        sincos_table(y[3 * j + 1], tab, &st, &ct);
+        sincos_table(y[3 * j + 2], tab, &sp, &cp);             // angle phi - pi
+        const uint32_t sg = static_cast<uint32_t>(__double2hiint(C.sig[j])) & 0x80000000u;
+        const double p = scaled ? r * C.inv_a : r;
+        const double nps = flip_sign(p * st, sg ^ 0x80000000u);     // cos(phi) = -cos(phi - pi)
+        px = fma(nps, cp, px);
+        py = fma(nps, sp, py);
+        pz = fma(flip_sign(p, sg), ct, pz);
+        const double E2 = fma(p, p, C.m2[j]);
+        const double rE = rsqrt_halley(E2);
+        const double E = E2 * rE;
+        cut |= less_pos(E, C.e_cut);
+        bal += flip_sign(E, static_cast<uint32_t>(__double2hiint(C.sgnE[j])) & 0x80000000u);
+        if (C.frac) Esum += E;
+        meas *= r * r * st;
+        rinv *= rE;
+        double f = spline64(s_spline + C.spc[j] * ncoef, knots, r, g, s32.inv_step, s32.q0, s32.lq0_step);
+        if (C.fd[j]) f = f < 1.0 ? f : 1.0;
+        stat *= fma(C.cb[j], f, C.ca[j]);
+    }
+    const double pc2 = fma(px, px, fma(py, py, pz * pz));
+    double rpc, rEc, Ec;
+    if (C.m2c == 0.0) {
+        rEc = rsqrt_halley(less_pos(0.0, pc2) ? pc2 : 1e-30);
+        Ec = pc2 * rEc;
+        rpc = less_pos(0.0, pc2) ? rEc : 0.0;
+    } else {
+        const double Ec2 = pc2 + C.m2c;
+        rEc = rsqrt_halley(Ec2);
+        Ec = Ec2 * rEc;
+        rpc = less_pos(0.0, pc2) ? rsqrt_halley(pc2) : 0.0;
+    }
+    cut |= less_pos(Ec, C.e_cut);
+    bal += flip_sign(Ec, static_cast<uint32_t>(__double2hiint(C.sgn_cons)) & 0x80000000u);
+    double qc = pc2 * rpc;
+    if (scaled) qc *= C.a;
+    double gauss;
+    if (C.frac) {
+        Esum += Ec;
+        const double iS = 1.0 / Esum;
+        const double x = bal * iS;
+        gauss = exp2_table(C.gauss_k * x * x, tab) * (2.0 * C.e_obs * iS);
+    } else {
+        gauss = exp2_table(C.gauss_k * bal * bal, tab);
+    }
+    const double kin = meas * rinv * rEc * gauss;
+    double fc;
+    const bool below = less_pos(qc, q0), above = less_pos(qN, qc);
+    if (!below && !above) {
+        fc = spline64(s_spline + C.sp_cons * ncoef, knots, qc, g, s32.inv_step, s32.q0, s32.lq0_step);
+    } else {
+        const double x = below ? C.tlo_a + C.tlo_b * Ec : C.thi_a + C.thi_b * Ec;
+        const double den = C.eta_c == 1.0 ? expm1(x) : exp(x) - C.eta_c;
+        fc = den > 0.0 ? 1.0 / den : 0.0;
+    }
+    if (C.fd_c) fc = fc < 1.0 ? fc : 1.0;
+    const double w = stat * fma(C.cbc, fc, C.cac) * kin;
+    return cut ? 0.0 : w;
+}
+
+// Upper bound of log2 of the kinematic part of a sample's weight from FP32
+// arithmetic, y the mapped point and jac the map's Jacobian; *gauss gets an
+// upper bound of the Gaussian's exponent.  Every momentum component carries at
+// most about 4e-6 of the momenta (sin.approx and cos.approx: 2^-21 absolute;
+// the FP32 map: 2^-22 of an angle), every energy 2e-7: 4e-5 of the energies'
+// sum covers the balance ten times.  +inf where a factor leaves the normal
+// range (or is not a number).
+template <int NLEG>
+__device__ __forceinline__ float log2_kin_bound(const SegConst<float, NLEG>& C, const float* y, float jac, float* gauss) {
+    constexpr int NI = NLEG - 2;
+    float px = 0.0f, py = 0.0f, pz = C.pobs_sig;
+    float bal = C.sgn_obs_E, Esum = C.e_obs;
+    float prod = jac;
+#pragma unroll
+    for (int j = 0; j < NI; ++j) {
+        const float r = y[3 * j];
+        float st, ct, sp, cp;
+        __sincosf(y[3 * j + 1], &st, &ct);
+        __sincosf(y[3 * j + 2], &sp, &cp);
+        const float p = r * C.inv_a;
+        const float nps = -C.sig[j] * (p * st);
+        px = fmaf(nps, cp, px);
+        py = fmaf(nps, sp, py);
+        pz = fmaf(C.sig[j] * p, ct, pz);
+        const float E2 = fmaf(p, p, C.m2[j]);
+        const float rE = rsqrt_ftz(E2);
+        const float E = E2 * rE;
+        bal = fmaf(C.sgnE[j], E, bal);
+        Esum += E;
+        prod *= r * r * st * rE;
+    }
+    const float Ec2 = fmaf(px, px, fmaf(py, py, fmaf(pz, pz, C.m2c)));
+    const float rEc = rsqrt_ftz(Ec2);
+    const float Ec = Ec2 * rEc;
+    bal = fmaf(C.sgn_cons, Ec, bal);
+    Esum += Ec;
+    prod *= rEc;
+    float d = fmaxf(fabsf(bal) - 4e-5f * Esum, 0.0f);
+    if (!(Esum < 1e30f)) d = 0.0f;                       // (overflowed, or not a number)
+    float extra = 0.0f;
+    if (C.frac) {
+        const float iS = __fdividef(1.0f, Esum);
+        d *= iS;
+        extra = lg2_ftz(2.0f * C.e_obs * iS);
+    }
+    const float e = C.gauss_k * d * d;
+    *gauss = e;
+    return prod > 1e-37f && prod < 1e37f ? lg2_ftz(prod) + extra + e : __int_as_float(0x7f800000);
+}
+
+// FP64 words of sample group g: the four Philox words of every block.
+template <int D, typename Keys>
+__device__ __forceinline__ void group_words64(uint32_t* w, uint32_t g, uint32_t itn, uint32_t call, uint32_t task,
+                                              const Keys& rk) {
+    using S = StreamShape<D, false>;
+    const uint32_t b0 = g * S::kBlocks;            // counter word 0 is the block index mod 2^32
+#pragma unroll
+    for (int j = 0; j < S::kBlocks; ++j) {
+        uint32_t c0 = b0 + j, c1 = itn, c2 = call, c3 = task;
+        philox4x32_10(c0, c1, c2, c3, rk);
+        w[4 * j + 0] = c0;
+        w[4 * j + 1] = c1;
+        w[4 * j + 2] = c2;
+        w[4 * j + 3] = c3;
+    }
+}
+
+// The samples of one segment.  map32: the map table rounded to FP32; tab: the
+// function tables; setup: this segment's FP64 constants, written here; all in
+// shared memory.
+template <int NLEG>
+__device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment& seg, const SideDesc& sd,
+                                              const TaskDesc& td, const TaskConst& tc, const double* s_spline,
+                                              const Real2<double>* s_map, const Real2<float>* s_map32,
+                                              double* w_hist, const double* tab, SegSetup<double, NLEG>* s_setup,
+                                              uint32_t* s_queue, Acc<double>& acc_w, Acc<double>& acc_w2) {
+    constexpr int NI = NLEG - 2;
+    constexpr int D = 3 * NI;
+    using SS = StreamShape<D, false>;
+    constexpr int G = SS::kGroup;
+    const Geometry& g = P.geo;
+    const int nb = td.nbins;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        SegSetup<double, NLEG> st;
+        seg_setup<double, NLEG>(P, sd, td, tc, &st);
+        *s_setup = st;
+    }
+    SegSetup<float, NLEG> s32;
+    seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
+    // log2 of an upper bound of c0 times the statistical factors on the grid
+    float stat_bits = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f)) + 1.0f;
+#pragma unroll
+    for (int j = 0; j <= NI; ++j)
+        stat_bits += fmaxf(P.sconst[sd.leg_species[j < NI ? sd.integ[j] : sd.cons]].log2_fmax, 0.0f) + 1.0f;
+    __syncthreads();
+    const SegConst<double, NLEG>& C = s_setup->C;
+    const double* knots = s_spline + g.n_species * 4 * (g.n_grid - 1);
+    const int ncoef = 4 * (g.n_grid - 1);
+    const uint32_t call = P.ts->call, task = td.gid;
+    uint32_t* q = s_queue + (tid >> 5) * (2 * D * kQueueSlots);
+    const uint32_t lanes_below = (1u << lane) - 1u;
+    int qn = 0;                             // queued samples (warp-uniform)
+    int wmax = 0;                           // high word of the largest |w_n| evaluated by this warp
+    float cutoff = -3.0e38f;                // samples with log2_kin_bound below this cannot matter
+
+    auto drain = [&](int slot) {
+        double y[D], jac = 1.0;
+        uint32_t bins[(D + 3) / 4] = {};
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            // (2 k + 1) nb, k the 52-bit uniform: the increment is the part above bit 53, the
+            // fraction the 53 bits below it (its last bit dropped)
+            const uint32_t x0 = q[(2 * d) * kQueueSlots + slot], x1 = q[(2 * d + 1) * kQueueSlots + slot];
+            const uint64_t k = (static_cast<uint64_t>(x0 >> 6) << 26) | (x1 >> 6);
+            const uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);
+            const uint32_t b = static_cast<uint32_t>(m >> 53);
+            const uint64_t fr = 0x3FF0000000000000ull | ((m >> 1) & 0x000FFFFFFFFFFFFFull);
+            const Real2<double> e = s_map[d * nb + b];
+            y[d] = fma(e.dy, __longlong_as_double(static_cast<long long>(fr)) - 1.0, e.y0);
+            jac = d == 0 ? e.dy : jac * e.dy;
+            bins[d >> 2] |= b << (8 * (d & 3));
+        }
+        const double w = weight64<NLEG>(C, y, jac, s_spline, knots, g, s32, s_setup->q0, s_setup->qN, ncoef, tab);
+        const double w2 = w * w;
+        acc_w.add(w);
+        acc_w2.add(w2);
+        if (w2 != 0.0) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) atomicAdd(&w_hist[d * nb + ((bins[d >> 2] >> (8 * (d & 3))) & 0xFFu)], w2);
+        }
+        return __double2hiint(w) & 0x7fffffff;
+    };
+
+    const uint32_t g1 = static_cast<uint32_t>(seg.g1), N = static_cast<uint32_t>(td.neval);
+    for (uint32_t gb = static_cast<uint32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
+        const uint32_t grp = gb + lane;
+        uint32_t uw[4 * SS::kBlocks];
+        group_words64<D>(uw, grp, P.itn, call, task, P.rk);
+#pragma unroll
+        for (int sgi = 0; sgi < G; ++sgi) {
+            const bool valid = grp < g1 && grp * G + sgi < N;
+            float y[D], jac = 1.0f;
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                // the uniform's first 32 bits (an increment's edge may fall to its neighbour: the
+                // mapped point is continuous there)
+                const uint32_t x = (uw[2 * (sgi * D + d)] & ~63u) | (uw[2 * (sgi * D + d) + 1] >> 26);
+                const uint64_t m = static_cast<uint64_t>(x) * static_cast<uint32_t>(nb);
+                const Real2<float> e = s_map32[d * nb + static_cast<uint32_t>(m >> 32)];
+                y[d] = fmaf(e.dy, static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f, e.y0);
+                jac *= e.dy;
+            }
+            float gauss;
+            const float l = log2_kin_bound<NLEG>(s32.C, y, jac, &gauss);
+            const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
+            const uint32_t vote = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
+#pragma unroll
+                for (int k = 0; k < 2 * D; ++k) q[k * kQueueSlots + slot] = uw[2 * sgi * D + k];
+            }
+            qn += __popc(vote);
+            if (qn >= 32) {
+                __syncwarp();
+                const int hi = drain(lane);
+                const int top = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(hi)));
+                if (top > wmax && top < 0x7FE00000) {
+                    wmax = top;
+                    cutoff = static_cast<float>((top >> 20) - 1023) - stat_bits - kDropBits;
+                }
+                __syncwarp();
+                if (lane < qn - 32) {
+#pragma unroll
+                    for (int k = 0; k < 2 * D; ++k) q[k * kQueueSlots + lane] = q[k * kQueueSlots + 32 + lane];
+                }
+                __syncwarp();
+                qn -= 32;
+            }
+        }
+    }
+    __syncwarp();
+    if (lane < qn) drain(lane);
+}
+
+}  // namespace best

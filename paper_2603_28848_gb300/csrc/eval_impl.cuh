@@ -556,6 +556,12 @@ __device__ __forceinline__ void seg_setup32(const SegConst32& S, SegSetup<float,
     out->inv_step = S.inv_step;
 }
 
+}  // namespace best
+
+#include "eval_f64q.cuh"
+
+namespace best {
+
 // STRAT: the instantiation also handles stratified tasks and s-dependent
 // matrix elements (kept apart so that the plain kernel's register allocation
 // is not affected).
@@ -568,6 +574,7 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     constexpr int NI = NLEG - 2;
     constexpr int D = 3 * NI;
     constexpr bool F32 = RMath<R>::kF32;
+    constexpr bool SCREEN = !F32 && SPL == 2;      // FP64 with the FP32 screen (eval_f64q.cuh)
     using SS = StreamShape<D, F32>;
     constexpr int G = SS::kGroup;
     const Geometry& g = P.geo;
@@ -602,6 +609,11 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
             v.y0 = static_cast<R>(lo + sc * e0);
             v.dy = static_cast<R>(sc * (e1 - e0));
             s_map[k] = v;
+            if constexpr (SCREEN) {
+                Real2<float>* s_map32 = reinterpret_cast<Real2<float>*>(reinterpret_cast<unsigned char*>(s_queue) +
+                                                                        sizeof(double) * kMathDoubles + kSetupBytes);
+                s_map32[k] = Real2<float>{static_cast<float>(v.y0), static_cast<float>(v.dy)};
+            }
         }
     }
     // per-warp histograms: atomics from different warps never share an
@@ -611,6 +623,16 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     for (int k = tid; k < nwarps * map_elems; k += blockDim.x) s_hist[k] = R(0);
     R* w_hist = s_hist + (tid >> 5) * map_elems;
 
+    Acc<R> acc_w, acc_w2;
+    if constexpr (SCREEN) {
+        // (the constants' barrier orders the tables written above)
+        double* tab = reinterpret_cast<double*>(s_queue);
+        SegSetup<double, NLEG>* s_setup = reinterpret_cast<SegSetup<double, NLEG>*>(tab + kMathDoubles);
+        static_assert(sizeof(SegSetup<double, NLEG>) <= kSetupBytes, "room for the segment constants");
+        Real2<float>* s_map32 = reinterpret_cast<Real2<float>*>(reinterpret_cast<unsigned char*>(s_setup) + kSetupBytes);
+        run_samples64<NLEG>(P, seg, sd, td, tc, s_spline, s_map, s_map32, w_hist, tab, s_setup,
+                            reinterpret_cast<uint32_t*>(s_map32 + map_elems), acc_w, acc_w2);
+    } else {
     // ---- per-segment constants ----------------------------------------------
     SegSetup<R, NLEG> setup;
     if constexpr (F32) seg_setup32<NLEG>(P.tconst32[seg.task], &setup);
@@ -624,7 +646,6 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     const uint32_t call = P.ts->call;
 
     // ---- samples ------------------------------------------------------------
-    Acc<R> acc_w, acc_w2;
     const int64_t N = td.neval;
     const uint32_t task = td.gid;                 // the stream is keyed by the global task id
     const int32_t g1 = static_cast<int32_t>(seg.g1);
@@ -1035,6 +1056,7 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
             }
         }
     }
+    }
 
     // ---- segment reduction into its partial record (FP64) -------------------
     double vw = acc_w.value(), vw2 = acc_w2.value();
@@ -1071,7 +1093,8 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
 
 // MB: CTAs per SM the kernel is register-limited to (__launch_bounds__);
 // THREADS: threads per CTA; SPL: samples a lane evaluates per step of the
-// FP32 loop (1, or 2 in packed FP32x2 arithmetic).  Several combinations are
+// FP32 loop (1, or 2 in packed FP32x2 arithmetic); for FP64, 2 is the loop
+// with the FP32 screen (eval_f64q.cuh).  Several combinations are
 // instantiated and the autotuner picks one at run time.
 template <typename R, int NMAX, int MB, bool STRAT = false, int THREADS = kThreads, int SPL = 1>
 __global__ void __launch_bounds__(THREADS, MB)
@@ -1085,12 +1108,16 @@ eval_kernel(EvalParams P) {
     // instantiations, the largest process of their NMAX (the stratified
     // queue's item sums need the room).  A compile-time constant: read as a
     // kernel parameter, the plain 2 -> 2 kernel measured 1.8% slower.
-    constexpr int kDims = STRAT ? 3 * (NMAX - 2) : kMaxDim;
+    constexpr bool kScreen = sizeof(R) == 8 && SPL == 2 && !STRAT;
+    constexpr int kDims = STRAT || kScreen ? 3 * (NMAX - 2) : kMaxDim;
     const int map_elems = kDims * P.geo.nbins_max;
     R* s_hist = reinterpret_cast<R*>(s_map + map_elems);      // [warps][map_elems]
     double* s_red = reinterpret_cast<double*>(s_hist + (((THREADS / 32) * map_elems + 3) & ~3));
-    float* s_queue = reinterpret_cast<float*>(s_red + 2 * 32);   // FP32: [warps][queue_words][kQueueSlots]
+    float* s_queue = reinterpret_cast<float*>(s_red + 2 * 32);   // FP32: [warps][queue_words][kQueueSlots]; FP64 screen: see run_segment
 
+    if constexpr (kScreen)                   // the FP64 loop's function tables
+        for (int k = threadIdx.x; k < 3 * kTrigEntries + kExpEntries; k += blockDim.x)
+            reinterpret_cast<double*>(s_queue)[k] = kMathTable[k];
     // spline tables of all species, once per CTA
     {
         const R* gc = static_cast<const R*>(P.coef);

@@ -184,7 +184,7 @@ struct SpeciesConst {
     double eta;             // +1 BE, -1 FD, 0 MB
     double tail_lo_a, tail_lo_b, tail_hi_a, tail_hi_b;
     int32_t stat;
-    int32_t pad_;
+    float log2_fmax;        // log2 of the largest grid value of this sweep (screen of the FP64 sample loop)
 };
 
 // The not-a-knot spline of one grid, laid out once per context: the tridiagonal
@@ -521,6 +521,31 @@ struct SampleVariant {
     int32_t spl;            // samples a lane evaluates per step of the FP32 loop
 };
 constexpr int kMaxVariants = 12;
+
+// Dynamic shared memory of a sample-kernel variant, in the kernel's layout:
+// spline tables of all species, the map table, per-warp histograms, the
+// reduction scratch and the per-warp sample queues.  Map table and histograms
+// hold 12 dimensions in the plain FP32 variants and in the plain FP64 one, and
+// those of the instantiation's largest process otherwise.  The FP64 variant
+// with the FP32 screen (spl 2) adds its function tables, the segment's
+// constants and the FP32 map table.
+constexpr int kMathDoubles = 3 * 65 + 32 + 1;      // math_table.cuh, rounded up to 16 bytes
+constexpr int kSetupBytes = 768;
+inline size_t sample_smem_bytes(bool f32, int n_grid, int n_species, int nbins_max, int nmax, bool ext, bool any_strat,
+                                int threads, int spl) {
+    const size_t rs = f32 ? 4 : 8;
+    const size_t tab = static_cast<size_t>(n_species) * 4 * (n_grid - 1) + n_grid;
+    const bool screen = !f32 && spl == 2;
+    const int dims = ext ? (nmax <= 4 ? 6 : 12) : (screen ? 3 * ((nmax <= 4 ? 4 : nmax) - 2) : kMaxDim);
+    const size_t map_elems = static_cast<size_t>(dims) * nbins_max;
+    const size_t warps = static_cast<size_t>(threads / 32);
+    size_t queue = 0;
+    if (f32) queue = sizeof(float) * warps * (any_strat ? strat_queue_floats(nmax) : kQueueSlots * queue_words(nmax));
+    if (screen)
+        queue = sizeof(double) * kMathDoubles + kSetupBytes + 8 * map_elems + sizeof(uint32_t) * warps * 2 * dims * kQueueSlots;
+    return rs * ((tab + 3) & ~size_t(3)) + 2 * rs * map_elems + rs * ((warps * map_elems + 3) & ~size_t(3)) +
+           2 * 32 * sizeof(double) + queue;
+}
 
 // Samples per Philox group of a D-dimensional task stream (FP32: 4 uniforms
 // per block, FP64: 2).

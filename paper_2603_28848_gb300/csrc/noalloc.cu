@@ -23,8 +23,7 @@ __global__ void prepare_kernel(Geometry, const SideDesc*, const TaskDesc*, const
                                const TimeState*, const double*, TaskConst*, TaskAcc*, int, const double*,
                                const SpeciesConst*, SegConst32*, const SideConst*);
 __global__ void map32_kernel(Geometry, const TaskDesc*, int, const double*, float2*);
-void* eval_kernel_ptr_f32(int nmax);
-void* eval_kernel_ptr_f64(int nmax);
+int eval_variants(bool f32, int nmax, SampleVariant* v, bool strat);
 best_status check_config(const best_config* cfg);
 best_status report(best_status st, const char* msg);
 bool describe_task(const best_config* cfg, int32_t task, SideDesc* sd, TaskDesc* td);
@@ -231,14 +230,20 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
     g.precision = cfg->precision;
 
     // Launch shape of the sample kernel (shared memory limit raised, never lowered).
-    void* fn = f32 ? eval_kernel_ptr_f32(sd.n) : eval_kernel_ptr_f64(sd.n);
-    const size_t rs = f32 ? 4 : 8;
     const size_t spl = static_cast<size_t>(S) * 4 * (n - 1) + n;
-    const size_t map_elems = static_cast<size_t>(kMaxDim) * nb;
-    const size_t hist_elems = static_cast<size_t>(kThreads / 32) * map_elems;
-    const size_t smem = rs * ((spl + 3) & ~size_t(3)) + 2 * rs * map_elems + rs * ((hist_elems + 3) & ~size_t(3)) +
-                        2 * 32 * sizeof(double) +
-                        (f32 ? sizeof(float) * (kThreads / 32) * kQueueSlots * queue_words(sd.n) : 0);
+    SampleVariant variants[kMaxVariants];
+    const int nv = eval_variants(f32, sd.n, variants, false);
+    int max_optin = 0;
+    if (cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return report(BEST_ERR_CUDA, "noalloc: kernel query failed");
+    // the first variant, or in FP64 the one with smaller tables where that does not fit
+    int pick = 0;
+    auto smem_of = [&](int v) {
+        return sample_smem_bytes(f32, n, S, nb, sd.n, false, false, variants[v].threads, variants[v].spl);
+    };
+    if (!f32 && nv > 1 && smem_of(0) > static_cast<size_t>(max_optin)) pick = 1;
+    void* fn = variants[pick].fn;
+    const size_t smem = smem_of(pick);
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return report(BEST_ERR_CUDA, "noalloc: kernel query failed");
     if (static_cast<size_t>(fa.maxDynamicSharedSizeBytes) < smem &&

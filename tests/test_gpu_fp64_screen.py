@@ -1,0 +1,72 @@
+"""The FP64 sample loop screens samples in FP32 and evaluates in FP64 only those
+that can matter.  Against the oracle (which evaluates every sample in FP64) at
+the sizes and widths where a screen can go wrong: fewer samples than a queue
+of a warp, odd budgets, few and many increments, a Gaussian so wide that every
+sample is kept, so narrow that hardly any is, a fractional width, massless and
+heavy legs, both sides of 2 -> 3, 2 -> 4, an expansion; and a grid whose tables
+leave no room for the queues (the plain loop runs).
+
+Tolerances: both sides evaluate the same samples in FP64; FP64 rounding of the
+energy balance (1e-15 of 50) over the narrowest width (1e-3) is 5e-11 of an
+exponent of at most 750, so 1e-7 of a task's mean, 1e-6 of its error.
+"""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import workloads as W
+from tests._helpers import oracle_sweep, task_arrays
+
+pytestmark = pytest.mark.gpu
+
+
+def _mb(n, neval, nbins=50, **kw):
+    prob, f0 = W.c1_maxwell_2to2(n, neval, 1)
+    return replace(prob, processes=tuple(replace(p, nbins=nbins, **kw) for p in prob.processes)), f0, 0.0
+
+
+CASES = {
+    "few samples": lambda: _mb(6, 7),
+    "one warp": lambda: _mb(6, 33),
+    "odd budget, 2 increments": lambda: _mb(8, 1023, nbins=2),
+    "256 increments": lambda: _mb(6, 1500, nbins=256),
+    "every sample kept": lambda: _mb(8, 1500, sigma_E=50.0),
+    "hardly any kept": lambda: _mb(8, 20_000, sigma_E=1e-3),
+    "fractional width": lambda: _mb(8, 3000, width_mode=1, width=0.02),
+    "massless Bose": lambda: (*W.c2_bose_2to2(8, 2999, 1), 0.0),
+    "2 to 3": lambda: (*W.c3_cannibal_2to3(6, 1501, 1, True), 0.0),
+    "2 to 4": lambda: (*W.c5_2to4(5, 700, 1), 0.0),
+    "expansion": lambda: (*W.c4_multi_species(6, 500, 900, 1), 2.0),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_matches_oracle(name):
+    import torch
+    from paper_2603_28848_gb300 import Collision
+    prob, f0, t = CASES[name]()
+    col = Collision(prob, W.PREC_FP64)
+    assert col.launch_shape()[2] == 2          # the screened loop
+    col.eval(torch.tensor(f0, device="cuda"), t)
+    mean, err = col.task_results()
+    col.close()
+    _, _, detail, _ = oracle_sweep(prob, f0, t, "f64")
+    om, oe = task_arrays(detail, len(mean))
+    ok = np.isfinite(om)                       # (the oracle's 1 / variance overflows for an estimate of 1e-159)
+    assert ok.mean() > 0.8
+    assert np.all(np.abs(mean - om)[ok] <= (1e-7 * np.abs(om) + 1e-300)[ok])
+    assert np.all(np.abs(err - oe)[ok] <= (1e-6 * np.abs(oe) + 1e-300)[ok])
+
+
+def test_large_grid_takes_the_plain_loop():
+    import torch
+    from paper_2603_28848_gb300 import Collision
+    prob, f0 = W.c2_bose_2to2(2500, 16, 1)     # 180 KB of spline tables
+    col = Collision(prob, W.PREC_FP64)
+    assert col.launch_shape()[2] == 1
+    f = torch.tensor(f0, device="cuda")
+    C, err = col.eval(f, 0.0)
+    col.check()
+    assert bool(torch.isfinite(C).all()) and bool((C != 0).any())
+    col.close()
