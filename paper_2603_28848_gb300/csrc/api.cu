@@ -594,6 +594,8 @@ best_status enqueue_sweep(best_ctx* ctx, const SweepStart& ss, const double* src
         P.chunk_counter = ctx->d_chunk_ctr + it;
         P.coef = f32 ? static_cast<const void*>(ctx->d_coef32) : static_cast<const void*>(ctx->d_coef64);
         P.knots = f32 ? static_cast<const void*>(ctx->d_knots32) : static_cast<const void*>(ctx->d_knots);
+        P.coef32 = ctx->d_coef32;
+        P.knots32 = ctx->d_knots32;
         P.partials = ctx->d_partials;
         P.item_h = ctx->d_item_h;
         P.strat_m = ctx->d_strat_m;

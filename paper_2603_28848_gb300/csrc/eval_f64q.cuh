@@ -14,13 +14,11 @@
 //   * samples whose Gaussian exponent is below -1100 (|dE| > 39 sigma): their
 //     FP64 weight is exactly 0 (2^-1075 is the smallest subnormal);
 //   * samples with L < log2(largest |w_n| this warp has evaluated in the
-//     segment) - kDropBits, kDropBits = 170.  L takes the kinematic factors
-//     from FP32 (a few bits) and the statistical factors from their maximum
-//     on the grid; a spline's overshoot or a tail above that maximum would
-//     have to exceed 2^60 for such a sample to reach 2^-110 of the largest.
-//     Even 2^31 of them are below the rounding of the sums of w and w^2, and
-//     an increment holding nothing else has a share below the 1e-30 that the
-//     refinement counts as empty.
+//     segment) - kDropBits, kDropBits = 120.  L takes the kinematic factors and
+//     the statistical ones from FP32 with their rounding bounded (a few bits).
+//     Even 2^31 samples of 2^-120 are far below the rounding of the sums of w
+//     and w^2, and an increment holding nothing else has a share below the
+//     1e-30 = 2^-100 of w^2 that the refinement counts as empty.
 // A sample whose FP32 quantities leave the normal range is kept.
 //
 // Measured per launch on trained maps, plain loop -> this one: MB 2 -> 2, 32
@@ -32,7 +30,7 @@
 
 namespace best {
 
-constexpr float kDropBits = 170.0f;
+constexpr float kDropBits = 120.0f;
 
 // ---- FP64 elementary functions of this loop: fewer FP64 operations than the
 // library's, at the price of a restricted range (checked or falling back) ----
@@ -201,16 +199,33 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
     return cut ? 0.0 : w;
 }
 
-// Upper bound of log2 of the kinematic part of a sample's weight from FP32
-// arithmetic, y the mapped point and jac the map's Jacobian; *gauss gets an
-// upper bound of the Gaussian's exponent.  Every momentum component carries at
-// most about 4e-6 of the momenta (sin.approx and cos.approx: 2^-21 absolute;
-// the FP32 map: 2^-22 of an angle), every energy 2e-7: 4e-5 of the energies'
-// sum covers the balance ten times.  +inf where a factor leaves the normal
-// range (or is not a number).
+// log2 of an upper bound of |ca + cb f| at comoving q inside the grid: the FP32
+// spline value plus its rounding bound (2^-18 of its terms' magnitudes).
+__device__ __forceinline__ float log2_factor_bound(const float* coef, const float* knots, float q, const Geometry& g,
+                                                   float inv_step, float q0, float lq0_step, float ca) {
+    int j = static_cast<int>(g.log_spaced ? fmaf(lg2_ftz(q), inv_step, -lq0_step) : (q - q0) * inv_step);
+    j = min(max(j, 0), g.n_grid - 2);
+    const float t = q - __ldg(knots + j);
+    const float4 c = __ldg(reinterpret_cast<const float4*>(coef) + j);
+    const float f = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);
+    const float at = fabsf(t);
+    const float size = fmaf(fmaf(fmaf(fabsf(c.w), at, fabsf(c.z)), at, fabsf(c.y)), at, fabsf(c.x));
+    return lg2_ftz(fmaxf(ca + fmaxf(f, 0.0f) + 3.8e-6f * size, 1e-36f));       // (FP32 subnormals flush to 0)
+}
+
+// Upper bound of log2 |w_n| of a sample from FP32 arithmetic, y the mapped
+// point and jac the map's Jacobian; gauss gets an upper bound of the
+// Gaussian's exponent.  Every momentum component carries at most about 4e-6
+// of the momenta (sin.approx and cos.approx: 2^-21 absolute; the FP32 map:
+// 2^-22 of an angle), every energy 2e-7: 4e-5 of the energies' sum covers the
+// balance ten times.  +inf where a factor leaves the normal range (or is not a
+// number).
 template <int NLEG>
-__device__ __forceinline__ float log2_kin_bound(const SegConst<float, NLEG>& C, const float* y, float jac, float* gauss) {
+__device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& S, const EvalParams& P, const float* y,
+                                                   float jac, float* gauss) {
     constexpr int NI = NLEG - 2;
+    const SegConst<float, NLEG>& C = S.C;
+    const Geometry& g = P.geo;
     float px = 0.0f, py = 0.0f, pz = C.pobs_sig;
     float bal = C.sgn_obs_E, Esum = C.e_obs;
     float prod = jac;
@@ -232,7 +247,8 @@ __device__ __forceinline__ float log2_kin_bound(const SegConst<float, NLEG>& C, 
         Esum += E;
         prod *= r * r * st * rE;
     }
-    const float Ec2 = fmaf(px, px, fmaf(py, py, fmaf(pz, pz, C.m2c)));
+    const float pc2 = fmaf(px, px, fmaf(py, py, pz * pz));
+    const float Ec2 = pc2 + C.m2c;
     const float rEc = rsqrt_ftz(Ec2);
     const float Ec = Ec2 * rEc;
     bal = fmaf(C.sgn_cons, Ec, bal);
@@ -248,7 +264,25 @@ __device__ __forceinline__ float log2_kin_bound(const SegConst<float, NLEG>& C, 
     }
     const float e = C.gauss_k * d * d;
     *gauss = e;
-    return prod > 1e-37f && prod < 1e37f ? lg2_ftz(prod) + extra + e : __int_as_float(0x7f800000);
+    if (!(prod > 1e-37f && prod < 1e37f)) return __int_as_float(0x7f800000);
+    const float kin = lg2_ftz(prod) + extra + e;
+    // the statistical factors, 1 + f or f of every leg (|ca + cb f| is at most ca + f)
+    const int ncoef = 4 * (g.n_grid - 1);
+    float stat = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NI; ++j)
+        stat += log2_factor_bound(P.coef32 + C.spc[j] * ncoef, P.knots32, y[3 * j], g, S.inv_step, S.q0, S.lq0_step,
+                                  C.ca[j]);
+    const float qc = sqrtf(pc2) * C.a;
+    if (qc > S.q0 && qc < S.qN) {
+        stat += log2_factor_bound(P.coef32 + C.sp_cons * ncoef, P.knots32, qc, g, S.inv_step, S.q0, S.lq0_step, C.cac);
+    } else {
+        // Eq. (13) tail: at most 1.6 e^-x for x > 1; anything for a smaller x
+        const float x = qc > S.q0 ? fmaf(C.thi_b, Ec, C.thi_a) : fmaf(C.tlo_b, Ec, C.tlo_a);
+        if (!(x > 1.0f)) return __int_as_float(0x7f800000);
+        stat += C.cac != 0.0f ? 1.0f : fmaf(-1.44268f, x, 0.7f + 1e-5f * x);
+    }
+    return kin + stat + 2.0f;
 }
 
 // FP64 words of sample group g: the four Philox words of every block.
@@ -291,11 +325,7 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
     }
     SegSetup<float, NLEG> s32;
     seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
-    // log2 of an upper bound of c0 times the statistical factors on the grid
-    float stat_bits = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f)) + 1.0f;
-#pragma unroll
-    for (int j = 0; j <= NI; ++j)
-        stat_bits += fmaxf(P.sconst[sd.leg_species[j < NI ? sd.integ[j] : sd.cons]].log2_fmax, 0.0f) + 1.0f;
+    const float log2_c0 = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f));     // (upper bound)
     __syncthreads();
     const SegConst<double, NLEG>& C = s_setup->C;
     const double* knots = s_spline + g.n_species * 4 * (g.n_grid - 1);
@@ -305,7 +335,7 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
     const uint32_t lanes_below = (1u << lane) - 1u;
     int qn = 0;                             // queued samples (warp-uniform)
     int wmax = 0;                           // high word of the largest |w_n| evaluated by this warp
-    float cutoff = -3.0e38f;                // samples with log2_kin_bound below this cannot matter
+    float cutoff = -3.0e38f;                // samples with log2_weight_bound below this cannot matter
 
     auto drain = [&](int slot) {
         double y[D], jac = 1.0;
@@ -355,7 +385,7 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
                 jac *= e.dy;
             }
             float gauss;
-            const float l = log2_kin_bound<NLEG>(s32.C, y, jac, &gauss);
+            const float l = log2_weight_bound<NLEG>(s32, P, y, jac, &gauss);
             const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
             const uint32_t vote = __ballot_sync(0xffffffffu, keep);
             if (keep) {
@@ -370,7 +400,7 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
                 const int top = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(hi)));
                 if (top > wmax && top < 0x7FE00000) {
                     wmax = top;
-                    cutoff = static_cast<float>((top >> 20) - 1023) - stat_bits - kDropBits;
+                    cutoff = static_cast<float>((top >> 20) - 1023) - log2_c0 - kDropBits;
                 }
                 __syncwarp();
                 if (lane < qn - 32) {

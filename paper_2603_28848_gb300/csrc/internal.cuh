@@ -184,7 +184,7 @@ struct SpeciesConst {
     double eta;             // +1 BE, -1 FD, 0 MB
     double tail_lo_a, tail_lo_b, tail_hi_a, tail_hi_b;
     int32_t stat;
-    float log2_fmax;        // log2 of the largest grid value of this sweep (screen of the FP64 sample loop)
+    int32_t pad_;
 };
 
 // The not-a-knot spline of one grid, laid out once per context: the tridiagonal
@@ -431,6 +431,8 @@ struct EvalParams {
     int32_t* chunk_counter;     // next chunk to take (reset to 0 before the launch); NULL: CTA b takes chunk b
     const void* coef;           // [species][n-1][4] in R
     const void* knots;          // [n] in R
+    const float* coef32;        // the same in FP32 (screen of the FP64 sample loop)
+    const float* knots32;
     double* partials;
     const uint32_t* item_h;     // stratified: hypercube of every item
     const int32_t* strat_m;     // stratified: items per hypercube

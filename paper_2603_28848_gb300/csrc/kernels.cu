@@ -198,14 +198,7 @@ __global__ void spline_build_kernel(Geometry g, SweepStart ss, const double* __r
                 if (warp == 1) { sc[s].tail_lo_a = a0; sc[s].tail_lo_b = b; }
                 else { sc[s].tail_hi_a = a0; sc[s].tail_hi_b = b; }
             }
-        } else {
-            float top = 0.0f;
-            for (int j = threadIdx.x - 96; j < n; j += 32) top = fmaxf(top, static_cast<float>(f[j]));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-            if (threadIdx.x == 96) sc[s].log2_fmax = log2f(fmaxf(top, 1e-37f));
-        }
-        if (ss.law && threadIdx.x == 96) {
+        } else if (ss.law && threadIdx.x == 96) {
             ts->mass[s] = mass;
             if (s == 0) {
                 ts->t = t;

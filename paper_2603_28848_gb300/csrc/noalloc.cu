@@ -342,6 +342,8 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
     P.chunk_counter = nullptr;
     P.coef = f32 ? static_cast<const void*>(coef32) : static_cast<const void*>(coef64);
     P.knots = f32 ? static_cast<const void*>(knots32) : static_cast<const void*>(knots);
+    P.coef32 = coef32;
+    P.knots32 = knots32;
     P.partials = reinterpret_cast<double*>(base + kOffPart);
     P.item_h = nullptr;                 // no stratified sampling here (rejected above)
     P.strat_m = nullptr;
