@@ -183,6 +183,7 @@ struct best_ctx {
     int nk_m = 0;
     int n_processes = 0;
     size_t vjp_smem = 0;
+    bool vjp_screen = false, jvp_screen = false;   // FP64 adjoint / tangent kernels with the FP32 screen
     // variance-driven budgets: per-process controls, the device budgets as last
     // read back (for host-built partitions), and the device partition builder
     bool any_budget = false;
@@ -1038,6 +1039,16 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
                         (f32 ? sizeof(float) * ngc + queue * vjp_queue_words(ctx->nmax_legs, false) : 0);
         ctx->jvp_smem = rs * ((spl + 3) & ~size_t(3)) + 2 * rs * map_elems + 12 * 8 * sizeof(double) + rs * ngc +
                         (f32 ? queue * vjp_queue_words(ctx->nmax_legs, true) : 0);
+        if (!f32) {
+            // the FP32 screen's tables and queues where they fit
+            int max_optin = 0;
+            cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            const size_t more = vjp_screen_bytes(nb_max, ctx->nmax_legs, kThreads);
+            ctx->vjp_screen = ctx->vjp_smem + more <= static_cast<size_t>(max_optin);
+            ctx->jvp_screen = ctx->jvp_smem + more <= static_cast<size_t>(max_optin);
+            if (ctx->vjp_screen) ctx->vjp_smem += more;
+            if (ctx->jvp_screen) ctx->jvp_smem += more;
+        }
     }
     CKI(cudaMemset(ctx->d_prev, 0, sizeof(double) * T));
     CKI(cudaMemcpy(ctx->d_sides, ctx->sides.data(), g.n_side * sizeof(SideDesc), cudaMemcpyHostToDevice));
@@ -1338,6 +1349,7 @@ best_status best_collision_vjp(best_ctx* ctx, const double* f_dev, double t, con
     for (int r = 0; r < 20; ++r) P.rk[r] = key.k[r];
     V.task_u = ctx->d_u;
     V.gcoef = ctx->d_gcoef;
+    V.screen = ctx->vjp_screen ? 1 : 0;
     V.dcoef = nullptr;
     V.dtail = nullptr;
     void* args[] = {&V};
@@ -1439,6 +1451,7 @@ static best_status enqueue_jvp(best_ctx* ctx, const double* f_dev, double t, con
     for (int r = 0; r < 20; ++r) P.rk[r] = key.k[r];
     V.task_u = ctx->d_u;
     V.gcoef = nullptr;
+    V.screen = ctx->jvp_screen ? 1 : 0;
     V.dcoef = f32 ? static_cast<const void*>(ctx->d_dcoef32) : static_cast<const void*>(ctx->d_dcoef64);
     V.dtail = ctx->d_dtail;
     void* args[] = {&V};

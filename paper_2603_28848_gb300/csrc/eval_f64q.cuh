@@ -199,6 +199,32 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
     return cut ? 0.0 : w;
 }
 
+// VEGAS map of one 52-bit uniform k + 1/2 from its Philox words, table: the
+// dimension's increments.  (2 k + 1) nb: the increment is the part above bit
+// 53, the fraction the 53 bits below it (the last bit dropped).
+__device__ __forceinline__ Real2<double> map_point64(uint32_t x0, uint32_t x1, int nb, const Real2<double>* table,
+                                                     double* y, uint32_t* bin = nullptr) {
+    const uint64_t k = (static_cast<uint64_t>(x0 >> 6) << 26) | (x1 >> 6);
+    const uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);
+    const uint32_t b = static_cast<uint32_t>(m >> 53);
+    const uint64_t fr = 0x3FF0000000000000ull | ((m >> 1) & 0x000FFFFFFFFFFFFFull);
+    const Real2<double> e = table[b];
+    *y = fma(e.dy, __longlong_as_double(static_cast<long long>(fr)) - 1.0, e.y0);
+    if (bin) *bin = b;
+    return e;
+}
+
+// The same in FP32 from the uniform's first 32 bits (an increment's edge may
+// fall to its neighbour: the mapped point is continuous there).  Returns the
+// increment's width.
+__device__ __forceinline__ float map_point32(uint32_t x0, uint32_t x1, int nb, const Real2<float>* table, float* y) {
+    const uint32_t x = (x0 & ~63u) | (x1 >> 26);
+    const uint64_t m = static_cast<uint64_t>(x) * static_cast<uint32_t>(nb);
+    const Real2<float> e = table[static_cast<uint32_t>(m >> 32)];
+    *y = fmaf(e.dy, static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f, e.y0);
+    return e.dy;
+}
+
 // log2 of an upper bound of |ca + cb f| at comoving q inside the grid: the FP32
 // spline value plus its rounding bound (2^-18 of its terms' magnitudes).
 __device__ __forceinline__ float log2_factor_bound(const float* coef, const float* knots, float q, const Geometry& g,
@@ -219,8 +245,8 @@ __device__ __forceinline__ float log2_factor_bound(const float* coef, const floa
 // of the momenta (sin.approx and cos.approx: 2^-21 absolute; the FP32 map:
 // 2^-22 of an angle), every energy 2e-7: 4e-5 of the energies' sum covers the
 // balance ten times.  +inf where a factor leaves the normal range (or is not a
-// number).
-template <int NLEG>
+// number).  STAT false: of the kinematic part alone.
+template <int NLEG, bool STAT>
 __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& S, const EvalParams& P, const float* y,
                                                    float jac, float* gauss) {
     constexpr int NI = NLEG - 2;
@@ -266,6 +292,7 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     *gauss = e;
     if (!(prod > 1e-37f && prod < 1e37f)) return __int_as_float(0x7f800000);
     const float kin = lg2_ftz(prod) + extra + e;
+    if constexpr (!STAT) return kin + 2.0f;
     // the statistical factors, 1 + f or f of every leg (|ca + cb f| is at most ca + f)
     const int ncoef = 4 * (g.n_grid - 1);
     float stat = 0.0f;
@@ -342,15 +369,9 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
         uint32_t bins[(D + 3) / 4] = {};
 #pragma unroll
         for (int d = 0; d < D; ++d) {
-            // (2 k + 1) nb, k the 52-bit uniform: the increment is the part above bit 53, the
-            // fraction the 53 bits below it (its last bit dropped)
-            const uint32_t x0 = q[(2 * d) * kQueueSlots + slot], x1 = q[(2 * d + 1) * kQueueSlots + slot];
-            const uint64_t k = (static_cast<uint64_t>(x0 >> 6) << 26) | (x1 >> 6);
-            const uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);
-            const uint32_t b = static_cast<uint32_t>(m >> 53);
-            const uint64_t fr = 0x3FF0000000000000ull | ((m >> 1) & 0x000FFFFFFFFFFFFFull);
-            const Real2<double> e = s_map[d * nb + b];
-            y[d] = fma(e.dy, __longlong_as_double(static_cast<long long>(fr)) - 1.0, e.y0);
+            uint32_t b;
+            const Real2<double> e = map_point64(q[(2 * d) * kQueueSlots + slot], q[(2 * d + 1) * kQueueSlots + slot], nb,
+                                                s_map + d * nb, &y[d], &b);
             jac = d == 0 ? e.dy : jac * e.dy;
             bins[d >> 2] |= b << (8 * (d & 3));
         }
@@ -375,17 +396,10 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
             const bool valid = grp < g1 && grp * G + sgi < N;
             float y[D], jac = 1.0f;
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                // the uniform's first 32 bits (an increment's edge may fall to its neighbour: the
-                // mapped point is continuous there)
-                const uint32_t x = (uw[2 * (sgi * D + d)] & ~63u) | (uw[2 * (sgi * D + d) + 1] >> 26);
-                const uint64_t m = static_cast<uint64_t>(x) * static_cast<uint32_t>(nb);
-                const Real2<float> e = s_map32[d * nb + static_cast<uint32_t>(m >> 32)];
-                y[d] = fmaf(e.dy, static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f, e.y0);
-                jac *= e.dy;
-            }
+            for (int d = 0; d < D; ++d)
+                jac *= map_point32(uw[2 * (sgi * D + d)], uw[2 * (sgi * D + d) + 1], nb, s_map32 + d * nb, &y[d]);
             float gauss;
-            const float l = log2_weight_bound<NLEG>(s32, P, y, jac, &gauss);
+            const float l = log2_weight_bound<NLEG, true>(s32, P, y, jac, &gauss);
             const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
             const uint32_t vote = __ballot_sync(0xffffffffu, keep);
             if (keep) {

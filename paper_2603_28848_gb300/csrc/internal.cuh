@@ -449,6 +449,8 @@ struct VjpParams {
     double* gcoef;              // VJP: [species][n-1][4] FP64 coefficient gradients (atomics)
     const void* dcoef;          // JVP: tangent spline coefficients of u, [species][n-1][4] in R
     const double* dtail;        // JVP: tail tangents [species][4] = (da, db) low end, (da, db) high end
+    int32_t screen;             // FP64: shared memory holds the tables and queues of the FP32 screen
+    int32_t pad_;
 };
 
 // Variance-driven budgets of one process: its tasks [first, first + count)
@@ -547,6 +549,12 @@ inline size_t sample_smem_bytes(bool f32, int n_grid, int n_species, int nbins_m
         queue = sizeof(double) * kMathDoubles + kSetupBytes + 8 * map_elems + sizeof(uint32_t) * warps * 2 * dims * kQueueSlots;
     return rs * ((tab + 3) & ~size_t(3)) + 2 * rs * map_elems + rs * ((warps * map_elems + 3) & ~size_t(3)) +
            2 * 32 * sizeof(double) + queue;
+}
+
+// Shared memory the FP32 screen adds to the FP64 adjoint and tangent kernels.
+inline size_t vjp_screen_bytes(int nbins_max, int nmax, int threads) {
+    return sizeof(double) * kMathDoubles + 8 * static_cast<size_t>(kMaxDim) * nbins_max +
+           sizeof(uint32_t) * static_cast<size_t>(threads / 32) * 2 * (3 * (nmax - 2)) * kQueueSlots;
 }
 
 // Samples per Philox group of a D-dimensional task stream (FP32: 4 uniforms

@@ -72,7 +72,7 @@ template <typename R, int NLEG, bool JVP, bool ME>
 __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& seg, const SideDesc& sd,
                                             const TaskDesc& td, const TaskConst& tc, R* s_spline,
                                             Real2<R>* s_map, double* s_gc, double* s_red, R* s_dsp,
-                                            float* s_queue) {
+                                            float* s_queue, Real2<float>* s_map32, const double* tab) {
     const EvalParams& P = V.E;
     constexpr int NI = NLEG - 2;
     constexpr int D = 3 * NI;
@@ -110,6 +110,7 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
             v.y0 = static_cast<R>(lo + sc * e0);
             v.dy = static_cast<R>(sc * (e1 - e0));
             s_map[k] = v;
+            if (V.screen) s_map32[k] = Real2<float>{static_cast<float>(v.y0), static_cast<float>(v.dy)};
         }
     }
 
@@ -205,7 +206,6 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
         dta_hi = static_cast<R>(V.dtail[spcn * 4 + 2]);
         dtb_hi = static_cast<R>(V.dtail[spcn * 4 + 3]);
     }
-    const R nbR = static_cast<R>(nb);
     const R q0 = F32 ? R(S->q0) : static_cast<R>(g.q_min), qN = F32 ? R(S->qN) : static_cast<R>(g.q_max);
     const R lq0_step = F32 ? R(S->lq0_step) : static_cast<R>(g.lq0_step);
     const R inv_step = F32 ? R(S->inv_step) : static_cast<R>(g.inv_step);
@@ -349,7 +349,7 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
     // FP32: samples with a non-zero kinematic part are queued per warp and
     // their statistical factors and derivatives evaluated 32 at a time (as in
     // the sample kernel); the warp runs the loop in step so that its votes
-    // see all 32 lanes.  FP64: every sample is accumulated where it is drawn.
+    // see all 32 lanes.
     constexpr int QW = vjp_queue_words(NLEG, JVP);
     float* q = F32 ? s_queue + (tid >> 5) * (kQueueSlots * QW) : nullptr;
     const int lane = tid & 31;
@@ -372,127 +372,137 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                        q[(5 + 2 * NI) * kQueueSlots + slot], q[(6 + 2 * NI) * kQueueSlots + slot]);
         }
     };
-    for (int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
-        const int64_t grp = static_cast<int64_t>(gb) + lane;
-        uint32_t uw[F32 ? SS::kUniforms : 1];
-        R u[F32 ? 1 : SS::kUniforms];
-        if constexpr (F32) group_words<D>(uw, static_cast<uint32_t>(grp), P.itn, ts.call, task, P.rk);
-        else group_uniforms<D, F32, R>(u, grp, P.itn, ts.call, task, P.rk);
+    // Kinematic part of one sample at the mapped point y with map Jacobian jac
+    // (kin_at of the sample kernel, plus what the derivatives need).
+    struct Kin {
+        R base, r[NI], rE[NI], qc, Ec, rEc, dEs, sig_term, me_d;
+    };
+    auto sincos_of = [&](R x, R* sn, R* cs) {
+        if constexpr (F32) RMath<R>::sincos_(x, sn, cs);
+        else sincos_table(x, tab, sn, cs);
+    };
+    auto rsqrt_of = [&](R x) {
+        if constexpr (F32) return RMath<R>::rsqrt_(x);
+        else return rsqrt_halley(x);
+    };
+    auto exp2_of = [&](R x) {
+        if constexpr (F32) return RMath<R>::exp2_(x);
+        else return exp2_table(x, tab);
+    };
+    auto kinematics = [&](const R* y, R jac, bool valid, Kin& k) {
+        R px = R(0), py = R(0), pz = pobs_sig;
+        EBal<R> bal(sgn_obs_E);
+        R Esum = e_obs;
+        R Qx = R(0), Qy = R(0), Qz = obs_in_p, Ein = obs_in_E;
+        R meas = jac;
+        R rinv = R(1);
+        bool cut = obs_cut;
 #pragma unroll
-        for (int sgi = 0; sgi < G; ++sgi) {
-            const bool valid = grp < g1 && grp * G + sgi < N;
-            R y[D];
-            R jac = R(1);
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                int b;
-                R fr;
-                if constexpr (F32) {
-                    const uint64_t m = static_cast<uint64_t>(uw[sgi * D + d]) * static_cast<uint32_t>(nb);
-                    b = static_cast<int>(m >> 32);
-                    fr = static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f;
-                } else {
-                    const R t = u[sgi * D + d] * nbR;
-                    b = static_cast<int>(t);
-                    b = b < nb - 1 ? b : nb - 1;
-                    fr = t - static_cast<R>(b);
-                }
-                const Real2<R> e = s_map[d * nb + b];
-                y[d] = fma(e.dy, fr, e.y0);
-                jac *= e.dy;
-            }
-            R px = R(0), py = R(0), pz = pobs_sig;
-            EBal<R> bal(sgn_obs_E);
-            R Esum = e_obs;
-            R Qx = R(0), Qy = R(0), Qz = obs_in_p, Ein = obs_in_E;
-            R meas = jac;
-            R rinv = R(1);
-            bool cut = obs_cut;
-            R r[NI], rE[NI];
-#pragma unroll
-            for (int j = 0; j < NI; ++j) {
-                r[j] = y[3 * j];
-                R st, ct, sp, cp;
-                RMath<R>::sincos_(y[3 * j + 1], &st, &ct);
-                RMath<R>::sincos_(y[3 * j + 2], &sp, &cp);
-                const R p = r[j] * inv_a;
-                const R ps = p * st;
-                px = fma(-sig[j] * ps, cp, px);
-                py = fma(-sig[j] * ps, sp, py);
-                pz = fma(sig[j] * p, ct, pz);
-                const R E2 = fma(p, p, m2[j]);
-                const R rr = RMath<R>::rsqrt_(E2);
-                const R E = E2 * rr;
-                cut |= E < e_cut;
-                bal.add(sgnE[j] * E);
-                Esum += E;
-                if (me_on) {
-                    Qx = fma(-inw[j] * ps, cp, Qx);
-                    Qy = fma(-inw[j] * ps, sp, Qy);
-                    Qz = fma(inw[j] * p, ct, Qz);
-                    Ein = fma(inw[j], E, Ein);
-                }
-                meas *= r[j] * r[j] * st;
-                rinv *= rr;
-                rE[j] = rr;
-            }
-            const R pc2 = fma(px, px, fma(py, py, pz * pz));
-            const R Ec2 = pc2 + m2c;
-            const R rEc = RMath<R>::rsqrt_(Ec2 > RMath<R>::kTiny ? Ec2 : R(1e-30));
-            const R Ec = Ec2 * rEc;
-            cut |= Ec < e_cut;
-            bal.add(sgn_cons * Ec);
-            const R dE = bal.value();
-            const R qc = pc2 * (pc2 > RMath<R>::kTiny ? RMath<R>::rsqrt_(pc2) : R(0)) * a;
-            // Gaussian and, for the adjoint, 1/sigma^2 and the derivative of
-            // log(1/sigma) with exp(-dE^2 / 2 sigma^2) through sigma(E_k)
-            R gs, inv_sig2, sig_term;
-            if (frac) {
-                Esum += Ec;
-                const R iS = RMath<R>::rcp_(Esum);
-                const R x = dE * iS;
-                gs = RMath<R>::exp2_(gauss_k * x * x) * (R(2) * e_obs * iS);
-                inv_sig2 = four_over_w2 * iS * iS;
-                // d log g / d E_k from sigma: (dE^2 / sigma^2 - 1) / S for every leg
-                sig_term = fma(dE * dE, inv_sig2, R(-1)) * iS;
-            } else {
-                gs = RMath<R>::exp2_(gauss_k * dE * dE);
-                inv_sig2 = inv_sig2_abs;
-                sig_term = R(0);
-            }
-            R base = meas * rinv * rEc * gs;
-            base = (cut || !valid) ? R(0) : base;
-            R me_d = R(0);          // d log P / d E_k of every initial leg: P'(s) / P(s) 2 E_in
+        for (int j = 0; j < NI; ++j) {
+            k.r[j] = y[3 * j];
+            R st, ct, sp, cp;
+            sincos_of(y[3 * j + 1], &st, &ct);
+            sincos_of(y[3 * j + 2], &sp, &cp);
+            const R p = k.r[j] * inv_a;
+            const R ps = p * st;
+            px = fma(-sig[j] * ps, cp, px);
+            py = fma(-sig[j] * ps, sp, py);
+            pz = fma(sig[j] * p, ct, pz);
+            const R E2 = fma(p, p, m2[j]);
+            const R rr = rsqrt_of(E2);
+            const R E = E2 * rr;
+            cut |= E < e_cut;
+            bal.add(sgnE[j] * E);
+            Esum += E;
             if (me_on) {
-                const R qx = fma(cons_inw, px, Qx), qy = fma(cons_inw, py, Qy), qz = fma(cons_inw, pz, Qz);
-                const R e = fma(cons_inw, Ec, Ein);
-                const R sv = fma(e, e, -fma(qx, qx, fma(qy, qy, qz * qz)));
-                const R Pv = fma(fma(fma(mec[3], sv, mec[2]), sv, mec[1]), sv, mec[0]);
-                const R dP = fma(fma(R(3) * mec[3], sv, R(2) * mec[2]), sv, mec[1]);
-                me_d = Pv != R(0) ? R(2) * e * dP * RMath<R>::rcp_(Pv) : R(0);
-                base *= Pv;
+                Qx = fma(-inw[j] * ps, cp, Qx);
+                Qy = fma(-inw[j] * ps, sp, Qy);
+                Qz = fma(inw[j] * p, ct, Qz);
+                Ein = fma(inw[j], E, Ein);
             }
-            const R dEs = dE * inv_sig2;
-            if constexpr (F32) {
-                const bool keep = base != R(0);
+            meas *= k.r[j] * k.r[j] * st;
+            rinv *= rr;
+            k.rE[j] = rr;
+        }
+        const R pc2 = fma(px, px, fma(py, py, pz * pz));
+        const R Ec2 = pc2 + m2c;
+        k.rEc = rsqrt_of(Ec2 > RMath<R>::kTiny ? Ec2 : R(1e-30));
+        k.Ec = Ec2 * k.rEc;
+        cut |= k.Ec < e_cut;
+        bal.add(sgn_cons * k.Ec);
+        const R dE = bal.value();
+        k.qc = pc2 * (pc2 > RMath<R>::kTiny ? rsqrt_of(pc2) : R(0)) * a;
+        // Gaussian and, for the adjoint, 1/sigma^2 and the derivative of
+        // log(1/sigma) with exp(-dE^2 / 2 sigma^2) through sigma(E_k)
+        R gs, inv_sig2;
+        if (frac) {
+            Esum += k.Ec;
+            const R iS = RMath<R>::rcp_(Esum);
+            const R x = dE * iS;
+            gs = exp2_of(gauss_k * x * x) * (R(2) * e_obs * iS);
+            inv_sig2 = four_over_w2 * iS * iS;
+            // d log g / d E_k from sigma: (dE^2 / sigma^2 - 1) / S for every leg
+            k.sig_term = fma(dE * dE, inv_sig2, R(-1)) * iS;
+        } else {
+            gs = exp2_of(gauss_k * dE * dE);
+            inv_sig2 = inv_sig2_abs;
+            k.sig_term = R(0);
+        }
+        R base = meas * rinv * k.rEc * gs;
+        base = (cut || !valid) ? R(0) : base;
+        k.me_d = R(0);          // d log P / d E_k of every initial leg: P'(s) / P(s) 2 E_in
+        if (me_on) {
+            const R qx = fma(cons_inw, px, Qx), qy = fma(cons_inw, py, Qy), qz = fma(cons_inw, pz, Qz);
+            const R e = fma(cons_inw, k.Ec, Ein);
+            const R sv = fma(e, e, -fma(qx, qx, fma(qy, qy, qz * qz)));
+            const R Pv = fma(fma(fma(mec[3], sv, mec[2]), sv, mec[1]), sv, mec[0]);
+            const R dP = fma(fma(R(3) * mec[3], sv, R(2) * mec[2]), sv, mec[1]);
+            k.me_d = Pv != R(0) ? R(2) * e * dP * RMath<R>::rcp_(Pv) : R(0);
+            base *= Pv;
+        }
+        k.base = base;
+        k.dEs = dE * inv_sig2;
+    };
+    if constexpr (F32) {
+        for (int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
+            const int64_t grp = static_cast<int64_t>(gb) + lane;
+            uint32_t uw[SS::kUniforms];
+            group_words<D>(uw, static_cast<uint32_t>(grp), P.itn, ts.call, task, P.rk);
+#pragma unroll
+            for (int sgi = 0; sgi < G; ++sgi) {
+                const bool valid = grp < g1 && grp * G + sgi < N;
+                R y[D];
+                R jac = R(1);
+#pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    const uint64_t m = static_cast<uint64_t>(uw[sgi * D + d]) * static_cast<uint32_t>(nb);
+                    const uint32_t b = static_cast<uint32_t>(m >> 32);
+                    const R fr = static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f;
+                    const Real2<R> e = s_map[d * nb + b];
+                    y[d] = fma(e.dy, fr, e.y0);
+                    jac *= e.dy;
+                }
+                Kin k;
+                kinematics(y, jac, valid, k);
+                const bool keep = k.base != R(0);
                 const uint32_t vote = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
-                    q[slot] = base;
+                    q[slot] = k.base;
 #pragma unroll
-                    for (int j = 0; j < NI; ++j) q[(1 + j) * kQueueSlots + slot] = r[j];
+                    for (int j = 0; j < NI; ++j) q[(1 + j) * kQueueSlots + slot] = k.r[j];
                     if constexpr (JVP) {
-                        q[(1 + NI) * kQueueSlots + slot] = qc;
-                        q[(2 + NI) * kQueueSlots + slot] = Ec;
+                        q[(1 + NI) * kQueueSlots + slot] = k.qc;
+                        q[(2 + NI) * kQueueSlots + slot] = k.Ec;
                     } else {
 #pragma unroll
-                        for (int j = 0; j < NI; ++j) q[(1 + NI + j) * kQueueSlots + slot] = rE[j];
-                        q[(1 + 2 * NI) * kQueueSlots + slot] = qc;
-                        q[(2 + 2 * NI) * kQueueSlots + slot] = Ec;
-                        q[(3 + 2 * NI) * kQueueSlots + slot] = rEc;
-                        q[(4 + 2 * NI) * kQueueSlots + slot] = dEs;
-                        q[(5 + 2 * NI) * kQueueSlots + slot] = sig_term;
-                        q[(6 + 2 * NI) * kQueueSlots + slot] = me_d;
+                        for (int j = 0; j < NI; ++j) q[(1 + NI + j) * kQueueSlots + slot] = k.rE[j];
+                        q[(1 + 2 * NI) * kQueueSlots + slot] = k.qc;
+                        q[(2 + 2 * NI) * kQueueSlots + slot] = k.Ec;
+                        q[(3 + 2 * NI) * kQueueSlots + slot] = k.rEc;
+                        q[(4 + 2 * NI) * kQueueSlots + slot] = k.dEs;
+                        q[(5 + 2 * NI) * kQueueSlots + slot] = k.sig_term;
+                        q[(6 + 2 * NI) * kQueueSlots + slot] = k.me_d;
                     }
                 }
                 qn += __popc(vote);
@@ -507,14 +517,85 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                     __syncwarp();
                     qn -= 32;
                 }
-            } else {
-                accumulate(base, r, rE, qc, Ec, rEc, dEs, sig_term, me_d);
             }
         }
-    }
-    if constexpr (F32) {
         __syncwarp();
         if (lane < qn) drain(lane);
+    } else {
+        // FP64: the screen of the FP64 sample loop (eval_f64q.cuh) queues the
+        // samples' Philox words, and 32 queued samples at a time are evaluated.
+        // It drops exact zeros and samples whose kinematic part is 2^-300 of the
+        // largest this warp has evaluated in the segment: their derivatives,
+        // which miss one statistical factor, stay below the rounding of the
+        // spline's transposed solve by any ratio of statistical factors a grid
+        // in FP64 can hold.  An s-dependent |M|^2 is not in the bound: exact
+        // zeros only.  Without room for the queues every sample is evaluated
+        // where it is drawn.
+        constexpr int W = 2 * D;
+        uint32_t* qw = reinterpret_cast<uint32_t*>(s_queue) + (tid >> 5) * (W * kQueueSlots);
+        int wmax = 0;
+        float cutoff = -3.0e38f;
+        auto sample = [&](const uint32_t* w, int stride, bool valid) {
+            R y[D], jac = R(1);
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const Real2<R> e = map_point64(w[(2 * d) * stride], w[(2 * d + 1) * stride], nb, s_map + d * nb, &y[d]);
+                jac *= e.dy;
+            }
+            Kin k;
+            kinematics(y, jac, valid, k);
+            accumulate(k.base, k.r, k.rE, k.qc, k.Ec, k.rEc, k.dEs, k.sig_term, k.me_d);
+            return __double2hiint(k.base) & 0x7fffffff;
+        };
+        SegSetup<float, NLEG> s32;
+        seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
+        for (int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
+            const int64_t grp = static_cast<int64_t>(gb) + lane;
+            uint32_t uw[2 * SS::kUniforms];
+            group_words64<D>(uw, static_cast<uint32_t>(grp), P.itn, ts.call, task, P.rk);
+#pragma unroll 1
+            for (int sgi = 0; sgi < G; ++sgi) {
+                const bool valid = grp < g1 && grp * G + sgi < N;
+                if (sgi > 0) {
+#pragma unroll
+                    for (int k = 0; k < W; ++k) uw[k] = uw[(G > 1 ? W : 0) + k];
+                }
+                if (!V.screen) {
+                    sample(uw, 1, valid);
+                    continue;
+                }
+                float y[D], jac = 1.0f, gauss;
+#pragma unroll
+                for (int d = 0; d < D; ++d) jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d]);
+                const float l = log2_weight_bound<NLEG, false>(s32, P, y, jac, &gauss);
+                const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
+                const uint32_t vote = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
+#pragma unroll
+                    for (int k = 0; k < W; ++k) qw[k * kQueueSlots + slot] = uw[k];
+                }
+                qn += __popc(vote);
+                if (qn >= 32) {
+                    __syncwarp();
+                    const int hi = sample(qw + lane, kQueueSlots, true);
+                    const int top = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(hi)));
+                    if (!me_on && top > wmax && top < 0x7FE00000) {
+                        wmax = top;
+                        cutoff = static_cast<float>((top >> 20) - 1023) - 300.0f;
+                    }
+                    __syncwarp();
+                    if (lane < qn - 32) {
+#pragma unroll
+                        for (int k = 0; k < W; ++k) qw[k * kQueueSlots + lane] = qw[k * kQueueSlots + 32 + lane];
+                    }
+                    __syncwarp();
+                    qn -= 32;
+                }
+            }
+        }
+        __syncwarp();
+        if (lane < qn) sample(qw + lane, kQueueSlots, true);
     }
 
     // ---- segment record: VJP [w, fobs, mobs, mc, tla, tlb, tha, thb, m_0 .. m_{NI-1}];
@@ -559,7 +640,7 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
 }
 
 template <typename R, int NMAX, bool JVP, bool ME = false>
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) vjp_kernel(VjpParams V) {
+__global__ void __launch_bounds__(kThreads, 2) vjp_kernel(VjpParams V) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const EvalParams& P = V.E;
     R* s_spline = reinterpret_cast<R*>(smem_raw);
@@ -571,8 +652,22 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) vjp_kernel(V
     double* s_red = s_gc + (JVP ? 0 : ngc);
     // JVP: tangent coefficients; FP32 VJP: the segment's coefficient-gradient sums
     R* s_dsp = reinterpret_cast<R*>(s_red + 12 * 8);
-    // FP32: per-warp sample queues after the coefficient table
-    float* s_queue = sizeof(R) == 4 ? reinterpret_cast<float*>(s_dsp + ngc) : nullptr;
+    // FP32: per-warp sample queues after the coefficient table.  FP64 with the
+    // screen: the function tables, the FP32 map table and the queues.
+    float* s_queue;
+    Real2<float>* s_map32 = nullptr;
+    const double* tab = kMathTable;
+    if constexpr (sizeof(R) == 4) {
+        s_queue = reinterpret_cast<float*>(s_dsp + ngc);
+    } else {
+        double* s_tab = reinterpret_cast<double*>(s_dsp) + (JVP ? ngc : 0);
+        s_map32 = reinterpret_cast<Real2<float>*>(s_tab + kMathDoubles);
+        s_queue = reinterpret_cast<float*>(s_map32 + map_elems);
+        if (V.screen) {
+            for (int k = threadIdx.x; k < 3 * kTrigEntries + kExpEntries; k += blockDim.x) s_tab[k] = kMathTable[k];
+            tab = s_tab;
+        }
+    }
     {
         const R* gc = static_cast<const R*>(P.coef);
         for (int k = threadIdx.x; k < ngc; k += blockDim.x) {
@@ -605,10 +700,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 2 : 1) vjp_kernel(V
             const TaskConst tc = P.tconst[seg.task];
             __syncthreads();
             switch (sd.n) {
-                case 3: if constexpr (NMAX >= 3) vjp_segment<R, 3, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue); break;
-                case 4: if constexpr (NMAX >= 4) vjp_segment<R, 4, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue); break;
-                case 5: if constexpr (NMAX >= 5) vjp_segment<R, 5, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue); break;
-                case 6: if constexpr (NMAX >= 6) vjp_segment<R, 6, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue); break;
+                case 3: if constexpr (NMAX >= 3) vjp_segment<R, 3, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue, s_map32, tab); break;
+                case 4: if constexpr (NMAX >= 4) vjp_segment<R, 4, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue, s_map32, tab); break;
+                case 5: if constexpr (NMAX >= 5) vjp_segment<R, 5, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue, s_map32, tab); break;
+                case 6: if constexpr (NMAX >= 6) vjp_segment<R, 6, JVP, ME>(V, seg, sd, td, tc, s_spline, s_map, s_gc, s_red, s_dsp, s_queue, s_map32, tab); break;
                 default: break;
             }
         }
