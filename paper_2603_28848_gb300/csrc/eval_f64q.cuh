@@ -201,15 +201,19 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
 
 // VEGAS map of one 52-bit uniform k + 1/2 from its Philox words, table: the
 // dimension's increments.  (2 k + 1) nb: the increment is the part above bit
-// 53, the fraction the 53 bits below it (the last bit dropped).
+// 53, the fraction the 53 bits below it, turned into an FP64 number in integer
+// operations.
 __device__ __forceinline__ Real2<double> map_point64(uint32_t x0, uint32_t x1, int nb, const Real2<double>* table,
                                                      double* y, uint32_t* bin = nullptr) {
     const uint64_t k = (static_cast<uint64_t>(x0 >> 6) << 26) | (x1 >> 6);
     const uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);
     const uint32_t b = static_cast<uint32_t>(m >> 53);
-    const uint64_t fr = 0x3FF0000000000000ull | ((m >> 1) & 0x000FFFFFFFFFFFFFull);
+    const uint64_t frac = m & ((1ull << 53) - 1);              // exact in FP64
+    const int lz = __clzll(static_cast<long long>(frac));
+    const uint64_t bits = (((frac << lz) >> 11) & 0x000FFFFFFFFFFFFFull) | (static_cast<uint64_t>(1033 - lz) << 52);
+    const double fr = __longlong_as_double(frac ? static_cast<long long>(bits) : 0);
     const Real2<double> e = table[b];
-    *y = fma(e.dy, __longlong_as_double(static_cast<long long>(fr)) - 1.0, e.y0);
+    *y = fma(e.dy, fr, e.y0);
     if (bin) *bin = b;
     return e;
 }
