@@ -26,7 +26,7 @@ __global__ void width_control_kernel(Geometry, const SideDesc*, const TaskDesc*,
                                      double*, double*);
 __global__ void refine_kernel(Geometry, const SideDesc*, const TaskDesc*, const TaskConst*, const int32_t*,
                               const int32_t*, const Segment*, const double*, double*, TaskAcc*, TaskConst*,
-                              const double*, SegConst32*, float2*);
+                              const double*, SegConst32*, float2*, int);
 __global__ void map32_kernel(Geometry, const TaskDesc*, int, const double*, float2*);
 __global__ void strat_init_kernel(const TaskDesc*, int32_t*, uint32_t*, int);
 __global__ void strat_refine_kernel(const TaskDesc*, const int32_t*, const double*, int32_t*, double*, double*,
@@ -106,7 +106,7 @@ struct best_ctx {
     size_t eval_smem = 0;
     size_t spline_smem = 0;
     size_t refine_smem = 0;
-    int refine_threads = 128;       // one thread per entry of a task's reduced record, 128 to 512
+    int refine_threads = 128;       // one thread per entry of one leg's reduced record, 128 to 512
     void* eval_fn = nullptr;
     int n_variants = 0;             // sample-kernel variants (register budget, CTA size, samples per step)
     SampleVariant variants[kMaxVariants] = {};
@@ -630,14 +630,15 @@ best_status enqueue_sweep(best_ctx* ctx, const SweepStart& ss, const double* src
                                                              ctx->d_item_h, ctx->d_strat_est);
             ctx->launches += 1;
         }
-        refine_kernel<<<pl.n_active, ctx->refine_threads, ctx->refine_smem, st>>>(
+        const int legs = ctx->nmax_legs - 2;
+        refine_kernel<<<pl.n_active * legs, ctx->refine_threads, ctx->refine_smem, st>>>(
             g, ctx->d_sides, ctx->d_tasks, ctx->d_tconst, pl.d_active, pl.d_task_seg, pl.d_segs,
             ctx->d_partials, ctx->d_edges, ctx->d_acc, ctx->d_tconst, ctx->d_strat_est, ctx->d_tconst32,
-            ctx->d_map32);
+            ctx->d_map32, legs);
         ctx->launches += 2;
     }
     const int total = g.n_species * g.n_grid;
-    assemble_kernel<<<(total + 255) / 256, 256, 0, st>>>(g, ctx->d_sides, ctx->d_acc, ctx->d_ts, C, err,
+    assemble_kernel<<<(2 * total + 31) / 32, 32, 0, st>>>(g, ctx->d_sides, ctx->d_acc, ctx->d_ts, C, err,
                                                          ctx->d_prev);
     ctx->launches += 1;
     if (ctx->any_adaptive) {
@@ -924,10 +925,10 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
                                      static_cast<int>(ctx->spline_smem)) != cudaSuccess)
                 return bail(fail(ctx, BEST_ERR_CUDA, "cannot set shared memory of the spline kernels"));
         }
-        ctx->refine_smem = sizeof(double) * (5 * static_cast<size_t>(kMaxDim) * nb_max + 4 * kMaxDim + 2);
-        // the refinement's first phase sums each entry of the records (2 + D nb) over the task's
-        // segments, one entry per thread where they fit: a chain of dependent loads per entry
-        ctx->refine_threads = std::min(512, std::max(128, (2 + 3 * (ctx->nmax_legs - 2) * nb_max + 31) / 32 * 32));
+        ctx->refine_smem = sizeof(double) * refine_doubles(nb_max);
+        // the refinement's first phase sums each entry of a leg's records (2 + 3 nb) over the task's
+        // segments, one entry per thread where they fit; at least its four working warps
+        ctx->refine_threads = std::min(512, std::max(128, (2 + 3 * nb_max + 31) / 32 * 32));
         if (cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(&refine_kernel)) != cudaSuccess)
             return bail(fail(ctx, BEST_ERR_CUDA, "cannot query the refinement kernel"));
         if (static_cast<size_t>(fa.maxDynamicSharedSizeBytes) < ctx->refine_smem &&

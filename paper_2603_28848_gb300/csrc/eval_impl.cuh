@@ -1059,27 +1059,25 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     }
 
     // ---- segment reduction into its partial record (FP64) -------------------
-    double vw = acc_w.value(), vw2 = acc_w2.value();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        vw += __shfl_xor_sync(0xffffffffu, vw, o);
-        vw2 += __shfl_xor_sync(0xffffffffu, vw2, o);
-    }
+    // After one exchange the warp's lower half holds w and its upper half w^2,
+    // so that one chain of additions reduces both (an FP64 operation takes its
+    // pipe for 64 cycles per warp: 16 -> 11 of them here).
     const int warp = tid >> 5, lane = tid & 31;
-    if (lane == 0) {
-        s_red[2 * warp] = vw;
-        s_red[2 * warp + 1] = vw2;
+    {
+        const double vw = acc_w.value(), vw2 = acc_w2.value();
+        const bool up = lane >= 16;
+        double v = up ? vw2 : vw;
+        v += __shfl_xor_sync(0xffffffffu, up ? vw : vw2, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0) s_red[2 * warp + (lane >> 4)] = v;
     }
     __syncthreads();
     double* part = P.partials + seg.part;
-    if (tid == 0) {
-        double a0 = 0.0, a1 = 0.0;
-        for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) {
-            a0 += s_red[2 * k];
-            a1 += s_red[2 * k + 1];
-        }
-        part[0] = a0;
-        part[1] = a1;
+    if (tid < 2) {
+        double v = 0.0;
+        for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) v += s_red[2 * k + tid];
+        part[tid] = v;
     }
     for (int k = tid; k < D * nb; k += blockDim.x) {
         // the per-warp histograms summed in their own precision (FP32 for

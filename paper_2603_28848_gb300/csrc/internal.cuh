@@ -401,9 +401,7 @@ __device__ inline SegConst32 seg_const32(const SideDesc& sd, const TaskDesc& td,
 // entry d * nb + b of the task's kMaxDim * nbins_max entries.  Written by
 // map32_kernel (every sweep) and by the refinement for the tasks it refines.
 __host__ __device__ inline int map32_stride(const Geometry& g) { return kMaxDim * g.nbins_max; }
-__device__ inline float2 map32_entry(const double* e_task, int d, int b, int nb, const Geometry& g) {
-    const double e0 = e_task[d * (nb + 1) + b];
-    const double e1 = e_task[d * (nb + 1) + b + 1];
+__device__ inline float2 map32_value(double e0, double e1, int d, const Geometry& g) {     // of edges e0, e1 of dimension d
     double lo, sc;
     switch (d % 3) {
         case 0: lo = g.q_min; sc = g.q_max - g.q_min; break;   // r (comoving)
@@ -412,6 +410,12 @@ __device__ inline float2 map32_entry(const double* e_task, int d, int b, int nb,
     }
     return make_float2(static_cast<float>(lo + sc * e0), static_cast<float>(sc * (e1 - e0)));
 }
+__device__ inline float2 map32_entry(const double* e_task, int d, int b, int nb, const Geometry& g) {
+    return map32_value(e_task[d * (nb + 1) + b], e_task[d * (nb + 1) + b + 1], d, g);
+}
+
+// Dynamic shared memory of refine_kernel, in doubles.
+constexpr int refine_doubles(int nb) { return 15 * nb + 8; }
 
 // Arguments of the sample kernel.
 struct EvalParams {

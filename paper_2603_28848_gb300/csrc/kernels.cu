@@ -678,66 +678,97 @@ __global__ void strat_refine_kernel(const TaskDesc* __restrict__ tasks, const in
 }
 
 // ---------------------------------------------------------------------------
-// End of one VEGAS iteration, one CTA per active task: sum the task's
-// segment records in a fixed order (deterministic), form the iteration
-// estimate and its variance, add them to the combination accumulators, and
-// refine the map (Lepage): smooth the per-increment sums of w^2 with the
-// (7,1)/8, (1,6,1)/8, (1,7)/8 stencil, normalise, compress with
-// ((1-d)/ln(1/d))^alpha, and re-partition into equal shares of the
-// compressed weight.  A normalised share below 1e-30 counts as an empty
-// increment (weight 0, like an exact zero) so that the map does not depend on
-// where underflow of w^2 falls.  Dynamic shared memory: (3 kMaxDim nbins_max
-// + 2 kMaxDim + 2) doubles.
+// End of one VEGAS iteration, one CTA per active task and integrated leg (its
+// three dimensions): sum the task's segment records in a fixed order
+// (deterministic), form the iteration estimate and its variance, add them to
+// the combination accumulators, and refine the map (Lepage): smooth the
+// per-increment sums of w^2 with the (7,1)/8, (1,6,1)/8, (1,7)/8 stencil,
+// normalise, compress with ((1-d)/ln(1/d))^alpha, and re-partition into equal
+// shares of the compressed weight.  A normalised share below 1e-30 counts as an
+// empty increment (weight 0, like an exact zero) so that the map does not
+// depend on where underflow of w^2 falls.
+//
+// Bound by the FP64 pipe (64 cycles per warp operation) and by dependent
+// loads: one warp per dimension runs its dimension from smoothing to edges
+// without block barriers (warp-wide sums and scans, comparisons as integers),
+// while a fourth warp makes the task's scalars; the legs' CTAs spread a small
+// problem over the SMs.  FP32 2 -> 2: 17.8 -> 7.3 us for 64 tasks, 83 -> 42 us for
+// 512.  Dynamic shared memory: refine_doubles(nbins_max) doubles.
 // ---------------------------------------------------------------------------
 __global__ void refine_kernel(Geometry g, const SideDesc* __restrict__ sides,
                               const TaskDesc* __restrict__ tasks, const TaskConst* tconst,
                               const int32_t* __restrict__ active, const int32_t* __restrict__ task_seg,
                               const Segment* __restrict__ segs, const double* __restrict__ partials,
                               double* edges, TaskAcc* acc, TaskConst* tconst_next,
-                              const double* __restrict__ strat_est, SegConst32* tconst32, float2* map32) {
+                              const double* __restrict__ strat_est, SegConst32* tconst32, float2* map32, int legs) {
     extern __shared__ double hist[];
-    const int t = active[blockIdx.x];
-    const TaskDesc td = tasks[t];
+    __shared__ int s_underflow;
+    const int a = blockIdx.x / legs, leg = blockIdx.x - a * legs;
+    const int t = active[a];
+    const int s0 = task_seg[a], s1 = task_seg[a + 1];
+    const TaskDesc& td = tasks[t];
     const int nb = td.nbins;
-    const int D = td.dim;
-    const int s0 = task_seg[blockIdx.x], s1 = task_seg[blockIdx.x + 1];
-    const int L = 2 + D * nb;
-    for (int k = threadIdx.x; k < L; k += blockDim.x) {
-        // the records in segment order; eight loads in flight at a time
-        double v = 0.0;
-        int s = s0;
-        for (; s + 8 <= s1; s += 8) {
-            double a[8];
+    if (3 * leg >= td.dim) return;
+    const int E = 3 * nb;
+    double* head = hist + E;                   // sum w, sum w^2
+    double* sm = head + 2;                     // smoothed, then compressed weights [3][nb]
+    double* olde = sm + E;                     // old edges [3][nb + 1]
+    double* rom = olde + E + 3;                // reciprocals of the compressed weights [3][nb]
+    double* cum = rom + E;                     // running sums of the compressed weights [3][nb + 1]
+    double* e_task = edges + static_cast<int64_t>(t) * g.map_stride + 3 * leg * (nb + 1);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double old0 = tid < E + 3 ? e_task[tid] : 0.0;           // (under way with the records)
+    {
+        // the records in segment order (one after the other in memory); eight loads in flight at a time
+        const int64_t rec = record_doubles(td.dim, nb);
+        const double* part = partials + segs[s0].part;
+        const int n = s1 - s0;
+        for (int k = tid; k < E + 2; k += blockDim.x) {
+            const double* p = part + (k < E ? 2 + leg * E + k : k - E);
+            double v = 0.0;
+            int s = 0;
+            for (; s + 8 <= n; s += 8, p += 8 * rec) {
+                double x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) a[u] = partials[segs[s + u].part + k];
+                for (int u = 0; u < 8; ++u) x[u] = p[u * rec];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v += a[u];
+                for (int u = 0; u < 8; ++u) v += x[u];
+            }
+            for (; s < n; ++s, p += rec) v += *p;
+            hist[k] = v;
         }
-        for (; s < s1; ++s) v += partials[segs[s].part + k];
-        hist[k] = v;
     }
+    if (tid < E + 3) olde[tid] = old0;
+    for (int k = tid + blockDim.x; k < E + 3; k += blockDim.x) olde[k] = e_task[k];
     __syncthreads();
-    // Sum w^2 >= (sum w)^2 / N holds exactly; if the computed sums violate it,
-    // squares of tiny weights underflowed (FP32 path with a poor scale): the
-    // iteration is discarded (no estimate, no refinement) and only the scale
-    // is corrected for the next iteration.
-    const double N = static_cast<double>(td.neval);
-    double mean_n, var_n;
-    bool underflow;
-    if (td.strat_H > 0) {
-        // stratified: estimate, variance and underflow flag from strat_refine_kernel
-        mean_n = strat_est[4 * t];
-        var_n = strat_est[4 * t + 1];
-        underflow = strat_est[4 * t + 2] != 0.0;
-    } else {
-        mean_n = hist[0] / N;
-        underflow = hist[1] / N < (1.0 - 1e-6) * mean_n * mean_n;
-        var_n = N > 1.0 ? (hist[1] / N - mean_n * mean_n) / (N - 1.0) : 0.0;
-        var_n = var_n > 0.0 ? var_n : 0.0;
-    }
-    if (threadIdx.x == 0) {
-        const TaskConst c = tconst[t];
-        const double sc = c.K * c.scale;
+    if (warp > 3) return;
+    if (warp == 3) {
+        // Sum w^2 >= (sum w)^2 / N holds exactly; if the computed sums violate
+        // it, squares of tiny weights underflowed (FP32 path with a poor scale):
+        // the iteration is discarded (no estimate, no refinement) and only the
+        // scale is corrected for the next iteration.
+        const double N = static_cast<double>(td.neval);
+        double mean_n, var_n;
+        bool underflow;
+        if (td.strat_H > 0) {
+            // stratified: estimate, variance and underflow flag from strat_refine_kernel
+            mean_n = strat_est[4 * t];
+            var_n = strat_est[4 * t + 1];
+            underflow = strat_est[4 * t + 2] != 0.0;
+        } else {
+            mean_n = head[0] / N;
+            const double sq = head[1] / N;
+            underflow = sq < (1.0 - 1e-6) * mean_n * mean_n;
+            var_n = N > 1.0 ? (sq - mean_n * mean_n) / (N - 1.0) : 0.0;
+            var_n = var_n > 0.0 ? var_n : 0.0;
+        }
+        if (lane == 0) s_underflow = underflow ? 1 : 0;
+        __syncwarp();
+        asm volatile("bar.arrive 1, 128;" ::: "memory");
+        if (leg != 0 || lane != 0) return;
+        const TaskConst& c = tconst[t];
+        const double K = c.K, old_scale = c.scale, obs_factor = c.obs_factor, c0 = c.c0;
+        const double sc = K * old_scale;
         const double mean = mean_n * sc;
         const double var = var_n * sc * sc;
         if (!underflow) {
@@ -751,120 +782,124 @@ __global__ void refine_kernel(Geometry g, const SideDesc* __restrict__ sides,
             }
         }
         if (mean_n != 0.0) {
-            const double scale = clamp_scale(fabs(mean_n) * c.scale, c.obs_factor);
+            const double scale = clamp_scale(fabs(mean_n) * old_scale, obs_factor);
+            const double next = c0 == 0.0 ? 0.0 : obs_factor / scale;   // a cut observed leg stays cut
             tconst_next[t].scale = scale;
-            tconst_next[t].c0 = c.c0 == 0.0 ? 0.0 : c.obs_factor / scale;   // a cut observed leg stays cut
-            if (tconst32) tconst32[t].c0 = static_cast<float>(tconst_next[t].c0);
+            tconst_next[t].c0 = next;
+            if (tconst32) tconst32[t].c0 = static_cast<float>(next);
         }
+        return;
     }
-    if (underflow) return;
-    // refinement: smoothing and compression in parallel over (dimension,
-    // increment); the running sums of the compressed weights per dimension
-    // (one thread each, in increment order); then every new edge in
-    // parallel: the increment where the running sum reaches k / nb of the
-    // total, and the linear interpolation inside it
-    double* sm = hist + 2 + D * nb;            // smoothed, then compressed weights [D][nb]
-    double* tot = sm + D * nb;                 // per-dimension sums [D], then (FP32 path) their reciprocals [D]
-    double* olde = tot + 2 * D;                // old edges [D][nb + 1]
-    double* rom = olde + D * (nb + 1);         // reciprocals of the compressed weights [D][nb]
-    double* cum = rom + D * nb;                // running sums of the compressed weights [D][nb + 1]
-    const double* e_task = edges + static_cast<int64_t>(t) * g.map_stride;
-    for (int k = threadIdx.x; k < D * (nb + 1); k += blockDim.x) olde[k] = e_task[k];
-    for (int k = threadIdx.x; k < D * nb; k += blockDim.x) {
-        const int d = k / nb, b = k - d * nb;
-        const double* dd = hist + 2 + d * nb;
+    // ---- one dimension per warp ----
+    const bool f32 = g.precision == BEST_FP32;
+    const double* dd = hist + warp * nb;
+    sm += warp * nb;
+    rom += warp * nb;
+    cum += warp * (nb + 1);
+    olde += warp * (nb + 1);
+    double tot = 0.0;
+    for (int b = lane; b < nb; b += 32) {
         double v;
-        if (nb == 1) v = dd[0];
-        else if (b == 0) v = (7.0 * dd[0] + dd[1]) / 8.0;
+        if (b == 0) v = (7.0 * dd[0] + dd[1]) / 8.0;
         else if (b == nb - 1) v = (dd[nb - 2] + 7.0 * dd[nb - 1]) / 8.0;
         else v = (dd[b - 1] + 6.0 * dd[b] + dd[b + 1]) / 8.0;
-        sm[k] = v;
+        sm[b] = v;
+        tot += v;
     }
-    __syncthreads();
-    const bool f32 = g.precision == BEST_FP32;
-    if (threadIdx.x < D) {
-        double t = 0.0;
-        for (int b = 0; b < nb; ++b) t += sm[threadIdx.x * nb + b];
-        tot[threadIdx.x] = t;
-        // FP32 path: the totals are sums of FP32 training data, so their
-        // reciprocals are finite (an FP64 total can be subnormal)
-        tot[D + threadIdx.x] = f32 && t > 0.0 ? 1.0 / t : 0.0;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < D * nb; k += blockDim.x) {
-        const int d = k / nb;
-        const double t = tot[d];
-        double o = 0.0, r = 0.0;
-        if (t > 0.0) {
+    tot = warp_sum(tot);
+    const bool refined = tot > 0.0;            // else no training data: the map is kept
+    if (refined) {
+        // FP32 path: the total is a sum of FP32 training data, so its
+        // reciprocal is finite (an FP64 total can be subnormal)
+        const double inv = f32 ? 1.0 / tot : 0.0;
+        for (int b = lane; b < nb; b += 32) {
+            double o, r;
             if (f32) {
                 // the FP32 path's training data carry FP32 rounding: its
-                // normalisation, compression and reciprocal are evaluated in
-                // FP32 (FP64 division, log and pow run at a small fraction of
-                // the FP32 rate on this GPU)
-                const float vf = static_cast<float>(sm[k] * tot[D + d]);
+                // compression and reciprocal are evaluated in FP32 (FP64
+                // division, log and pow run at a small fraction of the FP32
+                // rate on this GPU)
+                const float vf = static_cast<float>(sm[b] * inv);
                 float of = 1.0f;               // v >= 1, or not a number (FP32 training data overflowed)
                 if (vf < 1e-30f) of = 0.0f;    // numerically empty increment
                 else if (vf < 1.0f) of = powf((1.0f - vf) / -logf(vf), static_cast<float>(td.alpha));
                 o = of;
                 r = of > 0.0f ? __frcp_rn(of) : 0.0f;
             } else {
-                const double v = sm[k] / t;
+                const double v = sm[b] / tot;
                 if (v < 1e-30) o = 0.0;        // numerically empty increment
                 else if (v >= 1.0) o = 1.0;
-                else o = pow((1.0 - v) / -log(v), td.alpha);
+                else {
+                    const double x = (1.0 - v) / -log(v);
+                    o = td.alpha == 0.5 ? sqrt(x) : pow(x, td.alpha);
+                }
                 // the interpolation below multiplies by these reciprocals (o is
                 // 0 or at least (1 / ln 1e30)^alpha)
                 r = o > 0.0 ? 1.0 / o : 0.0;
             }
+            sm[b] = o;
+            rom[b] = r;
         }
-        sm[k] = o;
-        rom[k] = r;
+        __syncwarp();
+        // running sums: every lane its own increments, then a scan of the lanes
+        const int per = (nb + 31) / 32, b0 = min(lane * per, nb), b1 = min(b0 + per, nb);
+        double mine = 0.0;
+        for (int b = b0; b < b1; ++b) mine += sm[b];
+        double run = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double x = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += x;
+        }
+        run = __shfl_up_sync(0xffffffffu, run, 1);
+        if (lane == 0) {
+            run = 0.0;
+            cum[0] = 0.0;
+        }
+        for (int b = b0; b < b1; ++b) {
+            run += sm[b];
+            cum[b + 1] = run;
+        }
+        __syncwarp();
     }
-    __syncthreads();
-    if (threadIdx.x < D) {
-        const int d = threadIdx.x;
-        const double* om = sm + d * nb;
-        double* c = cum + d * (nb + 1);
-        double acc = 0.0;
-        c[0] = 0.0;
-        for (int b = 0; b < nb; ++b) {
-            acc += om[b];
-            c[b + 1] = acc;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (s_underflow) return;
+    // new edge k: starting from increment 0, step to the next increment while
+    // the running sum after it stays below the goal k T / nb (and an increment
+    // is left): the number of j in [1, nb - 1] with cum[j] < goal, and the
+    // linear interpolation inside it.  The sums and goals are not negative, so
+    // they compare as integers.
+    double* e = e_task + warp * (nb + 1);
+    if (refined) {
+        const double target = cum[nb] / nb;
+        for (int k = lane; k < nb; k += 32) {
+            double v = 0.0;
+            if (k > 0) {
+                const double goal = k * target;
+                const long long gi = __double_as_longlong(goal);
+                int lo = 0, hi = nb - 1;                     // first i in [0, nb - 1] with !(cum[i + 1] < goal), else nb - 1
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (__double_as_longlong(cum[mid + 1]) < gi) lo = mid + 1;
+                    else hi = mid;
+                }
+                double fr = (goal - cum[lo]) * rom[lo];
+                fr = fr < 0.0 ? 0.0 : (fr > 1.0 ? 1.0 : fr);
+                v = olde[lo] + fr * (olde[lo + 1] - olde[lo]);
+            }
+            e[k] = v;
+            sm[k] = v;                                       // (the compressed weights are done with)
         }
-    }
-    __syncthreads();
-    // new edge k of dimension d: starting from increment 0, step to the next
-    // increment while the running sum after it stays below the goal k T / nb
-    // (and an increment is left); the running sums are non-decreasing, so the
-    // increment reached is the number of j in [1, nb - 1] with cum[j] < goal
-    double* e = edges + static_cast<int64_t>(t) * g.map_stride;
-    for (int q = threadIdx.x; q < D * (nb + 1); q += blockDim.x) {
-        const int d = q / (nb + 1), k = q - d * (nb + 1);
-        if (!(tot[d] > 0.0)) continue;                   // no training data: the map is kept
-        if (k == 0 || k == nb) {
-            e[q] = k == 0 ? 0.0 : 1.0;
-            continue;
-        }
-        const double* c = cum + d * (nb + 1);
-        const double target = c[nb] / nb;
-        const double goal = k * target;
-        int lo = 0, hi = nb - 1;                         // first i in [0, nb - 1] with !(c[i + 1] < goal), else nb - 1
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (c[mid + 1] < goal) lo = mid + 1;
-            else hi = mid;
-        }
-        const int i = lo;
-        double fr = (goal - c[i]) * rom[d * nb + i];
-        fr = fr < 0.0 ? 0.0 : (fr > 1.0 ? 1.0 : fr);
-        const double* oe = olde + d * (nb + 1);
-        e[q] = oe[i] + fr * (oe[i + 1] - oe[i]);
+        if (lane == 0) e[nb] = 1.0;
+    } else {
+        for (int k = lane; k < nb; k += 32) sm[k] = olde[k];
     }
     if (map32) {
         // the FP32 kernels' table of the refined map
-        __syncthreads();
-        float2* m = map32 + static_cast<int64_t>(t) * map32_stride(g);
-        for (int k = threadIdx.x; k < D * nb; k += blockDim.x) m[k] = map32_entry(e, k / nb, k % nb, nb, g);
+        __syncwarp();
+        const double end = refined ? 1.0 : olde[nb];
+        float2* m = map32 + static_cast<int64_t>(t) * map32_stride(g) + (3 * leg + warp) * nb;
+        for (int k = lane; k < nb; k += 32) m[k] = map32_value(sm[k], k + 1 < nb ? sm[k + 1] : end, warp, g);
     }
 }
 
@@ -888,8 +923,10 @@ __global__ void map32_kernel(Geometry g, const TaskDesc* __restrict__ tasks, int
 // Combination of the iterations per task (inverse-variance weights; zero-
 // variance iterations are exact) and assembly of Eq. (7):
 // C_a(p_i) = sum_sides mult (I_gain - I_loss), err^2 = sum mult^2
-// (sigma_gain^2 + sigma_loss^2).  One thread per (species, grid point), each
-// owning the tasks observed there; thread 0 advances the evaluation counter.
+// (sigma_gain^2 + sigma_loss^2).  Two lanes per (species, grid point), one for
+// its gain and one for its loss tasks, 32 threads per CTA (the combination is
+// a chain of FP64 divisions: spread over the SMs, 4.5 -> 3.6 us for 32 points);
+// thread 0 advances the evaluation counter.
 // ---------------------------------------------------------------------------
 __device__ inline void combine_task(TaskAcc& A) {
     if (A.n_exact > 0.0) {
@@ -906,32 +943,39 @@ __device__ inline void combine_task(TaskAcc& A) {
 
 __global__ void assemble_kernel(Geometry g, const SideDesc* __restrict__ sides, TaskAcc* acc,
                                 TimeState* ts, double* C, double* err, double* prev) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = id >> 1, term = id & 1;
     const int n = g.n_grid;
-    if (k < g.n_species * n) {
-        const int s = k / n;
-        const int i = k - s * n;
-        double c = 0.0, v = 0.0;
-        const int nl = g.pt_hi - g.pt_lo;         // points of this context (a shard) in task order
-        const bool mine = i >= g.pt_lo && i < g.pt_hi;
-        for (int si = 0; si < (mine ? g.n_side : 0); ++si) {
-            const SideDesc& sd = sides[si];
-            if (sd.species_obs != s) continue;
-            const int tg = (si * nl + i - g.pt_lo) * 2;
-            TaskAcc& G = acc[tg];
-            TaskAcc& L = acc[tg + 1];
-            combine_task(G);
-            combine_task(L);
-            if (G.mean != 0.0) prev[tg] = fabs(G.mean);
-            if (L.mean != 0.0) prev[tg + 1] = fabs(L.mean);
-            c += sd.mult * (G.mean - L.mean);
-            v += static_cast<double>(sd.mult) * sd.mult * (G.err * G.err + L.err * L.err);
+    const bool in = k < g.n_species * n;
+    double c = 0.0, v = 0.0;
+    const int s = in ? k / n : 0;
+    const int i = in ? k - s * n : 0;
+    const int nl = g.pt_hi - g.pt_lo;         // points of this context (a shard) in task order
+    const bool mine = in && i >= g.pt_lo && i < g.pt_hi;
+    for (int si = 0; si < g.n_side; ++si) {
+        const bool here = mine && sides[si].species_obs == s;
+        double mean = 0.0, e2 = 0.0;
+        if (here) {
+            const int t = (si * nl + i - g.pt_lo) * 2 + term;
+            TaskAcc& A = acc[t];
+            combine_task(A);
+            if (A.mean != 0.0) prev[t] = fabs(A.mean);
+            mean = A.mean;
+            e2 = A.err * A.err;
         }
+        const double mean1 = __shfl_xor_sync(0xffffffffu, mean, 1), e1 = __shfl_xor_sync(0xffffffffu, e2, 1);
+        if (here) {
+            const double mult = sides[si].mult;
+            c += mult * (mean - mean1);       // (the gain lane's)
+            v += mult * mult * (e2 + e1);
+        }
+    }
+    if (in && term == 0) {
         if (!isfinite(c) || !isfinite(v)) ts->error = BEST_ERR_NUMERIC;
         C[k] = c;
         if (err) err[k] = sqrt(v);
     }
-    if (k == 0) ts->call += 1u;
+    if (id == 0) ts->call += 1u;
 }
 
 // ---------------------------------------------------------------------------
@@ -1023,20 +1067,23 @@ __global__ void width_control_kernel(Geometry g, const SideDesc* __restrict__ si
 // points.  max |C/f| is reduced in FP64 and the step used is
 // dt = min(dt_requested, eps / max |C/f|) (Eq. (16)).
 // ---------------------------------------------------------------------------
+// Maximum of v >= 0 (not NaN) over the CTA: non-negative doubles order like
+// their bits, so the reduction runs on integers (two redux operations per
+// warp; an FP64 comparison takes the FP64 pipe for 64 cycles).
+__device__ double warp_max_bits(double v) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(v)), lo = static_cast<uint32_t>(__double2loint(v));
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return __hiloint2double(static_cast<int>(mh), static_cast<int>(ml));
+}
 __device__ double block_max(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = warp_max_bits(v);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0) red[w] = v;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (threadIdx.x == 0) red[0] = v;
-    }
+    v = warp_max_bits(l < static_cast<int>(blockDim.x >> 5) ? red[l] : 0.0);
     __syncthreads();
-    const double r = red[0];
-    __syncthreads();
-    return r;
+    return v;
 }
 
 // Euler (Eq. (14)) or the Heun predictor: dt from k1, logf_out = logf + dt k1/f.
@@ -1049,12 +1096,17 @@ __global__ void step_first_kernel(Geometry g, double* logf, const double* __rest
     __shared__ double red[32];
     const int total = g.n_species * g.n_grid;
     double mx = 0.0;
-    for (int k = threadIdx.x; k < total; k += blockDim.x) mx = fmax(mx, fabs(k1[k] / fgrid[k]));
+    double rate = 0.0;                       // C/f of this thread's first point
+    for (int k = threadIdx.x; k < total; k += blockDim.x) {
+        const double q = k1[k] / fgrid[k];
+        if (k == static_cast<int>(threadIdx.x)) rate = q;
+        mx = fmax(mx, fabs(q));
+    }
     mx = block_max(mx, red);
     double dt = *dt_src;
     if (mx > 0.0) dt = fmin(dt, g.eps_dt / mx);
     for (int k = threadIdx.x; k < total; k += blockDim.x) {
-        const double step = dt * k1[k] / fgrid[k];
+        const double step = dt * (k == static_cast<int>(threadIdx.x) ? rate : k1[k] / fgrid[k]);
         if (heun) fstar[k] = exp(logf[k] + step);
         else logf[k] += step;
     }
