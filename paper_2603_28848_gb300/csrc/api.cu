@@ -452,6 +452,7 @@ best_status build_plan(best_ctx* ctx, int it, IterPlan& plan) {
             if (g1 <= g0) continue;
             Segment s{};
             s.task = active[a];
+            s.shape = segment_shape(ctx->tasks[active[a]].dim / 3 + 2, ctx->tasks[active[a]].nbins);
             s.g0 = g0 * unit[a];
             s.g1 = g1 * unit[a];
             segs.push_back(s);

@@ -168,6 +168,7 @@ __global__ void plan_kernel(const TaskDesc* __restrict__ tasks, int n_plans, con
                     if (pass) {
                         Segment sg{};
                         sg.task = pl.active[a];
+                        sg.shape = segment_shape(td.dim / 3 + 2, td.nbins);
                         sg.g0 = g0 * unit;
                         sg.g1 = g1 * unit;
                         sg.part = off;

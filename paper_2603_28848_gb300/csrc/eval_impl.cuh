@@ -566,9 +566,7 @@ namespace best {
 // matrix elements (kept apart so that the plain kernel's register allocation
 // is not affected).
 template <typename R, int NLEG, bool STRAT, int SPL>
-__device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& seg,
-                                            const SideDesc& sd, const TaskDesc& td,
-                                            const TaskConst& tc, R* s_spline,
+__device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& seg, R* s_spline,
                                             Real2<R>* s_map, R* s_hist, double* s_red, float* s_queue,
                                             int map_elems) {
     constexpr int NI = NLEG - 2;
@@ -578,8 +576,11 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     using SS = StreamShape<D, F32>;
     constexpr int G = SS::kGroup;
     const Geometry& g = P.geo;
-    const int nb = td.nbins;
+    const int nb = seg.shape >> 8;
     const int tid = threadIdx.x;
+    // (nothing of the FP32 set-up waits for the descriptors)
+    const TaskDesc& td = P.tasks[seg.task];
+    const TaskConst& tc = P.tconst[seg.task];
 
     // ---- map table of this task in shared memory ---------------------------
     if constexpr (F32) {
@@ -620,8 +621,8 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
     // address, and the warps are summed in a fixed order at the end, so the
     // training data do not depend on warp scheduling
     const int nwarps = blockDim.x >> 5;
-    for (int k = tid; k < nwarps * map_elems; k += blockDim.x) s_hist[k] = R(0);
     R* w_hist = s_hist + (tid >> 5) * map_elems;
+    for (int k = tid & 31; k < D * nb; k += 32) w_hist[k] = R(0);
 
     Acc<R> acc_w, acc_w2;
     if constexpr (SCREEN) {
@@ -630,13 +631,13 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
         SegSetup<double, NLEG>* s_setup = reinterpret_cast<SegSetup<double, NLEG>*>(tab + kMathDoubles);
         static_assert(sizeof(SegSetup<double, NLEG>) <= kSetupBytes, "room for the segment constants");
         Real2<float>* s_map32 = reinterpret_cast<Real2<float>*>(reinterpret_cast<unsigned char*>(s_setup) + kSetupBytes);
-        run_samples64<NLEG>(P, seg, sd, td, tc, s_spline, s_map, s_map32, w_hist, tab, s_setup,
+        run_samples64<NLEG>(P, seg, P.sides[td.si], td, tc, s_spline, s_map, s_map32, w_hist, tab, s_setup,
                             reinterpret_cast<uint32_t*>(s_map32 + map_elems), acc_w, acc_w2);
     } else {
     // ---- per-segment constants ----------------------------------------------
     SegSetup<R, NLEG> setup;
     if constexpr (F32) seg_setup32<NLEG>(P.tconst32[seg.task], &setup);
-    else seg_setup<R, NLEG>(P, sd, td, tc, &setup);
+    else seg_setup<R, NLEG>(P, P.sides[td.si], td, tc, &setup);
     const R nbR = static_cast<R>(nb);
     const int ncoef = 4 * (g.n_grid - 1);
     const R* knots = s_spline + g.n_species * ncoef;
@@ -1124,34 +1125,35 @@ eval_kernel(EvalParams P) {
         const R* gk = static_cast<const R*>(P.knots);
         for (int k = threadIdx.x; k < P.geo.n_grid; k += blockDim.x) s_spline[ncoef + k] = gk[k];
     }
-    // chunks of the partition: taken from the counter (dynamic), or chunk b
-    // by CTA b; every segment writes its own partial record, so the results
-    // do not depend on which CTA ran it
+    // chunks of the partition: chunk b first, then those the counter hands out
+    // (dynamic), or chunk b alone; every segment writes its own partial record,
+    // so the results do not depend on which CTA ran it.  The chunks past the
+    // last one with work are empty and start at the end of the segments: a CTA
+    // that meets one is done (a small iteration has up to 15 of 16 of them;
+    // taking them one by one from the counter was a fifth of its kernel's time).
+    // The next chunk is asked for when this one is done: reserved at its start,
+    // a CTA with a long chunk held back another (2 -> 4 sweep 4% slower).
     __shared__ int s_chunk;
-    for (int c = P.chunk_counter ? -1 : static_cast<int>(blockIdx.x);;) {
-        if (P.chunk_counter) {
-            __syncthreads();
-            if (threadIdx.x == 0) s_chunk = atomicAdd(P.chunk_counter, 1);
-            __syncthreads();
-            c = s_chunk;
-        }
-        if (c >= P.n_chunks) break;
+    const int seg_end = P.cta_seg[P.n_chunks];
+    for (int c = static_cast<int>(blockIdx.x); c < P.n_chunks;) {
         const int s0 = P.cta_seg[c], s1 = P.cta_seg[c + 1];
+        if (s0 >= seg_end) break;
         for (int si = s0; si < s1; ++si) {
             const Segment seg = P.segs[si];
-            const TaskDesc td = P.tasks[seg.task];
-            const SideDesc& sd = P.sides[td.si];
-            const TaskConst tc = P.tconst[seg.task];
             __syncthreads();
-            switch (sd.n) {
-                case 3: if constexpr (NMAX >= 3) run_segment<R, 3, STRAT, SPL>(P, seg, sd, td, tc, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
-                case 4: if constexpr (NMAX >= 4) run_segment<R, 4, STRAT, SPL>(P, seg, sd, td, tc, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
-                case 5: if constexpr (NMAX >= 5) run_segment<R, 5, STRAT, SPL>(P, seg, sd, td, tc, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
-                case 6: if constexpr (NMAX >= 6) run_segment<R, 6, STRAT, SPL>(P, seg, sd, td, tc, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
+            switch (seg.shape & 0xff) {
+                case 3: if constexpr (NMAX >= 3) run_segment<R, 3, STRAT, SPL>(P, seg, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
+                case 4: if constexpr (NMAX >= 4) run_segment<R, 4, STRAT, SPL>(P, seg, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
+                case 5: if constexpr (NMAX >= 5) run_segment<R, 5, STRAT, SPL>(P, seg, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
+                case 6: if constexpr (NMAX >= 6) run_segment<R, 6, STRAT, SPL>(P, seg, s_spline, s_map, s_hist, s_red, s_queue, map_elems); break;
                 default: break;
             }
         }
         if (!P.chunk_counter) break;
+        if (threadIdx.x == 0) s_chunk = atomicAdd(P.chunk_counter, 1) + static_cast<int>(gridDim.x);
+        __syncthreads();
+        c = s_chunk;
+        __syncthreads();
     }
 }
 

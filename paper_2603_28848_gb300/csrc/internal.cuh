@@ -161,10 +161,13 @@ struct TaskAcc {
 // A contiguous piece of one task's samples handled by one CTA.
 struct Segment {
     int32_t task;
-    int32_t pad_;
+    int32_t shape;          // segment_shape() of the task: known without another dependent load
     int64_t g0, g1;         // sample groups [g0, g1) of the task
     int64_t part;           // offset (in doubles) of this segment's partial record
 };
+
+// Legs and map increments of a segment's task.
+__host__ __device__ inline int32_t segment_shape(int n, int nbins) { return n | nbins << 8; }
 
 // Time-dependent scalars of the current sweep, resident on the device so
 // that whole steps can be captured in a CUDA graph.

@@ -126,6 +126,7 @@ __global__ void noalloc_setup_kernel(SetupArgs A, unsigned char* base) {
     for (int b = tid; b < A.ctas; b += blockDim.x) {
         Segment s{};
         s.task = 0;
+        s.shape = segment_shape(A.sd.n, A.td.nbins);
         s.g0 = A.groups * b / A.ctas;
         s.g1 = A.groups * (b + 1) / A.ctas;
         s.part = static_cast<int64_t>(b) * kRecord;

@@ -684,15 +684,10 @@ __global__ void __launch_bounds__(kThreads, 2) vjp_kernel(VjpParams V) {
     }
     // chunks of the partition, as in the sample kernel
     __shared__ int s_chunk;
-    for (int c = P.chunk_counter ? -1 : static_cast<int>(blockIdx.x);;) {
-        if (P.chunk_counter) {
-            __syncthreads();
-            if (threadIdx.x == 0) s_chunk = atomicAdd(P.chunk_counter, 1);
-            __syncthreads();
-            c = s_chunk;
-        }
-        if (c >= P.n_chunks) break;
+    const int seg_end = P.cta_seg[P.n_chunks];
+    for (int c = static_cast<int>(blockIdx.x); c < P.n_chunks;) {
         const int s0 = P.cta_seg[c], s1 = P.cta_seg[c + 1];
+        if (s0 >= seg_end) break;
         for (int si = s0; si < s1; ++si) {
             const Segment seg = P.segs[si];
             const TaskDesc td = P.tasks[seg.task];
@@ -708,6 +703,10 @@ __global__ void __launch_bounds__(kThreads, 2) vjp_kernel(VjpParams V) {
             }
         }
         if (!P.chunk_counter) break;
+        if (threadIdx.x == 0) s_chunk = atomicAdd(P.chunk_counter, 1) + static_cast<int>(gridDim.x);
+        __syncthreads();
+        c = s_chunk;
+        __syncthreads();
     }
     if constexpr (!JVP) {
         __syncthreads();
