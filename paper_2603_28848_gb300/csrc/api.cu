@@ -101,7 +101,8 @@ struct best_ctx {
     int precision = 0;
     int nmax_legs = 0;
     int grid = 0;                   // CTAs of the persistent sample kernel
-    int n_chunks = 0;               // chunks of the work partition (chunk_count(grid))
+    int plan_grid = 0;              // CTAs the work partition is cut for (grid, or the first variant's)
+    int n_chunks = 0;               // chunks of the work partition (chunk_count(plan_grid))
     int32_t* d_chunk_ctr = nullptr; // [max_nitn + 1] chunk counters: sample kernel per iteration, adjoint / tangent
     size_t eval_smem = 0;
     size_t spline_smem = 0;
@@ -181,6 +182,7 @@ struct best_ctx {
     // implicit Euler (best_step_implicit_euler): Krylov basis and work vectors
     double* d_nk = nullptr;
     int nk_m = 0;
+    double* h_nk = nullptr;         // pinned: the solver's scalars as read back (8 doubles)
     int n_processes = 0;
     size_t vjp_smem = 0;
     bool vjp_screen = false, jvp_screen = false;   // FP64 adjoint / tangent kernels with the FP32 screen
@@ -257,6 +259,8 @@ void free_all(best_ctx* c) {
     cudaFree(c->d_bctl); cudaFree(c->d_bv); cudaFree(c->d_plan_scratch); cudaFree(c->d_plandev);
     cudaFree(c->d_chunk_ctr);
     cudaFree(c->d_splplan); cudaFree(c->d_sideconst);
+    if (c->h_nk) cudaFreeHost(c->h_nk);
+    c->h_nk = nullptr;
 }
 
 best_status validate(const best_config* cfg) {
@@ -435,7 +439,7 @@ best_status build_plan(best_ctx* ctx, int it, IterPlan& plan) {
         cum[a + 1] = cum[a] + groups[a] * cost[a];
     }
     const int64_t W = cum[A];
-    const int B = ctx->grid, K = ctx->n_chunks;
+    const int B = ctx->plan_grid, K = ctx->n_chunks;
     const ChunkShape sh = chunk_shape(W, B);
     std::vector<Segment> segs;
     std::vector<int32_t> cta_seg(K + 1, 0);
@@ -502,8 +506,22 @@ best_status build_plan(best_ctx* ctx, int it, IterPlan& plan) {
     return BEST_OK;
 }
 
-// Selects sample-kernel variant v: raises its shared-memory limit, sizes the
-// persistent grid from its occupancy and rebuilds the work partition.
+// CTAs per SM of sample-kernel variant v, its shared-memory limit raised to
+// what the context needs.
+best_status variant_occupancy(best_ctx* ctx, int v, int* occ) {
+    const SampleVariant& sv = ctx->variants[v];
+    const size_t smem = sample_smem(ctx, sv);
+    cudaFuncAttributes fa{};
+    CK(cudaFuncGetAttributes(&fa, sv.fn));
+    if (static_cast<size_t>(fa.maxDynamicSharedSizeBytes) < smem)
+        CK(cudaFuncSetAttribute(sv.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, sv.fn, sv.threads, smem));
+    if (*occ < 1) return fail(ctx, BEST_ERR_INVALID, "sample kernel does not fit on an SM");
+    return BEST_OK;
+}
+
+// Selects sample-kernel variant v: sizes the persistent grid from its
+// occupancy and rebuilds the work partition.
 best_status set_variant(best_ctx* ctx, int v) {
     int dev = 0, nsm = 0;
     CK(cudaGetDevice(&dev));
@@ -511,13 +529,11 @@ best_status set_variant(best_ctx* ctx, int v) {
     void* fn = ctx->variants[v].fn;
     const int threads = ctx->variants[v].threads;
     ctx->eval_smem = sample_smem(ctx, ctx->variants[v]);
-    cudaFuncAttributes fa{};
-    CK(cudaFuncGetAttributes(&fa, fn));
-    if (static_cast<size_t>(fa.maxDynamicSharedSizeBytes) < ctx->eval_smem)
-        CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ctx->eval_smem)));
     int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, ctx->eval_smem));
-    if (occ < 1) return fail(ctx, BEST_ERR_INVALID, "sample kernel does not fit on an SM");
+    best_status so = variant_occupancy(ctx, v, &occ);
+    if (so != BEST_OK) return so;
+    int plan_occ = occ;
+    if (ctx->variants[v].first_plan && (so = variant_occupancy(ctx, 0, &plan_occ)) != BEST_OK) return so;
     // a captured step graph refers to the old partition: drop it
     if (ctx->graph) {
         CK(cudaGraphExecDestroy(ctx->graph));
@@ -527,7 +543,8 @@ best_status set_variant(best_ctx* ctx, int v) {
     ctx->variant = v;
     ctx->eval_threads = threads;
     ctx->grid = nsm * occ;
-    ctx->n_chunks = chunk_count(ctx->grid);
+    ctx->plan_grid = nsm * plan_occ;
+    ctx->n_chunks = chunk_count(ctx->plan_grid);
     for (auto& pl : ctx->plans) {
         cudaFree(pl.d_active); cudaFree(pl.d_task_seg); cudaFree(pl.d_segs); cudaFree(pl.d_cta_seg);
     }
@@ -651,7 +668,7 @@ best_status enqueue_sweep(best_ctx* ctx, const SweepStart& ss, const double* src
         // next sweep's budgets from this sweep's estimates, then its partition
         budget_kernel<<<static_cast<int>(ctx->bctl.size()), 1024, 0, st>>>(ctx->d_bctl, ctx->d_acc, ctx->d_tasks,
                                                                           ctx->d_bv);
-        plan_kernel<<<1, 1024, 0, st>>>(ctx->d_tasks, ctx->max_nitn, ctx->d_plandev, ctx->grid, f32 ? 1 : 0,
+        plan_kernel<<<1, 1024, 0, st>>>(ctx->d_tasks, ctx->max_nitn, ctx->d_plandev, ctx->plan_grid, f32 ? 1 : 0,
                                         ctx->d_plan_scratch);
         ctx->launches += 2;
     }
@@ -1087,7 +1104,19 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
         CKI(dalloc(&ctx->d_bv, static_cast<size_t>(T)));
     }
     {
-        best_status sv = set_variant(ctx, 0);
+        // Two packed samples per lane (four CTAs per SM) pay once the CTAs run several chunks each;
+        // with about one chunk per CTA five CTAs per SM finish sooner.  Sample kernel, one -> packed:
+        // MB 2 -> 2 at 1, 2, 10 chunks per CTA 88 -> 84, 153 -> 157, 645 -> 625 us; BE 2 -> 2 at 1, 2.5,
+        // 4, 41 chunks 113 -> 113, 207 -> 198, 319 -> 307, 2957 -> 2779 us.
+        int pick = 0, occ = 0;
+        for (int v = 1; v < ctx->n_variants; ++v)
+            if (ctx->variants[v].first_plan) pick = v;
+        best_status sv = pick ? variant_occupancy(ctx, 0, &occ) : BEST_OK;
+        if (sv != BEST_OK) return bail(sv);
+        int64_t W = 0;
+        for (const TaskDesc& td : ctx->tasks) W += td.neval * (td.dim + 6);
+        if (pick && W / kMinChunkCost < 4 * static_cast<int64_t>(nsm) * occ) pick = 0;
+        sv = set_variant(ctx, pick);
         if (sv != BEST_OK) return bail(sv);
     }
     CKI(cudaDeviceSynchronize());
@@ -1487,13 +1516,15 @@ static best_status nk_buffers(best_ctx* ctx, int m) {
     ctx->nk_m = 0;
     const size_t total = static_cast<size_t>(N) * (m + 1 + 10) + static_cast<size_t>(m + 1) * m + 3 * m + 2 + 8;
     CK(cudaMalloc(&ctx->d_nk, total * sizeof(double)));
+    if (!ctx->h_nk) CK(cudaMallocHost(&ctx->h_nk, 8 * sizeof(double)));
     ctx->nk_m = m;
     return BEST_OK;
 }
 
 static best_status read_stat(best_ctx* ctx, const double* d_stat, double* h_stat, cudaStream_t st) {
-    CK(cudaMemcpyAsync(h_stat, d_stat, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(ctx->h_nk, d_stat, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    std::memcpy(h_stat, ctx->h_nk, 8 * sizeof(double));
     return BEST_OK;
 }
 
@@ -1533,6 +1564,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
     double* stat = gvec + mm + 2;
     double hs[8] = {};
     const int eb = (N + 255) / 256;
+    const int nt = std::min(1024, (N + 31) / 32 * 32);     // threads of the one-CTA Krylov kernels
     const double t1 = t + dt;
 
     if (train) {
@@ -1546,7 +1578,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
     ctx->launches += 1;
     s = enqueue_jvp(ctx, f, t1, u, C, JU, st, true);
     if (s != BEST_OK) return s;
-    nk_residual_kernel<<<1, 1024, 0, st>>>(N, ga, gn, C, f, dt, r, Qd, stat);
+    nk_residual_kernel<<<1, nt, 0, st>>>(N, ga, gn, C, f, dt, r, Qd, stat);
     ctx->launches += 1;
     s = read_stat(ctx, stat, hs, st);
     if (s != BEST_OK) return s;
@@ -1554,7 +1586,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
     double rn2 = hs[0], rinf = hs[1];
     int newton = 0, krylov = 0, halvings = 0;
     while (rinf > tol && newton < max_newton) {
-        gmres_start_kernel<<<1, 1024, 0, st>>>(N, mm, r, V, gvec);
+        gmres_start_kernel<<<1, nt, 0, st>>>(N, mm, r, V, gvec);
         ctx->launches += 1;
         int k = 0;
         for (int j = 0; j < m; ++j) {
@@ -1562,7 +1594,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
             ctx->launches += 1;
             s = enqueue_jvp(ctx, f, t1, u, C, JU, st, false);
             if (s != BEST_OK) return s;
-            gmres_arnoldi_kernel<<<1, 1024, 0, st>>>(N, mm, j, dt, f, Qd, JU, V, H, cs, sn, gvec, stat);
+            gmres_arnoldi_kernel<<<1, nt, 0, st>>>(N, mm, j, dt, f, Qd, JU, V, H, cs, sn, gvec, stat);
             ctx->launches += 1;
             ++krylov;
             s = read_stat(ctx, stat, hs, st);
@@ -1570,7 +1602,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
             k = j + 1;
             if (hs[2] <= krylov_rtol * rn2 || !(hs[3] > 1e-300 * rn2)) break;
         }
-        gmres_update_kernel<<<1, 1024, 0, st>>>(N, mm, k, V, H, gvec, d);
+        gmres_update_kernel<<<1, nt, 0, st>>>(N, mm, k, V, H, gvec, d);
         ctx->launches += 1;
         // backtracking on ||R||_2 (Armijo with slope -||R||^2 of the exact Newton direction)
         double lambda = 1.0;
@@ -1581,7 +1613,7 @@ best_status best_step_implicit_euler(best_ctx* ctx, double* logf_dev, double t, 
             ctx->launches += 2;
             s = enqueue_jvp(ctx, f, t1, u, C, JU, st, true);
             if (s != BEST_OK) return s;
-            nk_residual_kernel<<<1, 1024, 0, st>>>(N, gt, gn, C, f, dt, r, Qd, stat);
+            nk_residual_kernel<<<1, nt, 0, st>>>(N, gt, gn, C, f, dt, r, Qd, stat);
             ctx->launches += 1;
             s = read_stat(ctx, stat, hs, st);
             if (s != BEST_OK) return s;
@@ -1689,7 +1721,7 @@ best_status best_load_state(best_ctx* ctx, const void* host_buf, int64_t size) {
         CK(cudaMemcpy(cur.data(), ctx->d_tasks, cur.size() * sizeof(TaskDesc), cudaMemcpyDeviceToHost));
         for (size_t t = 0; t < cur.size(); ++t) std::memcpy(&cur[t].neval, p + 8 * t, 8);
         CK(cudaMemcpy(ctx->d_tasks, cur.data(), cur.size() * sizeof(TaskDesc), cudaMemcpyHostToDevice));
-        plan_kernel<<<1, 1024>>>(ctx->d_tasks, ctx->max_nitn, ctx->d_plandev, ctx->grid,
+        plan_kernel<<<1, 1024>>>(ctx->d_tasks, ctx->max_nitn, ctx->d_plandev, ctx->plan_grid,
                                  ctx->precision == BEST_FP32 ? 1 : 0, ctx->d_plan_scratch);
         CK(cudaGetLastError());
         CK(cudaDeviceSynchronize());

@@ -343,19 +343,22 @@ __device__ __forceinline__ float2 kin_pair(const SegConst<float, NLEG>& C, const
     const float2 rpc = make_float2(pc2.x > 1e-30f ? rsqrt_ftz(pc2.x) : 0.0f, pc2.y > 1e-30f ? rsqrt_ftz(pc2.y) : 0.0f);
     qc = mul2(mul2(pc2, rpc), bc2(C.a));
     float2 gauss;
+    // up to four legs the products are taken in kin_at's order, so that both
+    // loops give the same bits (the default of a 2 -> 2 problem depends on its size)
+    constexpr bool kSame = NLEG <= 4;
     if (C.frac) {
         // sigma = w S / 2 with S = E_in + E_out: exponent -2 dE^2 / (w S)^2,
         // normalisation sigma_ref / sigma = 2 E_obs / S
         Esum = add2(Esum, Ec);
         const float2 iS = make_float2(__fdividef(1.0f, Esum.x), __fdividef(1.0f, Esum.y));
         const float2 x = mul2(dE, iS);
-        const float2 e = mul2(mul2(x, x), bc2(C.gauss_k));
+        const float2 e = kSame ? mul2(mul2(bc2(C.gauss_k), x), x) : mul2(mul2(x, x), bc2(C.gauss_k));
         gauss = mul2(make_float2(ex2_ftz(e.x), ex2_ftz(e.y)), mul2(bc2(2.0f * C.e_obs), iS));
     } else {
-        const float2 e = mul2(mul2(dE, dE), bc2(C.gauss_k));
+        const float2 e = kSame ? mul2(mul2(bc2(C.gauss_k), dE), dE) : mul2(mul2(dE, dE), bc2(C.gauss_k));
         gauss = make_float2(ex2_ftz(e.x), ex2_ftz(e.y));
     }
-    float2 w = mul2(mul2(meas, rinv), mul2(rEc, gauss));
+    float2 w = kSame ? mul2(mul2(mul2(meas, rinv), rEc), gauss) : mul2(mul2(meas, rinv), mul2(rEc, gauss));
     w.x = emin0 < C.e_cut ? 0.0f : w.x;
     w.y = emin1 < C.e_cut ? 0.0f : w.y;
     return w;

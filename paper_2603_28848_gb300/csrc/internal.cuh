@@ -530,6 +530,7 @@ struct SampleVariant {
     int32_t mb;             // CTAs per SM of its register budget (__launch_bounds__)
     int32_t threads;        // threads per CTA
     int32_t spl;            // samples a lane evaluates per step of the FP32 loop
+    int32_t first_plan;     // 1: it runs over the work partition of the first variant's grid (same sums in the same order)
 };
 constexpr int kMaxVariants = 12;
 

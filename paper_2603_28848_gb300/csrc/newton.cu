@@ -14,28 +14,32 @@ namespace best {
 
 namespace {
 
+// Sum and maximum over the CTA, the same value in every thread: warp trees and
+// a tree over the warps' values.  The CTA has no more warps than the vector
+// needs: an FP64 operation takes an SM partition's pipe for 64 cycles per warp,
+// and with 32 warps (each adding up 32 values one by one) a sum took 8 us.
 __device__ double nk_block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (nw == 1) return v;
     __syncthreads();
     if (lane == 0) red[w] = v;
     __syncthreads();
-    double s = 0.0;
-    const int nw = (blockDim.x + 31) >> 5;
-    for (int k = 0; k < nw; ++k) s += red[k];      // same order in every thread
-    return s;
+    v = lane < nw ? red[lane] : 0.0;
+    for (int o = 1; o < nw; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return __shfl_sync(0xffffffffu, v, 0);
 }
 
 __device__ double nk_block_max(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (nw == 1) return v;
     __syncthreads();
     if (lane == 0) red[w] = v;
     __syncthreads();
-    double s = 0.0;
-    const int nw = (blockDim.x + 31) >> 5;
-    for (int k = 0; k < nw; ++k) s = fmax(s, red[k]);
-    return s;
+    v = lane < nw ? red[lane] : 0.0;
+    for (int o = 1; o < nw; o <<= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return __shfl_sync(0xffffffffu, v, 0);
 }
 
 }  // namespace
