@@ -59,23 +59,26 @@ __device__ __forceinline__ double rsqrt_halley(double x) {
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-// sin and cos of |x| <= pi: the nearest a_k = k pi / 64 of the table, the
-// Taylor polynomials of r = |x| - a_k (|r| <= pi / 128, the difference is
+// sin and cos of |x| <= pi: the nearest a_k = k pi / 128 of the table, the
+// Taylor polynomials of r = |x| - a_k (|r| <= pi / 256, the difference is
 // exact) and the addition theorem (table-driven reduction after Gal and Tang).
+// The polynomials' tails, 1/120 - r^2/5040 and 1/24 - r^2/720, are FP32 numbers:
+// their rounding enters with r^4 < 2.3e-8, below 2^-53 of the results.
 __device__ __forceinline__ void sincos_table(double x, const double* tab, double* s, double* c) {
     const uint32_t sign = static_cast<uint32_t>(__double2hiint(x)) & 0x80000000u;
     const double ax = flip_sign(x, sign);
-    // a subnormal or zero |x| truncates to a huge or zero float: k is clamped
-    // either way (k = 0 for |x| < 2^-126 through the comparison below)
+    // (below 2^-126: k = 0)
     const uint32_t hx = static_cast<uint32_t>(__double2hiint(ax));
     const float xf = hx < 0x38100000u ? 0.0f : trunc_f32(ax);
-    const int k = min(__float2int_rn(xf * 20.371832715762603f), kTrigEntries - 1);      // 64 / pi
+    const int k = min(__float2int_rn(xf * 40.743665431525206f), kTrigEntries - 1);      // 128 / pi
     const double a = tab[3 * k], S = tab[3 * k + 1], C = tab[3 * k + 2];
     const double r = ax - a;
     const double r2 = r * r;
-    const double p = fma(r2, fma(r2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0);
-    const double sr = fma(r * r2, p, r);
-    const double cm = r2 * fma(r2, fma(r2, -1.0 / 720.0, 1.0 / 24.0), -0.5);
+    const float rf = static_cast<uint32_t>(__double2hiint(r2)) < 0x38100000u ? 0.0f : trunc_f32(r2);
+    const double p5 = widen_f32(fmaf(rf, -1.0f / 5040.0f, 1.0f / 120.0f));
+    const double p4 = widen_f32(fmaf(rf, -1.0f / 720.0f, 1.0f / 24.0f));
+    const double sr = fma(r * r2, fma(r2, p5, -1.0 / 6.0), r);
+    const double cm = r2 * fma(r2, p4, -0.5);
     *s = flip_sign(S + fma(C, sr, S * cm), sign);
     *c = C + fma(-S, sr, C * cm);
 }
@@ -101,6 +104,44 @@ __device__ __forceinline__ double exp2_table(double x, const double* tab) {
     return __hiloint2double(__double2hiint(v) + ((k >> 5) << 20), __double2loint(v));
 }
 
+// A product of doubles as a 64-bit significand m in [2^63, 2^64) and an
+// exponent, value m / 2^63 2^e: a multiplication is a 64 x 64 -> high 64-bit
+// integer product (about 16 issue slots instead of the 64 cycles an FP64
+// multiplication takes the pipe) and loses at most 2^-63.  A zero or subnormal
+// factor makes the product zero, an infinite one or a NaN makes it NaN.
+struct Product {
+    uint64_t m;
+    int e;
+    uint32_t sign;          // bit 31
+    bool zero, bad;
+    __device__ __forceinline__ explicit Product(double x) : m(1ull << 63), e(0), sign(0), zero(false), bad(false) { mul(x); }
+    __device__ __forceinline__ void mul(double x) {
+        const uint64_t b = static_cast<uint64_t>(__double_as_longlong(x));
+        const int ex = static_cast<int>((b >> 52) & 0x7FF);
+        sign ^= static_cast<uint32_t>(b >> 32);
+        zero |= ex == 0;
+        bad |= ex == 0x7FF;
+        const uint64_t h = __umul64hi(m, (b << 11) | (1ull << 63));
+        const int up = static_cast<int>(h >> 63);
+        m = h << (1 - up);
+        e += ex - 1023 + up;
+    }
+    __device__ __forceinline__ double value() const {
+        uint64_t t = m + 0x400;                     // rounded to 53 bits
+        int x = e;
+        if (t < m) {
+            t = 1ull << 63;
+            ++x;
+        }
+        const uint32_t sg = sign & 0x80000000u;
+        if (bad) return __longlong_as_double(0x7FF8000000000000ll);
+        if (zero || x < -1100) return 0.0;
+        if (x < -1022 || x > 1023) return flip_sign(scalbn(static_cast<double>(t >> 11), x - 52), sg);
+        return flip_sign(__longlong_as_double(static_cast<long long>((static_cast<uint64_t>(x + 1023) << 52) |
+                                                                     ((t >> 11) & 0x000FFFFFFFFFFFFFull))), sg);
+    }
+};
+
 // a < b for doubles neither of which is NaN, as integers (an FP64 comparison
 // takes the FP64 pipe): b > 0; a negative a compares less.
 __device__ __forceinline__ bool less_pos(double a, double b) {
@@ -122,9 +163,10 @@ __device__ __forceinline__ double spline64(const double* coef, const double* kno
 }
 
 // Weight of one sample in FP64 (kin_at and stat_at of eval_impl.cuh, the same
-// formulas) with the functions above; C lives in shared memory.
+// formulas) with the functions above; dy: the mapped increments' widths; C
+// lives in shared memory.
 template <int NLEG>
-__device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, const double* y, double jac,
+__device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, const double* y, const double* dy,
                                            const double* s_spline, const double* knots, const Geometry& g,
                                            const SegSetup<float, NLEG>& s32, double q0, double qN, int ncoef,
                                            const double* tab) {
@@ -132,7 +174,7 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
     double px = 0.0, py = 0.0, pz = C.pobs_sig;
     double bal = C.sgn_obs_E;
     double Esum = C.e_obs;
-    double meas = jac, rinv = 1.0, stat = C.c0;
+    Product w(C.c0);
     const bool scaled = C.inv_a != 1.0;
     bool cut = false;
 #pragma unroll
@@ -153,11 +195,18 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
         cut |= less_pos(E, C.e_cut);
         bal += flip_sign(E, static_cast<uint32_t>(__double2hiint(C.sgnE[j])) & 0x80000000u);
         if (C.frac) Esum += E;
-        meas *= r * r * st;
-        rinv *= rE;
-        double f = spline64(s_spline + C.spc[j] * ncoef, knots, r, g, s32.inv_step, s32.q0, s32.lq0_step);
-        if (C.fd[j]) f = f < 1.0 ? f : 1.0;
-        stat *= fma(C.cb[j], f, C.ca[j]);
+        w.mul(dy[3 * j]);
+        w.mul(dy[3 * j + 1]);
+        w.mul(dy[3 * j + 2]);
+        w.mul(r);
+        w.mul(r);
+        w.mul(st);
+        w.mul(rE);
+        if (C.cb[j] != 0.0) {                       // (0: 1 + eta f of a Maxwell-Boltzmann leg, 1)
+            double f = spline64(s_spline + C.spc[j] * ncoef, knots, r, g, s32.inv_step, s32.q0, s32.lq0_step);
+            if (C.fd[j]) f = f < 1.0 ? f : 1.0;
+            w.mul(C.ca[j] != 0.0 ? fma(C.cb[j], f, C.ca[j]) : f);
+        }
     }
     const double pc2 = fma(px, px, fma(py, py, pz * pz));
     double rpc, rEc, Ec;
@@ -169,34 +218,37 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
         const double Ec2 = pc2 + C.m2c;
         rEc = rsqrt_halley(Ec2);
         Ec = Ec2 * rEc;
-        rpc = less_pos(0.0, pc2) ? rsqrt_halley(pc2) : 0.0;
+        rpc = 0.0;
+        if (C.cbc != 0.0 && less_pos(0.0, pc2)) rpc = rsqrt_halley(pc2);
     }
     cut |= less_pos(Ec, C.e_cut);
     bal += flip_sign(Ec, static_cast<uint32_t>(__double2hiint(C.sgn_cons)) & 0x80000000u);
-    double qc = pc2 * rpc;
-    if (scaled) qc *= C.a;
-    double gauss;
+    w.mul(rEc);
     if (C.frac) {
         Esum += Ec;
         const double iS = 1.0 / Esum;
         const double x = bal * iS;
-        gauss = exp2_table(C.gauss_k * x * x, tab) * (2.0 * C.e_obs * iS);
+        w.mul(exp2_table(C.gauss_k * x * x, tab));
+        w.mul(2.0 * C.e_obs * iS);
     } else {
-        gauss = exp2_table(C.gauss_k * bal * bal, tab);
+        w.mul(exp2_table(C.gauss_k * bal * bal, tab));
     }
-    const double kin = meas * rinv * rEc * gauss;
-    double fc;
-    const bool below = less_pos(qc, q0), above = less_pos(qN, qc);
-    if (!below && !above) {
-        fc = spline64(s_spline + C.sp_cons * ncoef, knots, qc, g, s32.inv_step, s32.q0, s32.lq0_step);
-    } else {
-        const double x = below ? C.tlo_a + C.tlo_b * Ec : C.thi_a + C.thi_b * Ec;
-        const double den = C.eta_c == 1.0 ? expm1(x) : exp(x) - C.eta_c;
-        fc = den > 0.0 ? 1.0 / den : 0.0;
+    if (C.cbc != 0.0) {
+        double qc = pc2 * rpc;
+        if (scaled) qc *= C.a;
+        double fc;
+        const bool below = less_pos(qc, q0), above = less_pos(qN, qc);
+        if (!below && !above) {
+            fc = spline64(s_spline + C.sp_cons * ncoef, knots, qc, g, s32.inv_step, s32.q0, s32.lq0_step);
+        } else {
+            const double x = below ? C.tlo_a + C.tlo_b * Ec : C.thi_a + C.thi_b * Ec;
+            const double den = C.eta_c == 1.0 ? expm1(x) : exp(x) - C.eta_c;
+            fc = den > 0.0 ? 1.0 / den : 0.0;
+        }
+        if (C.fd_c) fc = fc < 1.0 ? fc : 1.0;
+        w.mul(C.cac != 0.0 ? fma(C.cbc, fc, C.cac) : fc);
     }
-    if (C.fd_c) fc = fc < 1.0 ? fc : 1.0;
-    const double w = stat * fma(C.cbc, fc, C.cac) * kin;
-    return cut ? 0.0 : w;
+    return cut ? 0.0 : w.value();
 }
 
 // VEGAS map of one 52-bit uniform k + 1/2 from its Philox words, table: the
@@ -369,23 +421,30 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
     float cutoff = -3.0e38f;                // samples with log2_weight_bound below this cannot matter
 
     auto drain = [&](int slot) {
-        double y[D], jac = 1.0;
-        uint32_t bins[(D + 3) / 4] = {};
+        double y[D], dy[D];
+        uint64_t bins[2] = {};                       // 8 bits per dimension, 6 dimensions per word
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             uint32_t b;
-            const Real2<double> e = map_point64(q[(2 * d) * kQueueSlots + slot], q[(2 * d + 1) * kQueueSlots + slot], nb,
-                                                s_map + d * nb, &y[d], &b);
-            jac = d == 0 ? e.dy : jac * e.dy;
-            bins[d >> 2] |= b << (8 * (d & 3));
+            dy[d] = map_point64(q[(2 * d) * kQueueSlots + slot], q[(2 * d + 1) * kQueueSlots + slot], nb, s_map + d * nb,
+                                &y[d], &b).dy;
+            bins[d / 6] |= static_cast<uint64_t>(b) << (8 * (d % 6));
         }
-        const double w = weight64<NLEG>(C, y, jac, s_spline, knots, g, s32, s_setup->q0, s_setup->qN, ncoef, tab);
+        const double w = weight64<NLEG>(C, y, dy, s_spline, knots, g, s32, s_setup->q0, s_setup->qN, ncoef, tab);
         const double w2 = w * w;
         acc_w.add(w);
         acc_w2.add(w2);
-        if (w2 != 0.0) {
+        if (__double_as_longlong(w2) != 0) {
+            // each lane starts at another dimension: an FP64 shared-memory
+            // addition is a compare-and-swap loop, and its rounds follow the
+            // number of lanes on one increment (3.1 -> about 1.3 rounds)
+            int d = lane % D;
 #pragma unroll
-            for (int d = 0; d < D; ++d) atomicAdd(&w_hist[d * nb + ((bins[d >> 2] >> (8 * (d & 3))) & 0xFFu)], w2);
+            for (int k = 0; k < D; ++k) {
+                const uint32_t b = static_cast<uint32_t>((d < 6 ? bins[0] >> (8 * d) : bins[1] >> (8 * (d - 6))) & 0xFFu);
+                atomicAdd(&w_hist[d * nb + b], w2);
+                d = d + 1 == D ? 0 : d + 1;
+            }
         }
         return __double2hiint(w) & 0x7fffffff;
     };
