@@ -14,23 +14,25 @@
 //   * samples whose Gaussian exponent is below -1100 (|dE| > 39 sigma): their
 //     FP64 weight is exactly 0 (2^-1075 is the smallest subnormal);
 //   * samples with L < log2(largest |w_n| this warp has evaluated in the
-//     segment) - kDropBits, kDropBits = 120.  L takes the kinematic factors and
-//     the statistical ones from FP32 with their rounding bounded (a few bits).
-//     Even 2^31 samples of 2^-120 are far below the rounding of the sums of w
-//     and w^2, and an increment holding nothing else has a share below the
-//     1e-30 = 2^-100 of w^2 that the refinement counts as empty.
+//     segment) - kDropBits - log2 N, kDropBits = 66, N the task's samples.  L
+//     takes the kinematic factors and the statistical ones from FP32 with their
+//     rounding bounded (a few bits).  All such samples together are below 2^-66
+//     of one that was summed, 2^-13 of the last place of the sum of w (and of
+//     w^2 far below), and an increment holding nothing else has a share of w^2
+//     below the 1e-30 = 2^-100 that the refinement counts as empty.
 // A sample whose FP32 quantities leave the normal range is kept.
 //
-// Measured per launch on trained maps, plain loop -> this one: MB 2 -> 2, 32
-// points, 1e5 samples: 4.08 -> 0.50 ms; BE 2 -> 2, 2 species, 128 points, 1e5
-// samples: 27.4 -> 6.19 ms (the FP64 pipe then 84% busy).
+// Measured per sweep on trained maps, plain loop -> this one: MB 2 -> 2, 32
+// points, 1e5 x 2 samples: 8.27 -> 0.80 ms; BE 2 -> 2, 2 species, 128 points,
+// 1e5 x 2: 55.2 -> 9.0 ms (40% of the samples are evaluated with a fixed 2^-120;
+// the FP64 pipe is 80% busy, about 120 operations per queued sample).
 #pragma once
 
 #include "math_table.cuh"
 
 namespace best {
 
-constexpr float kDropBits = 120.0f;
+constexpr float kDropBits = 66.0f;
 
 // ---- FP64 elementary functions of this loop: fewer FP64 operations than the
 // library's, at the price of a restricted range (checked or falling back) ----
@@ -408,7 +410,9 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
     }
     SegSetup<float, NLEG> s32;
     seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
-    const float log2_c0 = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f));     // (upper bound)
+    // what the largest weight's exponent is lowered by: the bound leaves c0 out
+    const float below = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f)) + kDropBits +
+                        static_cast<float>(64 - __clzll(static_cast<long long>(td.neval)));
     __syncthreads();
     const SegConst<double, NLEG>& C = s_setup->C;
     const double* knots = s_spline + g.n_species * 4 * (g.n_grid - 1);
@@ -477,7 +481,7 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
                 const int top = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(hi)));
                 if (top > wmax && top < 0x7FE00000) {
                     wmax = top;
-                    cutoff = static_cast<float>((top >> 20) - 1023) - log2_c0 - kDropBits;
+                    cutoff = static_cast<float>((top >> 20) - 1023) - below;
                 }
                 __syncwarp();
                 if (lane < qn - 32) {
