@@ -298,7 +298,9 @@ struct EBal2 {
 
 // kin_at for two samples at once (constant |M|^2), each FP32 operation
 // packed over the pair; the special-function operations stay per sample.
-template <int NLEG>
+// SAME: the products are taken in kin_at's order, so that both loops give the
+// same bits (the default loop of a 2 -> 2 problem depends on its size).
+template <int NLEG, bool SAME>
 __device__ __forceinline__ float2 kin_pair(const SegConst<float, NLEG>& C, const float2* y, float2 jac, float2* r,
                                            float2& qc, float2& Ec) {
     constexpr int NI = NLEG - 2;
@@ -343,22 +345,19 @@ __device__ __forceinline__ float2 kin_pair(const SegConst<float, NLEG>& C, const
     const float2 rpc = make_float2(pc2.x > 1e-30f ? rsqrt_ftz(pc2.x) : 0.0f, pc2.y > 1e-30f ? rsqrt_ftz(pc2.y) : 0.0f);
     qc = mul2(mul2(pc2, rpc), bc2(C.a));
     float2 gauss;
-    // up to four legs the products are taken in kin_at's order, so that both
-    // loops give the same bits (the default of a 2 -> 2 problem depends on its size)
-    constexpr bool kSame = NLEG <= 4;
     if (C.frac) {
         // sigma = w S / 2 with S = E_in + E_out: exponent -2 dE^2 / (w S)^2,
         // normalisation sigma_ref / sigma = 2 E_obs / S
         Esum = add2(Esum, Ec);
         const float2 iS = make_float2(__fdividef(1.0f, Esum.x), __fdividef(1.0f, Esum.y));
         const float2 x = mul2(dE, iS);
-        const float2 e = kSame ? mul2(mul2(bc2(C.gauss_k), x), x) : mul2(mul2(x, x), bc2(C.gauss_k));
+        const float2 e = SAME ? mul2(mul2(bc2(C.gauss_k), x), x) : mul2(mul2(x, x), bc2(C.gauss_k));
         gauss = mul2(make_float2(ex2_ftz(e.x), ex2_ftz(e.y)), mul2(bc2(2.0f * C.e_obs), iS));
     } else {
-        const float2 e = kSame ? mul2(mul2(bc2(C.gauss_k), dE), dE) : mul2(mul2(dE, dE), bc2(C.gauss_k));
+        const float2 e = SAME ? mul2(mul2(bc2(C.gauss_k), dE), dE) : mul2(mul2(dE, dE), bc2(C.gauss_k));
         gauss = make_float2(ex2_ftz(e.x), ex2_ftz(e.y));
     }
-    float2 w = kSame ? mul2(mul2(mul2(meas, rinv), rEc), gauss) : mul2(mul2(meas, rinv), mul2(rEc, gauss));
+    float2 w = SAME ? mul2(mul2(mul2(meas, rinv), rEc), gauss) : mul2(mul2(meas, rinv), mul2(rEc, gauss));
     w.x = emin0 < C.e_cut ? 0.0f : w.x;
     w.y = emin1 < C.e_cut ? 0.0f : w.y;
     return w;
@@ -719,7 +718,7 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
                     qn -= 32;
                 }
             };
-            if constexpr (!STRAT && SPL == 2) {
+            if constexpr (!STRAT && SPL >= 2) {
                 // Two samples per step in packed FP32x2 arithmetic: the two
                 // samples of a group (G even) or of two consecutive groups
                 // (G = 1, a lane then takes groups 2k and 2k + 1).  The
@@ -767,7 +766,7 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
                             jac = __fmul2_rn(jac, dy);
                         }
                         float2 r2[NI], qc2, Ec2;
-                        const float2 kin = kin_pair<NLEG>(C, y, jac, r2, qc2, Ec2);
+                        const float2 kin = kin_pair<NLEG, SPL == 3>(C, y, jac, r2, qc2, Ec2);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             float r[NI];
@@ -1095,8 +1094,8 @@ __device__ __forceinline__ void run_segment(const EvalParams& P, const Segment& 
 
 // MB: CTAs per SM the kernel is register-limited to (__launch_bounds__);
 // THREADS: threads per CTA; SPL: samples a lane evaluates per step of the
-// FP32 loop (1, or 2 in packed FP32x2 arithmetic); for FP64, 2 is the loop
-// with the FP32 screen (eval_f64q.cuh).  Several combinations are
+// FP32 loop (1, or 2 in packed FP32x2 arithmetic; 3: 2 with the products in the
+// order of 1); for FP64, 2 is the loop with the FP32 screen (eval_f64q.cuh).  Several combinations are
 // instantiated and the autotuner picks one at run time.
 template <typename R, int NMAX, int MB, bool STRAT = false, int THREADS = kThreads, int SPL = 1>
 __global__ void __launch_bounds__(THREADS, MB)
