@@ -131,8 +131,8 @@ struct best_ctx {
     double* d_edges = nullptr;
     double* d_knots = nullptr;
     float* d_knots32 = nullptr;
-    double* d_splplan = nullptr;    // elimination factors of the grid's spline (SplinePlan)
-    SideConst* d_sideconst = nullptr;
+    double* d_splplan = nullptr;    // elimination factors of the grid's spline (SplinePlan), then the side constants
+    SideConst* d_sideconst = nullptr;   // (in the same allocation)
     double* d_coef64 = nullptr;
     float* d_coef32 = nullptr;
     double* d_fgrid = nullptr;
@@ -258,7 +258,7 @@ void free_all(best_ctx* c) {
     for (void* b : bufs) cudaFree(b);
     cudaFree(c->d_bctl); cudaFree(c->d_bv); cudaFree(c->d_plan_scratch); cudaFree(c->d_plandev);
     cudaFree(c->d_chunk_ctr);
-    cudaFree(c->d_splplan); cudaFree(c->d_sideconst);
+    cudaFree(c->d_splplan);
     if (c->h_nk) cudaFreeHost(c->h_nk);
     c->h_nk = nullptr;
 }
@@ -1004,8 +1004,9 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
     CKI(dalloc(&ctx->d_edges, static_cast<size_t>(T) * g.map_stride));
     CKI(dalloc(&ctx->d_knots, n));
     CKI(dalloc(&ctx->d_knots32, n));
-    CKI(dalloc(&ctx->d_splplan, spline_plan_doubles(n)));
-    CKI(dalloc(&ctx->d_sideconst, g.n_side));
+    static_assert(sizeof(SideConst) == 3 * sizeof(double), "side constants are doubles");
+    CKI(dalloc(&ctx->d_splplan, spline_plan_doubles(n) + 3 * static_cast<size_t>(g.n_side)));
+    ctx->d_sideconst = reinterpret_cast<SideConst*>(ctx->d_splplan + spline_plan_doubles(n));
     CKI(dalloc(&ctx->d_coef64, static_cast<size_t>(S) * (n - 1) * 4));
     CKI(dalloc(&ctx->d_coef32, static_cast<size_t>(S) * (n - 1) * 4));
     CKI(dalloc(&ctx->d_fgrid, static_cast<size_t>(S) * n));
@@ -1078,12 +1079,13 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
     CKI(cudaMemcpy(ctx->d_knots, knots.data(), n * sizeof(double), cudaMemcpyHostToDevice));
     CKI(cudaMemcpy(ctx->d_knots32, knots32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
     {
-        std::vector<double> plan(spline_plan_doubles(n), 0.0);
+        std::vector<double> plan(spline_plan_doubles(n) + 3 * static_cast<size_t>(g.n_side), 0.0);
         spline_plan(n, knots.data(), plan.data());
+        for (int k = 0; k < g.n_side; ++k) {
+            const SideConst sc = side_const(ctx->sides[k], cfg->processes[ctx->sides[k].process].nbins);
+            std::memcpy(&plan[spline_plan_doubles(n) + 3 * static_cast<size_t>(k)], &sc, sizeof(sc));
+        }
         CKI(cudaMemcpy(ctx->d_splplan, plan.data(), plan.size() * sizeof(double), cudaMemcpyHostToDevice));
-        std::vector<SideConst> sc(g.n_side);
-        for (int k = 0; k < g.n_side; ++k) sc[k] = side_const(ctx->sides[k], cfg->processes[ctx->sides[k].process].nbins);
-        CKI(cudaMemcpy(ctx->d_sideconst, sc.data(), sc.size() * sizeof(SideConst), cudaMemcpyHostToDevice));
     }
     CKI(cudaMemcpy(ctx->d_mass_law, ctx->mass_law.data(), S * sizeof(MassLaw), cudaMemcpyHostToDevice));
     CKI(refresh_map32(ctx, nullptr));

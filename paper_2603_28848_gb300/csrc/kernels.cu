@@ -20,7 +20,7 @@ __device__ inline double scale_factor(const Geometry& g, double t) {
 // lanes' affine maps are combined by a shuffle scan, and the rows are run
 // again from the carry.  An FP64 operation of a warp takes the pipe for 64
 // cycles whatever its lanes do, so the 3 n / 32 + 10 operations here replace
-// 3 n dependent ones: 120 us -> 13 us for the whole spline build at n = 256.
+// 3 n dependent ones: 120 us -> 8 us for the whole spline build at n = 256.
 // Rows per lane are odd so that the lanes' shared-memory rows fall in
 // different banks.
 __device__ inline void tri_solve_warp(int m, double* y, const double* g, const double* c) {
@@ -396,7 +396,7 @@ __device__ inline double clamp_scale(double scale, double obs_factor) {
 // One thread per task; FP64 operations take an SM partition's pipe for 64
 // cycles per warp, so the CTAs are single warps (spread over the SMs), what
 // depends on neither time nor distribution comes from SideConst, and the
-// common a = 1 skips its powers (13.7 -> 6 us for 512 tasks).
+// common a = 1 skips its powers (13.7 -> 6.9 us for 512 tasks).
 __global__ void prepare_kernel(Geometry g, const SideDesc* __restrict__ sides,
                                const TaskDesc* __restrict__ tasks, const double* __restrict__ knots,
                                const double* __restrict__ fgrid, const TimeState* ts,
@@ -674,8 +674,8 @@ __global__ void strat_refine_kernel(const TaskDesc* __restrict__ tasks, const in
 // loads: one warp per dimension runs its dimension from smoothing to edges
 // without block barriers (warp-wide sums and scans, comparisons as integers),
 // while a fourth warp makes the task's scalars; the legs' CTAs spread a small
-// problem over the SMs.  FP32 2 -> 2: 17.8 -> 7.3 us for 64 tasks, 83 -> 42 us for
-// 512.  Dynamic shared memory: refine_doubles(nbins_max) doubles.
+// problem over the SMs.  FP32 2 -> 2: 17.8 -> 8.7 us for 64 tasks, 83 -> 52 us for
+// 512; 486 -> 302 us for 6144 tasks of 2 -> 2 and 2 -> 3.  Dynamic shared memory: refine_doubles(nbins_max) doubles.
 // ---------------------------------------------------------------------------
 __global__ void refine_kernel(Geometry g, const SideDesc* __restrict__ sides,
                               const TaskDesc* __restrict__ tasks, const TaskConst* tconst,
@@ -907,7 +907,7 @@ __global__ void map32_kernel(Geometry g, const TaskDesc* __restrict__ tasks, int
 // C_a(p_i) = sum_sides mult (I_gain - I_loss), err^2 = sum mult^2
 // (sigma_gain^2 + sigma_loss^2).  Two lanes per (species, grid point), one for
 // its gain and one for its loss tasks, 32 threads per CTA (the combination is
-// a chain of FP64 divisions: spread over the SMs, 4.5 -> 3.6 us for 32 points);
+// a chain of FP64 divisions: spread over the SMs, 4.5 -> 3.0 us for 32 points);
 // thread 0 advances the evaluation counter.
 // ---------------------------------------------------------------------------
 __device__ inline void combine_task(TaskAcc& A) {

@@ -90,15 +90,25 @@ struct SetupArgs {
 };
 
 // The grid's spline factors, made on the host (their recurrence is a chain of
-// dependent divisions) and handed over by value: 28 KB of kernel parameters,
-// so nothing on the host has to outlive the call.
+// dependent divisions) and handed over by value, up to 28 KB of kernel
+// parameters, so nothing on the host has to outlive the call.  A launch copies
+// its parameters: small grids take the small instantiation.
+template <int N>
 struct PlanArgs {
-    double v[spline_plan_doubles(kMaxGrid)];
+    double v[spline_plan_doubles(N)];
 };
-static_assert(sizeof(PlanArgs) < 32000, "kernel parameters are limited to 32764 bytes");
+static_assert(sizeof(PlanArgs<kMaxGrid>) < 32000, "kernel parameters are limited to 32764 bytes");
 
-__global__ void noalloc_plan_kernel(PlanArgs A, int count, double* out) {
+template <int N>
+__global__ void noalloc_plan_kernel(PlanArgs<N> A, int count, double* out) {
     for (int k = threadIdx.x; k < count; k += blockDim.x) out[k] = A.v[k];
+}
+
+template <int N>
+void send_plan(int n, const double* knots, double* out, cudaStream_t st) {
+    PlanArgs<N> plan;
+    spline_plan(n, knots, plan.v);
+    noalloc_plan_kernel<N><<<1, 512, 0, st>>>(plan, 6 * n + 4, out);
 }
 
 // Writes the descriptors, the grid, the time state and the partition of the
@@ -284,16 +294,12 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
     A.td = td;
     A.sideconst = side_const(sd, nb);
     A.ctas = ctas;
-    PlanArgs plan{};
-    {
-        double q[kMaxGrid];
-        for (int j = 0; j < n; ++j)
-            q[j] = g.log_spaced ? g.q_min * std::pow(g.q_max / g.q_min, static_cast<double>(j) / (n - 1))
-                                : g.q_min + (g.q_max - g.q_min) * j / (n - 1);
-        q[0] = g.q_min;
-        q[n - 1] = g.q_max;
-        spline_plan(n, q, plan.v);
-    }
+    double q[kMaxGrid];
+    for (int j = 0; j < n; ++j)
+        q[j] = g.log_spaced ? g.q_min * std::pow(g.q_max / g.q_min, static_cast<double>(j) / (n - 1))
+                            : g.q_min + (g.q_max - g.q_min) * j / (n - 1);
+    q[0] = g.q_min;
+    q[n - 1] = g.q_max;
     const int G = group_size(D, f32);
     A.groups = (td.neval + G - 1) / G;
 
@@ -314,7 +320,8 @@ extern "C" best_status best_vegas_iteration_noalloc(const best_config* cfg, int3
 
     noalloc_setup_kernel<<<1, 512, 0, st>>>(A, base);
     double* splplan = reinterpret_cast<double*>(base + kOffSplPlan);
-    noalloc_plan_kernel<<<1, 512, 0, st>>>(plan, spline_plan_doubles(n), splplan);
+    if (n <= 64) send_plan<64>(n, q, splplan, st);
+    else send_plan<kMaxGrid>(n, q, splplan, st);
     const size_t spline_smem = 4 * sizeof(double) * n;
     spline_build_kernel<<<S, 256, spline_smem, st>>>(g, SweepStart{nullptr, nullptr, nullptr, 0.0, 0, 0}, f_dev, 0,
                                                      knots, SplinePlan{splplan, n, 0}, ts, sc, fgrid, coef64, coef32);
