@@ -468,12 +468,16 @@ __device__ int64_t cta_exclusive_scan(int64_t v, int64_t* s, int64_t* total) {
     return incl - v;
 }
 
-// f(h, first, count) for every hypercube h of a task, first and count its items
-// (m, in hypercube order): hypercubes of at least 32 items by whole warps
-// (wide = true, every lane calls f with the same arguments), smaller ones by
-// one thread each.  s, off, cnt: 256 entries of shared memory each.
+// f(h, first, count, scope) for every hypercube h of a task, first and count
+// its items (m, in hypercube order).  Who calls it follows the count, so that
+// neither many small hypercubes nor one that drew most of the items leaves the
+// CTA idle: below 32 items one thread (scope 1), below 1024 or J / 16 (J: the
+// task's items) one warp (scope 32, every lane with the same arguments), else
+// every thread of the CTA (scope blockDim, together).  The caller's index within the scope is threadIdx.x %
+// scope.  s, off, cnt: 256 entries of shared memory each.
 template <typename F>
-__device__ void for_hypercubes(const int32_t* m, int H, int64_t* s, int64_t* off, int32_t* cnt, F&& f) {
+__device__ void for_hypercubes(const int32_t* m, int H, int64_t J, int64_t* s, int64_t* off, int32_t* cnt, F&& f) {
+    const int64_t large = max(int64_t(1024), J / 16);
     int64_t base = 0;
     for (int c0 = 0; c0 < H; c0 += blockDim.x) {
         const int h = c0 + static_cast<int>(threadIdx.x);
@@ -483,11 +487,13 @@ __device__ void for_hypercubes(const int32_t* m, int H, int64_t* s, int64_t* off
         off[threadIdx.x] = ex;
         cnt[threadIdx.x] = v;
         __syncthreads();
-        if (v > 0 && v < 32) f(h, ex, v, false);
+        if (v > 0 && v < 32) f(h, ex, v, 1);
         __syncwarp();
         const int nh = min(H - c0, static_cast<int>(blockDim.x));
         for (int k = threadIdx.x >> 5; k < nh; k += blockDim.x >> 5)
-            if (cnt[k] >= 32) f(c0 + k, off[k], cnt[k], true);
+            if (cnt[k] >= 32 && cnt[k] < large) f(c0 + k, off[k], cnt[k], 32);
+        for (int k = 0; k < nh; ++k)
+            if (cnt[k] >= large) f(c0 + k, off[k], cnt[k], static_cast<int>(blockDim.x));
         base += tot;
         __syncthreads();
     }
@@ -495,9 +501,8 @@ __device__ void for_hypercubes(const int32_t* m, int H, int64_t* s, int64_t* off
 
 __device__ void strat_write_items(const int32_t* m, int H, int64_t J, uint32_t* item_h, int64_t* s, int64_t* off,
                                   int32_t* cnt) {
-    for_hypercubes(m, H, s, off, cnt, [&](int h, int64_t first, int32_t count, bool wide) {
-        const int lane = threadIdx.x & 31;
-        for (int k = wide ? lane : 0; k < count; k += wide ? 32 : 1)
+    for_hypercubes(m, H, J, s, off, cnt, [&](int h, int64_t first, int32_t count, int scope) {
+        for (int k = threadIdx.x % scope; k < count; k += scope)
             if (first + k < J) item_h[first + k] = static_cast<uint32_t>(h);
     });
 }
@@ -534,7 +539,7 @@ __global__ void strat_init_kernel(const TaskDesc* __restrict__ tasks, int32_t* s
 // next allocation m_h = 1 + floor((J - H) d_h / sum d), d_h = (s_h^2)^(beta/2),
 // the remaining items one each to h = 0, 1, ... (uniform if every d_h = 0),
 // and the items rebuilt.  An underflowed iteration keeps its allocation.
-__global__ void strat_refine_kernel(const TaskDesc* __restrict__ tasks, const int32_t* __restrict__ active,
+__global__ void __launch_bounds__(256, 4) strat_refine_kernel(const TaskDesc* __restrict__ tasks, const int32_t* __restrict__ active,
                                     const double* __restrict__ item_rec, int32_t* strat_m, double* strat_d,
                                     double* strat_s2, uint32_t* item_h, double* est) {
     __shared__ int64_t s[256], off[256];
@@ -551,42 +556,74 @@ __global__ void strat_refine_kernel(const TaskDesc* __restrict__ tasks, const in
     double* S2h = strat_s2 + td.strat_off_h;
     const double2* rec = reinterpret_cast<const double2*>(item_rec) + td.strat_off_item;
     // per-hypercube sums of its items' records, in an order fixed by the
-    // allocation: coalesced loads, two FP64 additions per record and lane, and
-    // one chain of additions per hypercube (lower lanes w, upper lanes w^2).
-    // (Per-thread runs of items whose ends one thread added up took 204 us for
-    // 512 tasks of 12500 items, most of it that thread.)
-    for_hypercubes(m, H, s, off, cnt, [&](int h, int64_t first, int32_t count, bool wide) {
+    // allocation: coalesced loads, two FP64 additions per record and thread, one
+    // chain of additions per warp (lower lanes w, upper lanes w^2).  (Per-thread
+    // runs of items whose ends one thread added up took 204 us for 512 tasks of
+    // 12500 items, most of it that thread; now 104 us.  The additions alone take
+    // the FP64 pipe 22 us there and 220 us for 125000 items.)
+    __shared__ double s_w[16];
+    for_hypercubes(m, H, J, s, off, cnt, [&](int h, int64_t first, int32_t count, int scope) {
         double s1 = 0.0, s2 = 0.0;
-        const int lane = threadIdx.x & 31;
-        const int step = wide ? 32 : 1;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const double2* p = rec + first;
-        int k = wide ? lane : 0;
-        for (; k + 3 * step < count; k += 4 * step) {
+        int k = threadIdx.x % scope;
+        if (k + 3 * scope < count) {
+            // four records in flight while the four before are added
             double2 x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = p[k + u * step];
+            for (int u = 0; u < 4; ++u) x[u] = p[k + u * scope];
+            k += 4 * scope;
+            for (; k + 3 * scope < count; k += 4 * scope) {
+                double2 y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) y[u] = p[k + u * scope];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    s1 += x[u].x;
+                    s2 += x[u].y;
+                    x[u] = y[u];
+                }
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 s1 += x[u].x;
                 s2 += x[u].y;
             }
         }
-        for (; k < count; k += step) {
-            s1 += p[k].x;
-            s2 += p[k].y;
-        }
-        if (wide) {
-            const bool up = lane >= 16;
-            double v = up ? s2 : s1;
-            v += __shfl_xor_sync(0xffffffffu, up ? s1 : s2, 16);
+        for (; k < count; k += 4 * scope) {
+            double2 x[4];
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) S1h[h] = v;
-            if (lane == 16) S2h[h] = v;
-        } else {
+            for (int u = 0; u < 4; ++u) x[u] = k + u * scope < count ? p[k + u * scope] : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k + u * scope < count) {
+                    s1 += x[u].x;
+                    s2 += x[u].y;
+                }
+        }
+        if (scope == 1) {
             S1h[h] = s1;
             S2h[h] = s2;
+            return;
         }
+        const bool up = lane >= 16;
+        double v = up ? s2 : s1;
+        v += __shfl_xor_sync(0xffffffffu, up ? s1 : s2, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        double* S = up ? S2h : S1h;
+        if (scope == 32) {
+            if ((lane & 15) == 0) S[h] = v;
+            return;
+        }
+        if ((lane & 15) == 0) s_w[2 * warp + (up ? 1 : 0)] = v;
+        __syncthreads();
+        if (warp == 0 && (lane & 15) == 0) {
+            double sum = 0.0;
+            for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) sum += s_w[2 * w + (up ? 1 : 0)];
+            S[h] = sum;
+        }
+        __syncthreads();
     });
     __syncthreads();
     double a_mean = 0.0, a_var = 0.0, a_d = 0.0, a_abs = 0.0, a_bad = 0.0;
