@@ -299,11 +299,13 @@ __device__ __forceinline__ float log2_factor_bound(const float* coef, const floa
 
 // Upper bound of log2 |w_n| of a sample from FP32 arithmetic, y the mapped
 // point and jac the map's Jacobian; gauss gets an upper bound of the
-// Gaussian's exponent.  Every momentum component carries at most about 4e-6
-// of the momenta (sin.approx and cos.approx: 2^-21 absolute; the FP32 map:
-// 2^-22 of an angle), every energy 2e-7: 4e-5 of the energies' sum covers the
-// balance ten times.  +inf where a factor leaves the normal range (or is not a
-// number).  STAT false: of the kinematic part alone.
+// Gaussian's exponent.  Errors: a radius carries 2^-22 of itself and, from the
+// 32-bit uniform, up to 2^-24 of the largest increment (1.2e-7 q_max); an angle
+// and sin.approx / cos.approx 2^-20 absolute.  Every momentum component is then
+// within 4e-6 of the momenta plus 1e-6 q_max / a of the four radii, and 4e-5 of
+// the energies' sum plus that covers the balance ten times.  +inf where a
+// factor leaves the normal range (or is not a number) or the conserved leg's
+// energy is not resolved.  STAT false: of the kinematic part alone.
 template <int NLEG, bool STAT>
 __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& S, const EvalParams& P, const float* y,
                                                    float jac, float* gauss) {
@@ -329,7 +331,8 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
         const float E = E2 * rE;
         bal = fmaf(C.sgnE[j], E, bal);
         Esum += E;
-        prod *= r * r * st * rE;
+        const float ru = fmaf(1.2e-7f, S.qN, r);
+        prod *= ru * ru * (st + 2e-6f) * rE;
     }
     const float pc2 = fmaf(px, px, fmaf(py, py, pz * pz));
     const float Ec2 = pc2 + C.m2c;
@@ -338,7 +341,8 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     bal = fmaf(C.sgn_cons, Ec, bal);
     Esum += Ec;
     prod *= rEc;
-    float d = fmaxf(fabsf(bal) - 4e-5f * Esum, 0.0f);
+    const float err = fmaf(4e-5f, Esum, 1e-6f * S.qN * C.inv_a);
+    float d = fmaxf(fabsf(bal) - err, 0.0f);
     if (!(Esum < 1e30f)) d = 0.0f;                       // (overflowed, or not a number)
     float extra = 0.0f;
     if (C.frac) {
@@ -348,7 +352,7 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     }
     const float e = C.gauss_k * d * d;
     *gauss = e;
-    if (!(prod > 1e-37f && prod < 1e37f)) return __int_as_float(0x7f800000);
+    if (!(prod > 1e-37f && prod < 1e37f && Ec > 4.0f * err)) return __int_as_float(0x7f800000);
     const float kin = lg2_ftz(prod) + extra + e;
     if constexpr (!STAT) return kin + 2.0f;
     // the statistical factors, 1 + f or f of every leg (|ca + cb f| is at most ca + f)

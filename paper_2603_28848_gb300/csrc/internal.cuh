@@ -401,8 +401,9 @@ __device__ inline SegConst32 seg_const32(const SideDesc& sd, const TaskDesc& td,
 // The FP32 kernels' map table of one task: for dimension d and increment b,
 // the left end and the width of increment b in the physical variable (r
 // comoving, theta, phi - pi), from the FP64 edges in [0, 1] rounded to FP32;
-// entry d * nb + b of the task's kMaxDim * nbins_max entries.  Written by
-// map32_kernel (every sweep) and by the refinement for the tasks it refines.
+// entry d * nb + b of the task's kMaxDim * nbins_max entries.  Written by the
+// refinement for the tasks it refines, and by map32_kernel where the edges are
+// set from outside.
 __host__ __device__ inline int map32_stride(const Geometry& g) { return kMaxDim * g.nbins_max; }
 __device__ inline float2 map32_value(double e0, double e1, int d, const Geometry& g) {     // of edges e0, e1 of dimension d
     double lo, sc;
