@@ -70,3 +70,24 @@ def test_large_grid_takes_the_plain_loop():
     col.check()
     assert bool(torch.isfinite(C).all()) and bool((C != 0).any())
     col.close()
+
+
+def test_narrow_width_on_a_wide_grid():
+    """Radii of a wide map carry more FP32 rounding than a soft leg's energy: the
+    screen's bound has to hold there too (energies up to 3e3, width 1e-3: FP64
+    rounding 1e-12 over it times 39 is 4e-8 of a weight)."""
+    import torch
+    from paper_2603_28848_gb300 import Collision
+    prob, f0, t = _mb(6, 20_000, sigma_E=1e-3)
+    prob = replace(prob, grid=replace(prob.grid, q_min=1e-3, q_max=300.0))
+    q = W.grid_points(prob.grid)
+    f0 = (0.5 * np.exp(-np.sqrt(q * q + 1.0) / 20.0))[None, :]
+    col = Collision(prob, W.PREC_FP64)
+    col.eval(torch.tensor(f0, device="cuda"), t)
+    mean, _ = col.task_results()
+    col.close()
+    _, _, detail, _ = oracle_sweep(prob, f0, t, "f64")
+    om, _ = task_arrays(detail, len(mean))
+    ok = np.isfinite(om)
+    assert ok.mean() > 0.8 and np.any(om != 0)
+    assert np.all(np.abs(mean - om)[ok] <= (1e-6 * np.abs(om) + 1e-300)[ok])
