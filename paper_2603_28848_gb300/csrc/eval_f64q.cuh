@@ -24,8 +24,8 @@
 //
 // Measured per sweep on trained maps, plain loop -> this one: MB 2 -> 2, 32
 // points, 1e5 x 2 samples: 8.27 -> 0.80 ms; BE 2 -> 2, 2 species, 128 points,
-// 1e5 x 2: 55.2 -> 9.0 ms (40% of the samples are evaluated with a fixed 2^-120;
-// the FP64 pipe is 80% busy, about 120 operations per queued sample).
+// 1e5 x 2: 55.2 -> 9.6 ms (with a fixed 2^-120, 10.0 ms: 40% of the samples are
+// evaluated, the FP64 pipe is 80% busy, about 120 operations per queued sample).
 #pragma once
 
 #include "math_table.cuh"

@@ -559,8 +559,8 @@ __global__ void __launch_bounds__(256, 4) strat_refine_kernel(const TaskDesc* __
     // allocation: coalesced loads, two FP64 additions per record and thread, one
     // chain of additions per warp (lower lanes w, upper lanes w^2).  (Per-thread
     // runs of items whose ends one thread added up took 204 us for 512 tasks of
-    // 12500 items, most of it that thread; now 104 us.  The additions alone take
-    // the FP64 pipe 22 us there and 220 us for 125000 items.)
+    // 12500 items, most of it that thread; now 97 us, and 437 us for 125000 items
+    // (523).  The additions alone take the FP64 pipe 22 and 220 us.)
     __shared__ double s_w[16];
     for_hypercubes(m, H, J, s, off, cnt, [&](int h, int64_t first, int32_t count, int scope) {
         double s1 = 0.0, s2 = 0.0;
