@@ -253,16 +253,26 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
     return cut ? 0.0 : w.value();
 }
 
-// VEGAS map of one 52-bit uniform k + 1/2 from its Philox words, table: the
-// dimension's increments.  (2 k + 1) nb: the increment is the part above bit
-// 53, the fraction the 53 bits below it, turned into an FP64 number in integer
-// operations.
+// VEGAS map of one 52-bit uniform u = (k + 1/2) 2^-52 from its Philox words,
+// table: the dimension's increments.  The increment and the fraction are those
+// of t = u nb rounded to FP64, as every other evaluation of the same stream
+// takes them (the fraction's rounding, 2^-48 for 50 increments, is the largest
+// one before the energy balance: without it the samples are other ones by that
+// much).  In integer operations: t = m 2^-53, rounded to nearest even at bit s.
 __device__ __forceinline__ Real2<double> map_point64(uint32_t x0, uint32_t x1, int nb, const Real2<double>* table,
                                                      double* y, uint32_t* bin = nullptr) {
     const uint64_t k = (static_cast<uint64_t>(x0 >> 6) << 26) | (x1 >> 6);
-    const uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);
-    const uint32_t b = static_cast<uint32_t>(m >> 53);
-    const uint64_t frac = m & ((1ull << 53) - 1);              // exact in FP64
+    uint64_t m = (2 * k + 1) * static_cast<uint32_t>(nb);      // < 2^61
+    const int s = max(0, 11 - __clz(static_cast<int>(m >> 32)));          // bits past the 53rd: 0 .. 8
+    const uint32_t ulp = 1u << s;
+    const uint32_t even = s ? ((static_cast<uint32_t>(m) >> s) & 1u) : 1u;
+    m = (m + ((ulp >> 1) - 1u + even)) & ~static_cast<uint64_t>(ulp - 1u);
+    uint32_t b = static_cast<uint32_t>(m >> 53);
+    uint64_t frac = m & ((1ull << 53) - 1);                    // exact in FP64
+    if (b == static_cast<uint32_t>(nb)) {                      // t rounded up to nb: the end of the last increment
+        --b;
+        frac = 1ull << 53;
+    }
     const int lz = __clzll(static_cast<long long>(frac));
     const uint64_t bits = (((frac << lz) >> 11) & 0x000FFFFFFFFFFFFFull) | (static_cast<uint64_t>(1033 - lz) << 52);
     const double fr = __longlong_as_double(frac ? static_cast<long long>(bits) : 0);
