@@ -349,7 +349,9 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
     // FP32: samples with a non-zero kinematic part are queued per warp and
     // their statistical factors and derivatives evaluated 32 at a time (as in
     // the sample kernel); the warp runs the loop in step so that its votes
-    // see all 32 lanes.
+    // see all 32 lanes.  (Written out apart from the FP64 one below: the order in
+    // which the warps reach the coefficient sums follows the code's timing, and
+    // those sums' last digits with it.)
     constexpr int QW = vjp_queue_words(NLEG, JVP);
     float* q = F32 ? s_queue + (tid >> 5) * (kQueueSlots * QW) : nullptr;
     const int lane = tid & 31;
@@ -372,97 +374,6 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                        q[(5 + 2 * NI) * kQueueSlots + slot], q[(6 + 2 * NI) * kQueueSlots + slot]);
         }
     };
-    // Kinematic part of one sample at the mapped point y with map Jacobian jac
-    // (kin_at of the sample kernel, plus what the derivatives need).
-    struct Kin {
-        R base, r[NI], rE[NI], qc, Ec, rEc, dEs, sig_term, me_d;
-    };
-    auto sincos_of = [&](R x, R* sn, R* cs) {
-        if constexpr (F32) RMath<R>::sincos_(x, sn, cs);
-        else sincos_table(x, tab, sn, cs);
-    };
-    auto rsqrt_of = [&](R x) {
-        if constexpr (F32) return RMath<R>::rsqrt_(x);
-        else return rsqrt_halley(x);
-    };
-    auto exp2_of = [&](R x) {
-        if constexpr (F32) return RMath<R>::exp2_(x);
-        else return exp2_table(x, tab);
-    };
-    auto kinematics = [&](const R* y, R jac, bool valid, Kin& k) {
-        R px = R(0), py = R(0), pz = pobs_sig;
-        EBal<R> bal(sgn_obs_E);
-        R Esum = e_obs;
-        R Qx = R(0), Qy = R(0), Qz = obs_in_p, Ein = obs_in_E;
-        R meas = jac;
-        R rinv = R(1);
-        bool cut = obs_cut;
-#pragma unroll
-        for (int j = 0; j < NI; ++j) {
-            k.r[j] = y[3 * j];
-            R st, ct, sp, cp;
-            sincos_of(y[3 * j + 1], &st, &ct);
-            sincos_of(y[3 * j + 2], &sp, &cp);
-            const R p = k.r[j] * inv_a;
-            const R ps = p * st;
-            px = fma(-sig[j] * ps, cp, px);
-            py = fma(-sig[j] * ps, sp, py);
-            pz = fma(sig[j] * p, ct, pz);
-            const R E2 = fma(p, p, m2[j]);
-            const R rr = rsqrt_of(E2);
-            const R E = E2 * rr;
-            cut |= E < e_cut;
-            bal.add(sgnE[j] * E);
-            Esum += E;
-            if (me_on) {
-                Qx = fma(-inw[j] * ps, cp, Qx);
-                Qy = fma(-inw[j] * ps, sp, Qy);
-                Qz = fma(inw[j] * p, ct, Qz);
-                Ein = fma(inw[j], E, Ein);
-            }
-            meas *= k.r[j] * k.r[j] * st;
-            rinv *= rr;
-            k.rE[j] = rr;
-        }
-        const R pc2 = fma(px, px, fma(py, py, pz * pz));
-        const R Ec2 = pc2 + m2c;
-        k.rEc = rsqrt_of(Ec2 > RMath<R>::kTiny ? Ec2 : R(1e-30));
-        k.Ec = Ec2 * k.rEc;
-        cut |= k.Ec < e_cut;
-        bal.add(sgn_cons * k.Ec);
-        const R dE = bal.value();
-        k.qc = pc2 * (pc2 > RMath<R>::kTiny ? rsqrt_of(pc2) : R(0)) * a;
-        // Gaussian and, for the adjoint, 1/sigma^2 and the derivative of
-        // log(1/sigma) with exp(-dE^2 / 2 sigma^2) through sigma(E_k)
-        R gs, inv_sig2;
-        if (frac) {
-            Esum += k.Ec;
-            const R iS = RMath<R>::rcp_(Esum);
-            const R x = dE * iS;
-            gs = exp2_of(gauss_k * x * x) * (R(2) * e_obs * iS);
-            inv_sig2 = four_over_w2 * iS * iS;
-            // d log g / d E_k from sigma: (dE^2 / sigma^2 - 1) / S for every leg
-            k.sig_term = fma(dE * dE, inv_sig2, R(-1)) * iS;
-        } else {
-            gs = exp2_of(gauss_k * dE * dE);
-            inv_sig2 = inv_sig2_abs;
-            k.sig_term = R(0);
-        }
-        R base = meas * rinv * k.rEc * gs;
-        base = (cut || !valid) ? R(0) : base;
-        k.me_d = R(0);          // d log P / d E_k of every initial leg: P'(s) / P(s) 2 E_in
-        if (me_on) {
-            const R qx = fma(cons_inw, px, Qx), qy = fma(cons_inw, py, Qy), qz = fma(cons_inw, pz, Qz);
-            const R e = fma(cons_inw, k.Ec, Ein);
-            const R sv = fma(e, e, -fma(qx, qx, fma(qy, qy, qz * qz)));
-            const R Pv = fma(fma(fma(mec[3], sv, mec[2]), sv, mec[1]), sv, mec[0]);
-            const R dP = fma(fma(R(3) * mec[3], sv, R(2) * mec[2]), sv, mec[1]);
-            k.me_d = Pv != R(0) ? R(2) * e * dP * RMath<R>::rcp_(Pv) : R(0);
-            base *= Pv;
-        }
-        k.base = base;
-        k.dEs = dE * inv_sig2;
-    };
     if constexpr (F32) {
         for (int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
             const int64_t grp = static_cast<int64_t>(gb) + lane;
@@ -476,33 +387,103 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     const uint64_t m = static_cast<uint64_t>(uw[sgi * D + d]) * static_cast<uint32_t>(nb);
-                    const uint32_t b = static_cast<uint32_t>(m >> 32);
+                    const int b = static_cast<int>(m >> 32);
                     const R fr = static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f;
                     const Real2<R> e = s_map[d * nb + b];
                     y[d] = fma(e.dy, fr, e.y0);
                     jac *= e.dy;
                 }
-                Kin k;
-                kinematics(y, jac, valid, k);
-                const bool keep = k.base != R(0);
+                R px = R(0), py = R(0), pz = pobs_sig;
+                EBal<R> bal(sgn_obs_E);
+                R Esum = e_obs;
+                R Qx = R(0), Qy = R(0), Qz = obs_in_p, Ein = obs_in_E;
+                R meas = jac;
+                R rinv = R(1);
+                bool cut = obs_cut;
+                R r[NI], rE[NI];
+#pragma unroll
+                for (int j = 0; j < NI; ++j) {
+                    r[j] = y[3 * j];
+                    R st, ct, sp, cp;
+                    RMath<R>::sincos_(y[3 * j + 1], &st, &ct);
+                    RMath<R>::sincos_(y[3 * j + 2], &sp, &cp);
+                    const R p = r[j] * inv_a;
+                    const R ps = p * st;
+                    px = fma(-sig[j] * ps, cp, px);
+                    py = fma(-sig[j] * ps, sp, py);
+                    pz = fma(sig[j] * p, ct, pz);
+                    const R E2 = fma(p, p, m2[j]);
+                    const R rr = RMath<R>::rsqrt_(E2);
+                    const R E = E2 * rr;
+                    cut |= E < e_cut;
+                    bal.add(sgnE[j] * E);
+                    Esum += E;
+                    if (me_on) {
+                        Qx = fma(-inw[j] * ps, cp, Qx);
+                        Qy = fma(-inw[j] * ps, sp, Qy);
+                        Qz = fma(inw[j] * p, ct, Qz);
+                        Ein = fma(inw[j], E, Ein);
+                    }
+                    meas *= r[j] * r[j] * st;
+                    rinv *= rr;
+                    rE[j] = rr;
+                }
+                const R pc2 = fma(px, px, fma(py, py, pz * pz));
+                const R Ec2 = pc2 + m2c;
+                const R rEc = RMath<R>::rsqrt_(Ec2 > RMath<R>::kTiny ? Ec2 : R(1e-30));
+                const R Ec = Ec2 * rEc;
+                cut |= Ec < e_cut;
+                bal.add(sgn_cons * Ec);
+                const R dE = bal.value();
+                const R qc = pc2 * (pc2 > RMath<R>::kTiny ? RMath<R>::rsqrt_(pc2) : R(0)) * a;
+                // Gaussian and, for the adjoint, 1/sigma^2 and the derivative of
+                // log(1/sigma) with exp(-dE^2 / 2 sigma^2) through sigma(E_k)
+                R gs, inv_sig2, sig_term;
+                if (frac) {
+                    Esum += Ec;
+                    const R iS = RMath<R>::rcp_(Esum);
+                    const R x = dE * iS;
+                    gs = RMath<R>::exp2_(gauss_k * x * x) * (R(2) * e_obs * iS);
+                    inv_sig2 = four_over_w2 * iS * iS;
+                    // d log g / d E_k from sigma: (dE^2 / sigma^2 - 1) / S for every leg
+                    sig_term = fma(dE * dE, inv_sig2, R(-1)) * iS;
+                } else {
+                    gs = RMath<R>::exp2_(gauss_k * dE * dE);
+                    inv_sig2 = inv_sig2_abs;
+                    sig_term = R(0);
+                }
+                R base = meas * rinv * rEc * gs;
+                base = (cut || !valid) ? R(0) : base;
+                R me_d = R(0);          // d log P / d E_k of every initial leg: P'(s) / P(s) 2 E_in
+                if (me_on) {
+                    const R qx = fma(cons_inw, px, Qx), qy = fma(cons_inw, py, Qy), qz = fma(cons_inw, pz, Qz);
+                    const R e = fma(cons_inw, Ec, Ein);
+                    const R sv = fma(e, e, -fma(qx, qx, fma(qy, qy, qz * qz)));
+                    const R Pv = fma(fma(fma(mec[3], sv, mec[2]), sv, mec[1]), sv, mec[0]);
+                    const R dP = fma(fma(R(3) * mec[3], sv, R(2) * mec[2]), sv, mec[1]);
+                    me_d = Pv != R(0) ? R(2) * e * dP * RMath<R>::rcp_(Pv) : R(0);
+                    base *= Pv;
+                }
+                const R dEs = dE * inv_sig2;
+                const bool keep = base != R(0);
                 const uint32_t vote = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
-                    q[slot] = k.base;
+                    q[slot] = base;
 #pragma unroll
-                    for (int j = 0; j < NI; ++j) q[(1 + j) * kQueueSlots + slot] = k.r[j];
+                    for (int j = 0; j < NI; ++j) q[(1 + j) * kQueueSlots + slot] = r[j];
                     if constexpr (JVP) {
-                        q[(1 + NI) * kQueueSlots + slot] = k.qc;
-                        q[(2 + NI) * kQueueSlots + slot] = k.Ec;
+                        q[(1 + NI) * kQueueSlots + slot] = qc;
+                        q[(2 + NI) * kQueueSlots + slot] = Ec;
                     } else {
 #pragma unroll
-                        for (int j = 0; j < NI; ++j) q[(1 + NI + j) * kQueueSlots + slot] = k.rE[j];
-                        q[(1 + 2 * NI) * kQueueSlots + slot] = k.qc;
-                        q[(2 + 2 * NI) * kQueueSlots + slot] = k.Ec;
-                        q[(3 + 2 * NI) * kQueueSlots + slot] = k.rEc;
-                        q[(4 + 2 * NI) * kQueueSlots + slot] = k.dEs;
-                        q[(5 + 2 * NI) * kQueueSlots + slot] = k.sig_term;
-                        q[(6 + 2 * NI) * kQueueSlots + slot] = k.me_d;
+                        for (int j = 0; j < NI; ++j) q[(1 + NI + j) * kQueueSlots + slot] = rE[j];
+                        q[(1 + 2 * NI) * kQueueSlots + slot] = qc;
+                        q[(2 + 2 * NI) * kQueueSlots + slot] = Ec;
+                        q[(3 + 2 * NI) * kQueueSlots + slot] = rEc;
+                        q[(4 + 2 * NI) * kQueueSlots + slot] = dEs;
+                        q[(5 + 2 * NI) * kQueueSlots + slot] = sig_term;
+                        q[(6 + 2 * NI) * kQueueSlots + slot] = me_d;
                     }
                 }
                 qn += __popc(vote);
@@ -522,6 +503,85 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
         __syncwarp();
         if (lane < qn) drain(lane);
     } else {
+        // Kinematic part of one sample at the mapped point y with map Jacobian jac
+        // (kin_at of the sample kernel, plus what the derivatives need).
+        struct Kin {
+            R base, r[NI], rE[NI], qc, Ec, rEc, dEs, sig_term, me_d;
+        };
+        auto kinematics = [&](const R* y, R jac, bool valid, Kin& k) {
+            R px = R(0), py = R(0), pz = pobs_sig;
+            EBal<R> bal(sgn_obs_E);
+            R Esum = e_obs;
+            R Qx = R(0), Qy = R(0), Qz = obs_in_p, Ein = obs_in_E;
+            R meas = jac;
+            R rinv = R(1);
+            bool cut = obs_cut;
+#pragma unroll
+            for (int j = 0; j < NI; ++j) {
+                k.r[j] = y[3 * j];
+                R st, ct, sp, cp;
+                sincos_table(y[3 * j + 1], tab, &st, &ct);
+                sincos_table(y[3 * j + 2], tab, &sp, &cp);
+                const R p = k.r[j] * inv_a;
+                const R ps = p * st;
+                px = fma(-sig[j] * ps, cp, px);
+                py = fma(-sig[j] * ps, sp, py);
+                pz = fma(sig[j] * p, ct, pz);
+                const R E2 = fma(p, p, m2[j]);
+                const R rr = rsqrt_halley(E2);
+                const R E = E2 * rr;
+                cut |= E < e_cut;
+                bal.add(sgnE[j] * E);
+                Esum += E;
+                if (me_on) {
+                    Qx = fma(-inw[j] * ps, cp, Qx);
+                    Qy = fma(-inw[j] * ps, sp, Qy);
+                    Qz = fma(inw[j] * p, ct, Qz);
+                    Ein = fma(inw[j], E, Ein);
+                }
+                meas *= k.r[j] * k.r[j] * st;
+                rinv *= rr;
+                k.rE[j] = rr;
+            }
+            const R pc2 = fma(px, px, fma(py, py, pz * pz));
+            const R Ec2 = pc2 + m2c;
+            k.rEc = rsqrt_halley(Ec2 > RMath<R>::kTiny ? Ec2 : R(1e-30));
+            k.Ec = Ec2 * k.rEc;
+            cut |= k.Ec < e_cut;
+            bal.add(sgn_cons * k.Ec);
+            const R dE = bal.value();
+            k.qc = pc2 * (pc2 > RMath<R>::kTiny ? rsqrt_halley(pc2) : R(0)) * a;
+            // Gaussian and, for the adjoint, 1/sigma^2 and the derivative of
+            // log(1/sigma) with exp(-dE^2 / 2 sigma^2) through sigma(E_k)
+            R gs, inv_sig2;
+            if (frac) {
+                Esum += k.Ec;
+                const R iS = RMath<R>::rcp_(Esum);
+                const R x = dE * iS;
+                gs = exp2_table(gauss_k * x * x, tab) * (R(2) * e_obs * iS);
+                inv_sig2 = four_over_w2 * iS * iS;
+                // d log g / d E_k from sigma: (dE^2 / sigma^2 - 1) / S for every leg
+                k.sig_term = fma(dE * dE, inv_sig2, R(-1)) * iS;
+            } else {
+                gs = exp2_table(gauss_k * dE * dE, tab);
+                inv_sig2 = inv_sig2_abs;
+                k.sig_term = R(0);
+            }
+            R base = meas * rinv * k.rEc * gs;
+            base = (cut || !valid) ? R(0) : base;
+            k.me_d = R(0);          // d log P / d E_k of every initial leg: P'(s) / P(s) 2 E_in
+            if (me_on) {
+                const R qx = fma(cons_inw, px, Qx), qy = fma(cons_inw, py, Qy), qz = fma(cons_inw, pz, Qz);
+                const R e = fma(cons_inw, k.Ec, Ein);
+                const R sv = fma(e, e, -fma(qx, qx, fma(qy, qy, qz * qz)));
+                const R Pv = fma(fma(fma(mec[3], sv, mec[2]), sv, mec[1]), sv, mec[0]);
+                const R dP = fma(fma(R(3) * mec[3], sv, R(2) * mec[2]), sv, mec[1]);
+                k.me_d = Pv != R(0) ? R(2) * e * dP * RMath<R>::rcp_(Pv) : R(0);
+                base *= Pv;
+            }
+            k.base = base;
+            k.dEs = dE * inv_sig2;
+        };
         // FP64: the screen of the FP64 sample loop (eval_f64q.cuh) queues the
         // samples' Philox words, and 32 queued samples at a time are evaluated.
         // It drops exact zeros and samples whose kinematic part is 2^-300 of the
