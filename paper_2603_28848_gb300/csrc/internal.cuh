@@ -542,7 +542,7 @@ constexpr int kMaxVariants = 12;
 // those of the instantiation's largest process otherwise.  The FP64 variant
 // with the FP32 screen (spl 2) adds its function tables, the segment's
 // constants and the FP32 map table.
-constexpr int kMathDoubles = 3 * 129 + 32 + 1;     // math_table.cuh, rounded up to 16 bytes
+constexpr int kMathDoubles = 5 * 129 + 2 * 32 + 1; // math_table.cuh, rounded up to 16 bytes
 constexpr int kSetupBytes = 768;
 inline size_t sample_smem_bytes(bool f32, int n_grid, int n_species, int nbins_max, int nmax, bool ext, bool any_strat,
                                 int threads, int spl) {

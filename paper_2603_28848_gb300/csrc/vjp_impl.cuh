@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(kThreads, 2) vjp_kernel(VjpParams V) {
         s_map32 = reinterpret_cast<Real2<float>*>(s_tab + kMathDoubles);
         s_queue = reinterpret_cast<float*>(s_map32 + map_elems);
         if (V.screen) {
-            for (int k = threadIdx.x; k < 3 * kTrigEntries + kExpEntries; k += blockDim.x) s_tab[k] = kMathTable[k];
+            for (int k = threadIdx.x; k < kMathEntries; k += blockDim.x) s_tab[k] = kMathTable[k];
             tab = s_tab;
         }
     }
