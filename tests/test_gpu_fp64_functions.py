@@ -44,6 +44,18 @@ extern "C" int test_function(int n, int which, int library, const void* x, void*
     function_kernel<<<(n + 255) / 256, 256>>>(n, which, library, (const double*)x, (double*)out);
     return cudaDeviceSynchronize();
 }
+
+__global__ void product_kernel(int n, int m, const double* x, double* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    Product p(x[i * m]);
+    for (int k = 1; k < m; ++k) p.mul_f(x[i * m + k]);
+    out[i] = p.rare ? -1.0 : p.value();
+}
+extern "C" int test_product(int n, int m, const void* x, void* out) {
+    product_kernel<<<(n + 255) / 256, 256>>>(n, m, (const double*)x, (double*)out);
+    return cudaDeviceSynchronize();
+}
 """
 
 
@@ -125,3 +137,38 @@ def test_elementary_functions(lib, which, name, lo, hi, log):
     (rms, top), (lrms, _) = err
     assert rms <= 0.36 and top <= 2.0
     assert rms <= 1.15 * lrms
+
+
+def test_product(lib):
+    """Products of 12 factors against exact ones: half a unit of the last place
+    and 12 roundings of 2^-62 (2^-5 of a unit together), one more rounding where
+    the result is subnormal; a factor that is not a normal number is told."""
+    from fractions import Fraction
+    import torch
+    rng = np.random.RandomState(3)
+    m = 12
+    rows = [rng.uniform(-2.0, 2.0, (400, m)), np.exp(rng.uniform(-60, 60, (400, m)))]
+    far = np.exp(rng.uniform(-2, 2, (4, m)))            # over and under the range on the way
+    far[:, 1], far[:, 2], far[:, 3], far[:, 4] = 1e300, 1e300, 1e-300, [1e-290, 1e-300, 1e300, 1e-200]
+    sub = np.exp(rng.uniform(-2, 2, (50, m)))
+    sub[:, 1], sub[:, 2] = 1e-200, 1e-115
+    x = np.concatenate(rows + [far, sub])
+    special = np.exp(rng.uniform(-2, 2, (5, m)))
+    special[np.arange(5), [0, 3, 5, 7, 11]] = np.inf, np.inf, np.nan, 1e-310, -np.inf
+    x[0, 4] = x[1, 0] = 0.0
+    out = torch.zeros(len(x) + 5, dtype=torch.float64, device="cuda")
+    X = _dev(np.concatenate([x, special]))
+    assert lib.test_product(len(x) + 5, m, _ptr(X), _ptr(out)) == 0
+    got = out.cpu().numpy()
+    assert np.all(got[len(x):] == -1.0)
+    big = Fraction(np.finfo(np.float64).max)
+    for row, v in zip(x, got):
+        want = Fraction(1)
+        for f in row:
+            want *= Fraction(float(f))
+        if abs(want) > big:
+            assert np.isinf(v) and (v > 0) == (want > 0)
+            continue
+        unit = Fraction(float(np.spacing(abs(float(want)))))
+        low = abs(want) < Fraction(2.0 ** -1022)
+        assert abs(Fraction(float(v)) - want) <= unit * (Fraction(17, 32) + (Fraction(1, 2) if low else 0))

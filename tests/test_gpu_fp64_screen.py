@@ -91,3 +91,31 @@ def test_narrow_width_on_a_wide_grid():
     ok = np.isfinite(om)
     assert ok.mean() > 0.8 and np.any(om != 0)
     assert np.all(np.abs(mean - om)[ok] <= (1e-6 * np.abs(om) + 1e-300)[ok])
+
+
+def test_factors_that_are_not_normal_numbers():
+    """A species whose values are partly subnormal (below 2.2e-308) next to one of
+    order one: in a gain task that observes it, c0 is up to 2^100 and the weights
+    are normal numbers.  The spline's cubic coefficient is a multiple of 5e-324 and
+    enters with the interval's length cubed, 13^3: 2e-12 of the smallest value,
+    1e-10 of a task's mean with room for a handful of such roundings.  (In the
+    other tasks the weights themselves are subnormal.)"""
+    import torch
+    from paper_2603_28848_gb300 import Collision
+    prob, f0, t = _mb(8, 2000, sigma_E=0.5)
+    q = W.grid_points(prob.grid)
+    E = np.sqrt(q * q + 1.0)
+    proc = replace(prob.processes[0], species_in=(0, 1), species_out=(0, 1), coupling=1e10)
+    prob = replace(prob, species=(prob.species[0], prob.species[0]), processes=(proc,))
+    f0 = np.stack([f0[0], 4e-308 * np.exp(-(E - 1.0) / 10.5)])
+    assert f0[1].min() > 5.7e-309
+    col = Collision(prob, W.PREC_FP64)
+    assert col.launch_shape()[2] == 2
+    col.eval(torch.tensor(f0, device="cuda"), t)
+    mean, _ = col.task_results()
+    col.close()
+    _, _, detail, _ = oracle_sweep(prob, f0, t, "f64")
+    om, _ = task_arrays(detail, len(mean))
+    gain = slice(16, 32, 2)                    # the second side integral's, which observes that species
+    assert np.all(om[gain] > 0)
+    assert np.all(np.abs(mean - om)[gain] <= 1e-10 * om[gain])
