@@ -469,8 +469,9 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
     }
     SegSetup<float, NLEG> s32;
     seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
-    // what the largest weight's exponent is lowered by: the bound leaves c0 out
-    const float below = lg2_ftz(fmaxf(static_cast<float>(tc.c0), 1e-37f)) + kDropBits +
+    // what the largest weight's exponent is lowered by: the bound leaves |c0| out
+    // (c0 < 0: a Fermi-Dirac gain task observed where f > 1)
+    const float below = lg2_ftz(fmaxf(fabsf(static_cast<float>(tc.c0)), 1e-37f)) + kDropBits +
                         static_cast<float>(64 - __clzll(static_cast<long long>(td.neval)));
     __syncthreads();
     const SegConst<double, NLEG>& C = s_setup->C;

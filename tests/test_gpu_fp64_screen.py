@@ -119,3 +119,30 @@ def test_factors_that_are_not_normal_numbers():
     gain = slice(16, 32, 2)                    # the second side integral's, which observes that species
     assert np.all(om[gain] > 0)
     assert np.all(np.abs(mean - om)[gain] <= 1e-10 * om[gain])
+
+
+def _against_oracle(prob, f0, t):
+    import torch
+    from paper_2603_28848_gb300 import Collision
+    col = Collision(prob, W.PREC_FP64)
+    assert col.launch_shape()[2] == 2
+    col.eval(torch.tensor(f0, device="cuda"), t)
+    mean, err = col.task_results()
+    col.close()
+    _, _, detail, _ = oracle_sweep(prob, f0, t, "f64")
+    om, oe = task_arrays(detail, len(mean))
+    assert np.all(np.isfinite(om)) and np.any(om != 0)
+    assert np.all(np.abs(mean - om) <= 1e-7 * np.abs(om) + 1e-300)
+    assert np.all(np.abs(err - oe) <= 1e-6 * np.abs(oe) + 1e-300)
+    return om
+
+
+def test_negative_observed_factor():
+    """Fermi-Dirac values above 1 inside the grid: the observed leg's 1 - f, and
+    every weight of that gain task, is negative."""
+    prob, f0, t = _mb(12, 20_000, sigma_E=0.1)
+    prob = replace(prob, species=(replace(prob.species[0], stat=W.STAT_FD),))
+    f0 = np.where((np.arange(12) >= 4) & (np.arange(12) < 8), 1.2, 1.6 * f0)
+    assert f0[:, :4].max() < 1 and f0[:, 8:].max() < 1
+    om = _against_oracle(prob, f0, t)
+    assert np.all(om[8:16:2] < 0)
