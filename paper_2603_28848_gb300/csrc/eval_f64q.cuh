@@ -166,11 +166,19 @@ __device__ __forceinline__ bool less_pos(double a, double b) {
 }
 
 // Cubic spline value at comoving q inside [q_0, q_{n-1}], the interval from
-// FP32 (a guess within one interval, as in spline_eval).
+// FP32 (a guess within one interval, as in spline_eval).  On an evenly spaced
+// grid the distance from q_0 is taken in FP64 first, as there: a grid far from
+// zero is narrower than FP32 resolves.
 __device__ __forceinline__ double spline64(const double* coef, const double* knots, double q, const Geometry& g,
-                                           float inv_step, float q0, float lq0_step) {
-    const float qf = trunc_f32(q);
-    int j = static_cast<int>(g.log_spaced ? fmaf(lg2_ftz(qf), inv_step, -lq0_step) : (qf - q0) * inv_step);
+                                           float inv_step, double q0, float lq0_step) {
+    float x;
+    if (g.log_spaced) {
+        x = fmaf(lg2_ftz(trunc_f32(q)), inv_step, -lq0_step);
+    } else {
+        const double d = q - q0;
+        x = static_cast<uint32_t>(__double2hiint(d)) < 0x38100000u ? 0.0f : trunc_f32(d) * inv_step;   // (below 2^-126: 0)
+    }
+    int j = static_cast<int>(x);
     j = min(max(j, 0), g.n_grid - 2);
     const double t = q - knots[j];
     const double2* cp = reinterpret_cast<const double2*>(coef) + 2 * j;
@@ -221,7 +229,7 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
         w.mul(st);
         w.mul(rE);
         if (C.cb[j] != 0.0) {                       // (0: 1 + eta f of a Maxwell-Boltzmann leg, 1)
-            double f = spline64(s_spline + C.spc[j] * ncoef, knots, r, g, s32.inv_step, s32.q0, s32.lq0_step);
+            double f = spline64(s_spline + C.spc[j] * ncoef, knots, r, g, s32.inv_step, q0, s32.lq0_step);
             if (C.fd[j]) f = f < 1.0 ? f : 1.0;
             w.mul_f(C.ca[j] != 0.0 ? fma(C.cb[j], f, C.ca[j]) : f);
         }
@@ -266,7 +274,7 @@ __device__ __forceinline__ double weight64(const SegConst<double, NLEG>& C, cons
         double fc;
         const bool below = less_pos(qc, q0), above = less_pos(qN, qc);
         if (!below && !above) {
-            fc = spline64(s_spline + C.sp_cons * ncoef, knots, qc, g, s32.inv_step, s32.q0, s32.lq0_step);
+            fc = spline64(s_spline + C.sp_cons * ncoef, knots, qc, g, s32.inv_step, q0, s32.lq0_step);
         } else {
             const double x = below ? C.tlo_a + C.tlo_b * Ec : C.thi_a + C.thi_b * Ec;
             const double den = C.eta_c == 1.0 ? expm1(x) : exp(x) - C.eta_c;

@@ -146,3 +146,15 @@ def test_negative_observed_factor():
     assert f0[:, :4].max() < 1 and f0[:, 8:].max() < 1
     om = _against_oracle(prob, f0, t)
     assert np.all(om[8:16:2] < 0)
+
+
+def test_narrow_linear_grid():
+    """An evenly spaced grid of 11 FP32 numbers per interval, values alternating
+    from knot to knot: a lookup that takes a neighbouring interval's cubic a tenth
+    of an interval outside is 1e-3 off.  FP64 resolves 1e-10 of an interval.  (Two
+    equal values at each end: flat tails.)"""
+    prob, f0, t = _mb(16, 5000, sigma_E=0.5)
+    prob = replace(prob, grid=W.Grid(16, 1.0, 1.0 + 2e-5, False), tail_points=2)
+    f0 = (1.0 + 0.5 * (-1.0) ** np.arange(16))[None, :]
+    f0[:, [0, -1]] = f0[:, [1, -2]]
+    _against_oracle(prob, f0, t)
