@@ -347,7 +347,8 @@ __device__ __forceinline__ float map_point32(uint32_t x0, uint32_t x1, int nb, c
 }
 
 // log2 of an upper bound of |ca + cb f| at comoving q inside the grid: the FP32
-// spline value plus its rounding bound (2^-18 of its terms' magnitudes).
+// spline value plus its rounding bound (2^-18 of its terms' magnitudes); +inf
+// where FP32 coefficients overflowed (their sum is then infinite or a NaN).
 __device__ __forceinline__ float log2_factor_bound(const float* coef, const float* knots, float q, const Geometry& g,
                                                    float inv_step, float q0, float lq0_step, float ca) {
     int j = static_cast<int>(g.log_spaced ? fmaf(lg2_ftz(q), inv_step, -lq0_step) : (q - q0) * inv_step);
@@ -357,6 +358,7 @@ __device__ __forceinline__ float log2_factor_bound(const float* coef, const floa
     const float f = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);
     const float at = fabsf(t);
     const float size = fmaf(fmaf(fmaf(fabsf(c.w), at, fabsf(c.z)), at, fabsf(c.y)), at, fabsf(c.x));
+    if (!(size < 1e37f)) return __int_as_float(0x7f800000);                    // (f is a NaN only if size is not finite)
     return lg2_ftz(fmaxf(ca + fmaxf(f, 0.0f) + 3.8e-6f * size, 1e-36f));       // (FP32 subnormals flush to 0)
 }
 

@@ -158,3 +158,18 @@ def test_narrow_linear_grid():
     f0 = (1.0 + 0.5 * (-1.0) ** np.arange(16))[None, :]
     f0[:, [0, -1]] = f0[:, [1, -2]]
     _against_oracle(prob, f0, t)
+
+
+def test_spline_coefficients_beyond_fp32():
+    """A species whose values alternate by 1e25 on a grid of 56 FP32 numbers per
+    interval: its cubic coefficients (f over the interval cubed, 1e40) are infinite
+    in FP32, and the screen's spline value is a NaN where the lookup falls on a
+    knot, in about 1% of the samples.  Small equal values at the ends, so that the
+    conserved leg's tail is no reason to keep them."""
+    prob, f0, t = _mb(16, 20_000, sigma_E=0.5)
+    proc = replace(prob.processes[0], species_in=(0, 1), species_out=(0, 1))
+    prob = replace(prob, grid=W.Grid(16, 1.0, 1.0 + 1e-4, False), tail_points=2,
+                   species=(prob.species[0], prob.species[0]), processes=(proc,))
+    f0 = np.stack([1e25 * (1.0 + 0.5 * (-1.0) ** np.arange(16)), np.full(16, 0.2)])
+    f0[0, [0, 1, -2, -1]] = 0.1
+    _against_oracle(prob, f0, t)
