@@ -335,16 +335,21 @@ __device__ __noinline__ double plain_weight64(const uint32_t* q, int nb, const R
                                           S->lq0_step, S->qN, ncoef);
 }
 
-// The same in FP32 from the uniform's first 32 bits (an increment's edge may
-// fall to its neighbour: the mapped point is continuous there).  Returns the
-// increment's width.
-__device__ __forceinline__ float map_point32(uint32_t x0, uint32_t x1, int nb, const Real2<float>* table, float* y) {
+// The same in FP32 from the uniform's first 32 bits.  The 20 bits left out, and
+// FP64's rounding, can take the point over an increment's edge: the mapped point
+// is continuous there, the increment's width is not.  frac becomes the largest
+// fraction seen, near_edge says whether any may have crossed (nb 2^-32 of the
+// samples per dimension).  Returns the increment's width.
+__device__ __forceinline__ float map_point32(uint32_t x0, uint32_t x1, int nb, const Real2<float>* table, float* y,
+                                             uint32_t* frac) {
     const uint32_t x = (x0 & ~63u) | (x1 >> 26);
     const uint64_t m = static_cast<uint64_t>(x) * static_cast<uint32_t>(nb);
     const Real2<float> e = table[static_cast<uint32_t>(m >> 32)];
+    *frac = max(*frac, static_cast<uint32_t>(m));
     *y = fmaf(e.dy, static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f, e.y0);
     return e.dy;
 }
+__device__ __forceinline__ bool near_edge(uint32_t frac, int nb) { return frac >= 0u - static_cast<uint32_t>(nb); }
 
 // log2 of an upper bound of |ca + cb f| at comoving q inside the grid: the FP32
 // spline value plus its rounding bound (2^-18 of its terms' magnitudes); +inf
@@ -535,12 +540,13 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
         for (int sgi = 0; sgi < G; ++sgi) {
             const bool valid = grp < g1 && grp * G + sgi < N;
             float y[D], jac = 1.0f;
+            uint32_t frac = 0;
 #pragma unroll
             for (int d = 0; d < D; ++d)
-                jac *= map_point32(uw[2 * (sgi * D + d)], uw[2 * (sgi * D + d) + 1], nb, s_map32 + d * nb, &y[d]);
+                jac *= map_point32(uw[2 * (sgi * D + d)], uw[2 * (sgi * D + d) + 1], nb, s_map32 + d * nb, &y[d], &frac);
             float gauss;
             const float l = log2_weight_bound<NLEG, true>(s32, P, y, jac, &gauss);
-            const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
+            const bool keep = valid && !(gauss < -1100.0f) && (near_edge(frac, nb) || !(l < cutoff));
             const uint32_t vote = __ballot_sync(0xffffffffu, keep);
             if (keep) {
                 const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32

@@ -625,10 +625,12 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                     continue;
                 }
                 float y[D], jac = 1.0f, gauss;
+                uint32_t frac = 0;
 #pragma unroll
-                for (int d = 0; d < D; ++d) jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d]);
+                for (int d = 0; d < D; ++d)
+                    jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
                 const float l = log2_weight_bound<NLEG, false>(s32, P, y, jac, &gauss);
-                const bool keep = valid && !(gauss < -1100.0f) && !(l < cutoff);
+                const bool keep = valid && !(gauss < -1100.0f) && (near_edge(frac, nb) || !(l < cutoff));
                 const uint32_t vote = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32

@@ -25,6 +25,22 @@ extern "C" int test_map(int n, const void* x0, const void* x1, int nb, void* fr,
     return cudaDeviceSynchronize();
 }
 
+__global__ void edge_kernel(int n, const uint32_t* x0, const uint32_t* x1, int nb, uint32_t* bin, uint32_t* edge) {
+    __shared__ Real2<float> table[256];
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) table[k] = Real2<float>{0.0f, (float)k};
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float y;
+    uint32_t frac = 0;
+    bin[i] = (uint32_t)map_point32(x0[i], x1[i], nb, table, &y, &frac);
+    edge[i] = near_edge(frac, nb);
+}
+extern "C" int test_edge(int n, const void* x0, const void* x1, int nb, void* bin, void* edge) {
+    edge_kernel<<<(n + 255) / 256, 256>>>(n, (const uint32_t*)x0, (const uint32_t*)x1, nb, (uint32_t*)bin, (uint32_t*)edge);
+    return cudaDeviceSynchronize();
+}
+
 // which 0: 1/sqrt, 1: sin, 2: cos, 3: 2^x; library: CUDA's function
 __global__ void function_kernel(int n, int which, int library, const double* x, double* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -80,6 +96,33 @@ def _ptr(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _words(k, rng):
+    """Philox words of the 52-bit integers k (the bits the stream drops at random)."""
+    k = k.astype(np.uint64)
+    x0 = (k >> np.uint64(26) << np.uint64(6)).astype(np.uint32) | rng.randint(0, 64, k.size).astype(np.uint32)
+    x1 = ((k & np.uint64(2 ** 26 - 1)) << np.uint64(6)).astype(np.uint32) | rng.randint(0, 64, k.size).astype(np.uint32)
+    return _dev(x0.view(np.int32)), _dev(x1.view(np.int32))
+
+
+@pytest.mark.parametrize("nb", [2, 3, 17, 50, 64, 255, 256])
+def test_increment_of_the_screen(lib, nb):
+    """Wherever 32 bits give another increment than 52 (within 2^-32 of an edge),
+    the screen is told; in all it is told for at most nb 2^-31 of the points."""
+    import torch
+    rng = np.random.RandomState(nb)
+    edge = ((np.arange(nb + 1, dtype=object) << 52) // nb).astype(np.int64)
+    near = (edge[:, None] + np.concatenate([-(2 ** np.arange(21)), [0], 2 ** np.arange(21)])).reshape(-1)
+    k = np.concatenate([np.clip(near, 0, 2 ** 52 - 1), rng.randint(0, 2 ** 52, 100_000)])
+    a, b = _words(k, rng)
+    bins, told = (torch.zeros(k.size, dtype=torch.int32, device="cuda") for _ in range(2))
+    assert lib.test_edge(k.size, _ptr(a), _ptr(b), nb, _ptr(bins), _ptr(told)) == 0
+    t = (k.astype(np.float64) + 0.5) * 2.0 ** -52 * nb
+    other = bins.cpu().numpy() != np.minimum(t.astype(np.int64), nb - 1)
+    told = told.cpu().numpy() != 0
+    assert np.any(other) == (nb not in (2, 64, 256)) and np.all(told[other])
+    assert told[near.size:].sum() <= 3         # (256 2^-31 1e5 = 0.012 expected)
+
+
 @pytest.mark.parametrize("nb", [2, 3, 17, 50, 64, 255, 256])
 def test_map_point(lib, nb):
     """Increment and fraction of u nb in FP64, bit for bit (the published
@@ -89,11 +132,9 @@ def test_map_point(lib, nb):
     edge = (np.arange(nb, dtype=np.uint64) << np.uint64(52)) // np.uint64(nb)
     k = np.concatenate([rng.randint(0, 2 ** 52, 20_000).astype(np.uint64), edge, edge + np.uint64(1),
                         edge[1:] - np.uint64(1), np.array([0, 2 ** 52 - 1, 2 ** 51], dtype=np.uint64)])
-    x0 = (k >> np.uint64(26) << np.uint64(6)).astype(np.uint32) | rng.randint(0, 64, k.size).astype(np.uint32)
-    x1 = ((k & np.uint64(2 ** 26 - 1)) << np.uint64(6)).astype(np.uint32) | rng.randint(0, 64, k.size).astype(np.uint32)
+    a, b = _words(k, rng)
     fr = torch.zeros(k.size, dtype=torch.float64, device="cuda")
     bins = torch.zeros(k.size, dtype=torch.int32, device="cuda")
-    a, b = _dev(x0.view(np.int32)), _dev(x1.view(np.int32))
     assert lib.test_map(k.size, _ptr(a), _ptr(b), nb, _ptr(fr), _ptr(bins)) == 0
     t = (k.astype(np.float64) + 0.5) * 2.0 ** -52 * nb
     want = np.minimum(t.astype(np.int64), nb - 1)
