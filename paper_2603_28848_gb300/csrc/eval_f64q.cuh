@@ -413,7 +413,7 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     prod *= rEc;
     const float err = fmaf(4e-5f, Esum, 1e-6f * S.qN * C.inv_a);
     float d = fmaxf(fabsf(bal) - err, 0.0f);
-    if (!(Esum < 1e30f)) d = 0.0f;                       // (overflowed, or not a number)
+    if (!(Esum < 1e30f && C.gauss_k > -1e37f)) d = 0.0f; // (overflowed, or not a number: no bound)
     float extra = 0.0f;
     if (C.frac) {
         const float iS = __fdividef(1.0f, Esum);

@@ -173,3 +173,13 @@ def test_spline_coefficients_beyond_fp32():
     f0 = np.stack([1e25 * (1.0 + 0.5 * (-1.0) ** np.arange(16)), np.full(16, 0.2)])
     f0[0, [0, 1, -2, -1]] = 0.1
     _against_oracle(prob, f0, t)
+
+
+def test_small_units():
+    """Energies of 1e-18 and a width of 1e-20, whose inverse square FP32 does not
+    hold: the Gaussian is no reason to drop a sample then."""
+    prob, f0, t = _mb(8, 5000, sigma_E=1e-20)
+    prob = replace(prob, grid=replace(prob.grid, q_min=1e-20, q_max=2e-17), e_cut=1e-60,
+                   species=(replace(prob.species[0], mass0=1e-18),))
+    om = _against_oracle(prob, f0, t)
+    assert np.all(om > 0)
