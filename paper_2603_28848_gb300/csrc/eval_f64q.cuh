@@ -175,8 +175,8 @@ __device__ __forceinline__ double spline64(const double* coef, const double* kno
     if (g.log_spaced) {
         x = fmaf(lg2_ftz(trunc_f32(q)), inv_step, -lq0_step);
     } else {
-        const double d = q - q0;
-        x = static_cast<uint32_t>(__double2hiint(d)) < 0x38100000u ? 0.0f : trunc_f32(d) * inv_step;   // (below 2^-126: 0)
+        const double d = (q - q0) * g.inv_step;
+        x = static_cast<uint32_t>(__double2hiint(d)) < 0x38100000u ? 0.0f : trunc_f32(d);      // (below 2^-126: 0)
     }
     int j = static_cast<int>(x);
     j = min(max(j, 0), g.n_grid - 2);

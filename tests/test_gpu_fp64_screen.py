@@ -183,3 +183,14 @@ def test_small_units():
                    species=(replace(prob.species[0], mass0=1e-18),))
     om = _against_oracle(prob, f0, t)
     assert np.all(om > 0)
+
+
+@pytest.mark.parametrize("unit", [1e-45, 1e45])
+def test_units_beyond_fp32(unit):
+    """The same problem on an evenly spaced grid in units that FP32 does not hold at
+    all: every sample is kept, and the lookups count in intervals."""
+    prob, f0, t = _mb(8, 1500, sigma_E=0.5 * unit)
+    prob = replace(prob, grid=W.Grid(8, 0.01 * unit, 20.0 * unit, False), e_cut=0.0,
+                   species=(replace(prob.species[0], mass0=unit),))
+    om = _against_oracle(prob, f0, t)
+    assert np.all(om > 0)
