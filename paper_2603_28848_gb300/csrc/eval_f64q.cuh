@@ -375,8 +375,8 @@ __device__ __forceinline__ float log2_factor_bound(const float* coef, const floa
 // within 4e-6 of the momenta plus 1e-6 q_max / a of the four radii, and 4e-5 of
 // the energies' sum plus that covers the balance ten times.  +inf where a
 // factor leaves the normal range (or is not a number) or the conserved leg's
-// energy is not resolved.  STAT false: of the kinematic part alone.
-template <int NLEG, bool STAT>
+// energy is not resolved.  WEIGHT false: gauss alone.
+template <int NLEG, bool WEIGHT>
 __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& S, const EvalParams& P, const float* y,
                                                    float jac, float* gauss) {
     constexpr int NI = NLEG - 2;
@@ -422,9 +422,9 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     }
     const float e = C.gauss_k * d * d;
     *gauss = e;
+    if constexpr (!WEIGHT) return 0.0f;
     if (!(prod > 1e-37f && prod < 1e37f && Ec > 4.0f * err)) return __int_as_float(0x7f800000);
     const float kin = lg2_ftz(prod) + extra + e;
-    if constexpr (!STAT) return kin + 2.0f;
     // the statistical factors, 1 + f or f of every leg (|ca + cb f| is at most ca + f)
     const int ncoef = 4 * (g.n_grid - 1);
     float stat = 0.0f;

@@ -584,17 +584,15 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
         };
         // FP64: the screen of the FP64 sample loop (eval_f64q.cuh) queues the
         // samples' Philox words, and 32 queued samples at a time are evaluated.
-        // It drops exact zeros and samples whose kinematic part is 2^-300 of the
-        // largest this warp has evaluated in the segment: their derivatives,
-        // which miss one statistical factor, stay below the rounding of the
-        // spline's transposed solve by any ratio of statistical factors a grid
-        // in FP64 can hold.  An s-dependent |M|^2 is not in the bound: exact
-        // zeros only.  Without room for the queues every sample is evaluated
-        // where it is drawn.
+        // It drops exact zeros of the Gaussian only: a derivative by f_j misses
+        // f_j's factor and is one output of many, so no sample is small against
+        // all that it goes into.  (With what was 2^-300 of the largest kinematic
+        // part dropped as well: 2 -> 3 reverse, 48 points, 2e4 samples 0.44
+        // instead of 0.46 ms, massless 2 -> 2 forward, 40 points 0.37 instead of
+        // 0.49 ms; C~ was wrong where f falls much faster than the Gaussian.)
+        // Without room for the queues every sample is evaluated where it is drawn.
         constexpr int W = 2 * D;
         uint32_t* qw = reinterpret_cast<uint32_t*>(s_queue) + (tid >> 5) * (W * kQueueSlots);
-        int wmax = 0;
-        float cutoff = -3.0e38f;
         auto sample = [&](const uint32_t* w, int stride, bool valid) {
             R y[D], jac = R(1);
 #pragma unroll
@@ -605,7 +603,6 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
             Kin k;
             kinematics(y, jac, valid, k);
             accumulate(k.base, k.r, k.rE, k.qc, k.Ec, k.rEc, k.dEs, k.sig_term, k.me_d);
-            return __double2hiint(k.base) & 0x7fffffff;
         };
         SegSetup<float, NLEG> s32;
         seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
@@ -624,13 +621,12 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                     sample(uw, 1, valid);
                     continue;
                 }
-                float y[D], jac = 1.0f, gauss;
+                float y[D], gauss;
                 uint32_t frac = 0;
 #pragma unroll
-                for (int d = 0; d < D; ++d)
-                    jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
-                const float l = log2_weight_bound<NLEG, false>(s32, P, y, jac, &gauss);
-                const bool keep = valid && !(gauss < -1100.0f) && (near_edge(frac, nb) || !(l < cutoff));
+                for (int d = 0; d < D; ++d) map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
+                log2_weight_bound<NLEG, false>(s32, P, y, 1.0f, &gauss);
+                const bool keep = valid && !(gauss < -1100.0f);
                 const uint32_t vote = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
@@ -640,12 +636,7 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                 qn += __popc(vote);
                 if (qn >= 32) {
                     __syncwarp();
-                    const int hi = sample(qw + lane, kQueueSlots, true);
-                    const int top = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<unsigned>(hi)));
-                    if (!me_on && top > wmax && top < 0x7FE00000) {
-                        wmax = top;
-                        cutoff = static_cast<float>((top >> 20) - 1023) - 300.0f;
-                    }
+                    sample(qw + lane, kQueueSlots, true);
                     __syncwarp();
                     if (lane < qn - 32) {
 #pragma unroll
