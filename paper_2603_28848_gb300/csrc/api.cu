@@ -1109,7 +1109,8 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
         // Two packed samples per lane (four CTAs per SM) pay once the CTAs run several chunks each;
         // with about one chunk per CTA five CTAs per SM finish sooner.  Sample kernel, one -> packed:
         // MB 2 -> 2 at 1, 2, 10 chunks per CTA 88 -> 84, 153 -> 157, 645 -> 625 us; BE 2 -> 2 at 1, 2.5,
-        // 4, 41 chunks 113 -> 113, 207 -> 198, 319 -> 307, 2957 -> 2779 us.
+        // 4, 41 chunks 113 -> 113, 207 -> 198, 319 -> 307, 2957 -> 2779 us.  From kPackedChunks of them
+        // per CTA on, then; which loop runs does not show in the results.
         int pick = 0, occ = 0;
         for (int v = 1; v < ctx->n_variants; ++v)
             if (ctx->variants[v].first_plan) pick = v;
@@ -1117,7 +1118,7 @@ best_status best_collision_init(const best_config* cfg, best_ctx** out) {
         if (sv != BEST_OK) return bail(sv);
         int64_t W = 0;
         for (const TaskDesc& td : ctx->tasks) W += td.neval * (td.dim + 6);
-        if (pick && W / kMinChunkCost < 4 * static_cast<int64_t>(nsm) * occ) pick = 0;
+        if (pick && W / kMinChunkCost < kPackedChunks * nsm * occ) pick = 0;
         sv = set_variant(ctx, pick);
         if (sv != BEST_OK) return bail(sv);
     }

@@ -535,6 +535,12 @@ struct SampleVariant {
 };
 constexpr int kMaxVariants = 12;
 
+// Chunks per CTA from which an FP32 2 -> 2 context defaults to packed pairs.
+#ifndef BEST_PACKED_CHUNKS
+#define BEST_PACKED_CHUNKS 4
+#endif
+constexpr int64_t kPackedChunks = BEST_PACKED_CHUNKS;
+
 // Dynamic shared memory of a sample-kernel variant, in the kernel's layout:
 // spline tables of all species, the map table, per-warp histograms, the
 // reduction scratch and the per-warp sample queues.  Map table and histograms
