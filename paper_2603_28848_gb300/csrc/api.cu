@@ -1294,9 +1294,17 @@ best_status best_autotune(best_ctx* ctx, const double* f_dev, double t, int32_t*
             break;
         }
         const bool prof = ctx->profiling;
-        int best_v = ctx->variant;
+        const int first = ctx->variant;
+        int best_v = first;
         double best_ms = 1e300;
         for (int v = 0; v < ctx->n_variants && s == BEST_OK; ++v) {
+            // a kernel that stands there twice (over its own and over the first variant's partition) is
+            // timed once, over the partition the context has where it runs already
+            bool again = false;
+            for (int u = 0; u < ctx->n_variants; ++u)
+                again = again || (u != v && ctx->variants[u].fn == ctx->variants[v].fn &&
+                                  (u == first || (v != first && ctx->variants[v].first_plan)));
+            if (again) continue;
             // restored first: the partition is built from the restored budgets
             if ((s = restore()) != BEST_OK) break;
             if ((s = set_variant(ctx, v)) != BEST_OK) break;
