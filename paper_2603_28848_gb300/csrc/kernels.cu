@@ -473,21 +473,24 @@ __device__ int64_t cta_exclusive_scan(int64_t v, int64_t* s, int64_t* total) {
 // neither many small hypercubes nor one that drew most of the items leaves the
 // CTA idle: below 32 items one thread (scope 1), below 1024 or J / 16 (J: the
 // task's items) one warp (scope 32, every lane with the same arguments), else
-// every thread of the CTA (scope blockDim, together).  The caller's index within the scope is threadIdx.x %
-// scope.  s, off, cnt: 256 entries of shared memory each.
+// every thread of the CTA (scope blockDim, together).  The caller's index within
+// the scope is threadIdx.x % scope.  The items named lie in [0, J) whatever m
+// holds (a loaded state's allocation is not checked): negative counts and what
+// goes past J are cut off.  s, off, cnt: 256 entries of shared memory each.
 template <typename F>
 __device__ void for_hypercubes(const int32_t* m, int H, int64_t J, int64_t* s, int64_t* off, int32_t* cnt, F&& f) {
     const int64_t large = max(int64_t(1024), J / 16);
     int64_t base = 0;
     for (int c0 = 0; c0 < H; c0 += blockDim.x) {
         const int h = c0 + static_cast<int>(threadIdx.x);
-        const int32_t v = h < H ? m[h] : 0;
+        const int32_t m_h = h < H ? max(m[h], 0) : 0;
         int64_t tot;
-        const int64_t ex = base + cta_exclusive_scan(v, s, &tot);
+        const int64_t ex = base + cta_exclusive_scan(m_h, s, &tot);
+        const int32_t v = static_cast<int32_t>(min(static_cast<int64_t>(m_h), max(int64_t(0), J - ex)));
         off[threadIdx.x] = ex;
         cnt[threadIdx.x] = v;
         __syncthreads();
-        if (v > 0 && v < 32) f(h, ex, v, 1);
+        if (h < H && v < 32) f(h, ex, v, 1);
         __syncwarp();
         const int nh = min(H - c0, static_cast<int>(blockDim.x));
         for (int k = threadIdx.x >> 5; k < nh; k += blockDim.x >> 5)
@@ -503,7 +506,7 @@ __device__ void strat_write_items(const int32_t* m, int H, int64_t J, uint32_t* 
                                   int32_t* cnt) {
     for_hypercubes(m, H, J, s, off, cnt, [&](int h, int64_t first, int32_t count, int scope) {
         for (int k = threadIdx.x % scope; k < count; k += scope)
-            if (first + k < J) item_h[first + k] = static_cast<uint32_t>(h);
+            item_h[first + k] = static_cast<uint32_t>(h);
     });
 }
 
