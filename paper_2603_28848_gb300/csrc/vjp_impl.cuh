@@ -606,49 +606,64 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
         };
         SegSetup<float, NLEG> s32;
         seg_setup32<NLEG>(P.tconst32[seg.task], &s32);
-        for (int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31); gb < g1; gb += blockDim.x) {
+        uint32_t uw[2 * SS::kUniforms];
+        int32_t gb = static_cast<int32_t>(seg.g0) + (tid & ~31);
+        int sgi = 0;
+        // the next sample of this lane's group (words in front), false past the end
+        auto next = [&]() {
             const int64_t grp = static_cast<int64_t>(gb) + lane;
-            uint32_t uw[2 * SS::kUniforms];
-            group_words64<D>(uw, static_cast<uint32_t>(grp), P.itn, ts.call, task, P.rk);
-#pragma unroll 1
-            for (int sgi = 0; sgi < G; ++sgi) {
-                const bool valid = grp < g1 && grp * G + sgi < N;
-                if (sgi > 0) {
+            if (G == 1 || sgi == 0) {
+                group_words64<D>(uw, static_cast<uint32_t>(grp), P.itn, ts.call, task, P.rk);
+            } else {
 #pragma unroll
-                    for (int k = 0; k < W; ++k) uw[k] = uw[(G > 1 ? W : 0) + k];
-                }
-                if (!V.screen) {
-                    sample(uw, 1, valid);
-                    continue;
-                }
-                float y[D], gauss;
-                uint32_t frac = 0;
+                for (int k = 0; k < W; ++k) uw[k] = uw[(G > 1 ? W : 0) + k];
+            }
+            const bool valid = grp < g1 && grp * G + sgi < N;
+            if (++sgi == G) {
+                sgi = 0;
+                gb += blockDim.x;
+            }
+            return valid;
+        };
+        if (!V.screen) {
+            while (gb < g1) {
+                const bool valid = next();
+                sample(uw, 1, valid);
+            }
+        } else {
+            // one copy of sample() for full and last queues, as in run_samples64
+            for (;;) {
+                const bool more = gb < g1;
+                if (more) {
+                    const bool valid = next();
+                    float y[D], gauss;
+                    uint32_t frac = 0;
 #pragma unroll
-                for (int d = 0; d < D; ++d) map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
-                log2_weight_bound<NLEG, false>(s32, P, y, 1.0f, &gauss);
-                const bool keep = valid && !(gauss < -1100.0f);
-                const uint32_t vote = __ballot_sync(0xffffffffu, keep);
-                if (keep) {
-                    const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
+                    for (int d = 0; d < D; ++d)
+                        map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
+                    log2_weight_bound<NLEG, false>(s32, P, y, 1.0f, &gauss);
+                    const bool keep = valid && !(gauss < -1100.0f);
+                    const uint32_t vote = __ballot_sync(0xffffffffu, keep);
+                    if (keep) {
+                        const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32
 #pragma unroll
-                    for (int k = 0; k < W; ++k) qw[k * kQueueSlots + slot] = uw[k];
-                }
-                qn += __popc(vote);
-                if (qn >= 32) {
-                    __syncwarp();
-                    sample(qw + lane, kQueueSlots, true);
-                    __syncwarp();
-                    if (lane < qn - 32) {
-#pragma unroll
-                        for (int k = 0; k < W; ++k) qw[k * kQueueSlots + lane] = qw[k * kQueueSlots + 32 + lane];
+                        for (int k = 0; k < W; ++k) qw[k * kQueueSlots + slot] = uw[k];
                     }
-                    __syncwarp();
-                    qn -= 32;
+                    qn += __popc(vote);
+                    if (qn < 32) continue;
                 }
+                __syncwarp();
+                if (lane < qn) sample(qw + lane, kQueueSlots, true);
+                if (!more) break;
+                __syncwarp();
+                if (lane < qn - 32) {
+#pragma unroll
+                    for (int k = 0; k < W; ++k) qw[k * kQueueSlots + lane] = qw[k * kQueueSlots + 32 + lane];
+                }
+                __syncwarp();
+                qn -= 32;
             }
         }
-        __syncwarp();
-        if (lane < qn) sample(qw + lane, kQueueSlots, true);
     }
 
     // ---- segment record: VJP [w, fobs, mobs, mc, tla, tlb, tha, thb, m_0 .. m_{NI-1}];
