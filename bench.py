@@ -371,7 +371,9 @@ def run_native(args, rank, world):
             "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the sample kernel "
                               "(profiles/eval_kernel_f32_c2_bose_2to2.md); the tables it reads do not "
                               "grow with the sample count",
-            "kernel": f"best::eval_kernel<float,{max(n_legs, 4)},{ctas_per_sm},_,{shape[1]},{shape[2]}> (persistent "
+            # (packed pairs of up to four legs are the instantiation with the products in the order of one sample, 3)
+            "kernel": f"best::eval_kernel<float,{max(n_legs, 4)},{ctas_per_sm},_,{shape[1]},"
+                      f"{3 if shape[2] == 2 and n_legs <= 4 else shape[2]}> (persistent "
                       "sample kernel)",
             "flops_per_sample": fps,
             "samples_per_launch": samples_per_launch, "launch_ms": per_launch_ms,

@@ -260,7 +260,9 @@ best_status best_evolve(best_ctx* ctx, int32_t method, int32_t n_steps, double* 
  * NULL) receives the chosen budget; best_launch_shape reports the rest.
  */
 /* The sample kernel's current launch shape: CTAs per SM of its register
- * budget, threads per CTA and samples per lane per step (any may be NULL). */
+ * budget, threads per CTA and samples per lane per step (any may be NULL); for
+ * FP64 the last is 2 where samples are screened in FP32 and 1 where every one
+ * is evaluated in FP64. */
 best_status best_launch_shape(const best_ctx* ctx, int32_t* ctas_per_sm, int32_t* threads,
                               int32_t* samples_per_lane);
 

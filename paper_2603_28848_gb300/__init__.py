@@ -369,7 +369,8 @@ class Collision:
         return mean, err
 
     def launch_shape(self):
-        """(CTAs per SM, threads per CTA, samples per lane per step) of the sample kernel."""
+        """(CTAs per SM, threads per CTA, samples per lane per step) of the sample kernel;
+        for FP64 the last is 2 for the loop with the FP32 screen and 1 for the plain one."""
         a, b, c = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
         check(self.lib.best_launch_shape(self.ctx, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)), self.ctx)
         return a.value, b.value, c.value
