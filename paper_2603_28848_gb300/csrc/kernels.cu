@@ -540,7 +540,8 @@ __global__ void strat_init_kernel(const TaskDesc* __restrict__ tasks, int32_t* s
 // underflow flag (S2 < S1^2 / n violated, i.e. FP32 squares underflowed, in
 // hypercubes holding more than 1e-6 of sum_h |S1_h| / n_h); then the
 // next allocation m_h = 1 + floor((J - H) d_h / sum d), d_h = (s_h^2)^(beta/2),
-// the remaining items one each to h = 0, 1, ... (uniform if every d_h = 0),
+// the remaining items one each to h = 0, 1, ... (uniform if every d_h = 0 or one
+// is infinite),
 // and the items rebuilt.  An underflowed iteration keeps its allocation.
 __global__ void __launch_bounds__(256, 4) strat_refine_kernel(const TaskDesc* __restrict__ tasks, const int32_t* __restrict__ active,
                                     const double* __restrict__ item_rec, int32_t* strat_m, double* strat_d,
@@ -671,7 +672,9 @@ __global__ void __launch_bounds__(256, 4) strat_refine_kernel(const TaskDesc* __
     }
     if (underflow) return;
     __syncthreads();
-    if (sum_d > 0.0) {
+    // (an infinite sum -- FP32 squares that overflowed -- has no shares: inf / inf would become the integer
+    // of a NaN, -2^31)
+    if (sum_d > 0.0 && isfinite(sum_d)) {
         int64_t cnt = 0;
         for (int h = threadIdx.x; h < H; h += blockDim.x) {
             const int32_t v = 1 + static_cast<int32_t>(floor(static_cast<double>(J - H) * S1h[h] / sum_d));

@@ -1,5 +1,6 @@
-"""A loaded state's allocation may not add up to the task's items: the sweep stays
-within them, as if the allocation ended where the items do."""
+"""Allocations at their limits.  A loaded state's may not add up to the task's
+items: the sweep stays within them, as if the allocation ended where the items
+do.  And FP32 squares that overflow leave no shares to allocate by."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,31 @@ def test_allocation_that_does_not_add_up(precision, h, add):
     col.close()
     C, err, C0, e0 = (x.cpu().numpy() for x in (C, err, C0, e0))
     assert np.all(np.isfinite(C)) and np.all(np.abs(C - C0) < 8 * np.hypot(err, e0) + 1e-300)
+
+
+def test_squares_beyond_fp32():
+    """First iterations scale the weights by 1 / f_obs (at most 2^100): where f_obs is
+    1e-36 and a wide Gaussian lets in samples with f of order one, w^2 is infinite
+    in FP32 and so is a hypercube's variance.  The allocation starts afresh and the
+    next iterations are ordinary ones (FP64 is the reference, 8 standard errors)."""
+    from dataclasses import replace
+    from paper_2603_28848_gb300 import Collision
+    prob, _ = W.c1_maxwell_2to2(n=8, neval=64 * 8 * 40, nitn=4)
+    prob = _strat(replace(prob, processes=tuple(replace(p, sigma_E=5.0) for p in prob.processes)))
+    q = W.grid_points(prob.grid)
+    f0 = np.exp(-np.sqrt(q * q + 1.0) / 0.25)[None, :]
+    assert 0 < f0.min() < 1e-34
+    f = _f(f0)
+    out = []
+    for precision in (W.PREC_FP32, W.PREC_FP64):
+        col = Collision(prob, precision)
+        col.eval(f, 0.0)
+        for t in range(col.n_tasks):
+            _, H, m = col.strata(t)
+            assert H == 64 and m.sum() == 64 * 40 and np.all(m >= 1)
+        col.eval(f, 0.0)
+        col.check()
+        out.append(col.task_results())
+        col.close()
+    (a, ea), (b, eb) = out
+    assert np.all(np.isfinite(a)) and np.all(np.abs(a - b) <= 8 * np.hypot(ea, eb) + 1e-5 * np.abs(b))
