@@ -44,16 +44,16 @@ def test_allocation_that_does_not_add_up(precision, h, add):
 
 def test_squares_beyond_fp32():
     """First iterations scale the weights by 1 / f_obs (at most 2^100): where f_obs is
-    1e-36 and a wide Gaussian lets in samples with f of order one, w^2 is infinite
-    in FP32 and so is a hypercube's variance.  The allocation starts afresh and the
+    1e-36 and a wide Gaussian lets in samples with f of order one, weights reach
+    1e22, w^2 is infinite in FP32 and so is a hypercube's variance.  The allocation starts afresh and the
     next iterations are ordinary ones (FP64 is the reference, 8 standard errors)."""
     from dataclasses import replace
     from paper_2603_28848_gb300 import Collision
     prob, _ = W.c1_maxwell_2to2(n=8, neval=64 * 8 * 40, nitn=4)
-    prob = _strat(replace(prob, processes=tuple(replace(p, sigma_E=5.0) for p in prob.processes)))
+    prob = replace(prob, grid=replace(prob.grid, log_spaced=False))
+    prob = _strat(replace(prob, processes=tuple(replace(p, sigma_E=20.0) for p in prob.processes)))
     q = W.grid_points(prob.grid)
-    f0 = np.exp(-np.sqrt(q * q + 1.0) / 0.25)[None, :]
-    assert 0 < f0.min() < 1e-34
+    f0 = 0.5 * np.exp(-82.0 * (q / 20.0) ** 2)[None, :]
     f = _f(f0)
     out = []
     for precision in (W.PREC_FP32, W.PREC_FP64):
