@@ -337,23 +337,23 @@ __device__ __noinline__ double plain_weight64(const uint32_t* q, int nb, const R
 
 // The same in FP32 from the uniform's first 32 bits.  The 20 bits left out, and
 // FP64's rounding, can take the point over an increment's edge: the mapped point
-// is continuous there, the increment's width is not.  frac becomes the largest
-// fraction seen, near_edge says whether any may have crossed (nb 2^-32 of the
-// samples per dimension).  Returns the increment's width.
+// is continuous there, the increment's width is not.  near_edge of the largest
+// fraction says whether any may have crossed (nb 2^-32 of the samples per
+// dimension).  Returns the increment's width.
 __device__ __forceinline__ float map_point32(uint32_t x0, uint32_t x1, int nb, const Real2<float>* table, float* y,
                                              uint32_t* frac) {
     const uint32_t x = (x0 & ~63u) | (x1 >> 26);
     const uint64_t m = static_cast<uint64_t>(x) * static_cast<uint32_t>(nb);
     const Real2<float> e = table[static_cast<uint32_t>(m >> 32)];
-    *frac = max(*frac, static_cast<uint32_t>(m));
+    *frac = static_cast<uint32_t>(m);
     *y = fmaf(e.dy, static_cast<float>(static_cast<uint32_t>(m)) * 2.3283064365386963e-10f, e.y0);
     return e.dy;
 }
 __device__ __forceinline__ bool near_edge(uint32_t frac, int nb) { return frac >= 0u - static_cast<uint32_t>(nb); }
 
 // log2 of an upper bound of |ca + cb f| at comoving q inside the grid: the FP32
-// spline value plus its rounding bound (2^-18 of its terms' magnitudes); +inf
-// where FP32 coefficients overflowed (their sum is then infinite or a NaN).
+// spline value plus its rounding bound (2^-18 of its terms' magnitudes); +inf or
+// a NaN, either of which keeps the sample, where FP32 coefficients overflowed.
 __device__ __forceinline__ float log2_factor_bound(const float* coef, const float* knots, float q, const Geometry& g,
                                                    float inv_step, float q0, float lq0_step, float ca) {
     int j = static_cast<int>(g.log_spaced ? fmaf(lg2_ftz(q), inv_step, -lq0_step) : (q - q0) * inv_step);
@@ -363,8 +363,8 @@ __device__ __forceinline__ float log2_factor_bound(const float* coef, const floa
     const float f = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);
     const float at = fabsf(t);
     const float size = fmaf(fmaf(fmaf(fabsf(c.w), at, fabsf(c.z)), at, fabsf(c.y)), at, fabsf(c.x));
-    if (!(size < 1e37f)) return __int_as_float(0x7f800000);                    // (f is a NaN only if size is not finite)
-    return lg2_ftz(fmaxf(ca + fmaxf(f, 0.0f) + 3.8e-6f * size, 1e-36f));       // (FP32 subnormals flush to 0)
+    // (at least 1e-36: FP32 subnormals flush to 0; the size, not f, carries what is not finite through)
+    return lg2_ftz(ca + fmaxf(f, 0.0f) + fmaf(3.8e-6f, size, 1e-36f));
 }
 
 // Upper bound of log2 |w_n| of a sample from FP32 arithmetic, y the mapped
@@ -411,9 +411,10 @@ __device__ __forceinline__ float log2_weight_bound(const SegSetup<float, NLEG>& 
     bal = fmaf(C.sgn_cons, Ec, bal);
     Esum += Ec;
     prod *= rEc;
-    const float err = fmaf(4e-5f, Esum, 1e-6f * S.qN * C.inv_a);
+    // (no bound from a Gaussian whose factor FP32 does not hold: infinite error)
+    const float err = fmaf(4e-5f, Esum, C.gauss_k > -1e37f ? 1e-6f * S.qN * C.inv_a : __int_as_float(0x7f800000));
     float d = fmaxf(fabsf(bal) - err, 0.0f);
-    if (!(Esum < 1e30f && C.gauss_k > -1e37f)) d = 0.0f; // (overflowed, or not a number: no bound)
+    if (!(Esum < 1e30f)) d = 0.0f;                       // (overflowed, or not a number)
     float extra = 0.0f;
     if (C.frac) {
         const float iS = __fdividef(1.0f, Esum);
@@ -552,12 +553,15 @@ __device__ __forceinline__ void run_samples64(const EvalParams& P, const Segment
             }
             const bool valid = grp < g1 && grp * G + sgi < N;
             float y[D], jac = 1.0f;
-            uint32_t frac = 0;
+            uint32_t frac[D], top_frac = 0;
 #pragma unroll
-            for (int d = 0; d < D; ++d) jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
+            for (int d = 0; d < D; ++d)
+                jac *= map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac[d]);
+#pragma unroll
+            for (int d = 0; d < D; d += 2) top_frac = __vimax3_u32(top_frac, frac[d], frac[d + 1 < D ? d + 1 : d]);
             float gauss;
             const float l = log2_weight_bound<NLEG, true>(s32, P, y, jac, &gauss);
-            const bool keep = valid && !(gauss < -1100.0f) && (near_edge(frac, nb) || !(l < cutoff));
+            const bool keep = valid && !(gauss < -1100.0f) && (near_edge(top_frac, nb) || !(l < cutoff));
             const uint32_t vote = __ballot_sync(0xffffffffu, keep);
             if (keep) {
                 const int slot = qn + __popc(vote & lanes_below);     // < 2 * 32

@@ -637,7 +637,7 @@ __device__ __forceinline__ void vjp_segment(const VjpParams& V, const Segment& s
                 if (more) {
                     const bool valid = next();
                     float y[D], gauss;
-                    uint32_t frac = 0;
+                    uint32_t frac;
 #pragma unroll
                     for (int d = 0; d < D; ++d)
                         map_point32(uw[2 * d], uw[2 * d + 1], nb, s_map32 + d * nb, &y[d], &frac);
