@@ -23,9 +23,9 @@
 // A sample whose FP32 quantities leave the normal range is kept.
 //
 // Measured per sweep on trained maps, plain loop -> this one: MB 2 -> 2, 32
-// points, 1e5 x 2 samples: 8.27 -> 0.80 ms; BE 2 -> 2, 2 species, 128 points,
-// 1e5 x 2: 55.2 -> 9.6 ms (with a fixed 2^-120, 10.0 ms: 40% of the samples are
-// evaluated, the FP64 pipe is 80% busy, about 120 operations per queued sample).
+// points, 1e5 x 2 samples: 8.28 -> 0.77 ms; BE 2 -> 2, 2 species, 128 points,
+// 1e5 x 2: 55.2 -> 9.5 ms (up to 40% of the samples are evaluated, the FP64 pipe
+// is 79% busy, about 120 operations per queued sample).
 #pragma once
 
 #include "math_table.cuh"
